@@ -179,20 +179,20 @@ __global__ void __launch_bounds__(STAGED_THREADS, 5) k_force_staged(Links<float,
     }
 }
 
-// U <- exp(s B) U on every link; the FP32 formats are reunitarised.
+// U <- exp(s B) U on every link; the FP32 formats are reunitarised.  One thread
+// per link, block row y of the grid holding the links of one (mu, parity).
 template <class T, int NP>
 __global__ void __launch_bounds__(128) k_exp_update(Links<T, NP> U, Geom g, Alg<T> B, T s) {
     pdl_launch_dependents();
+    const int mu = blockIdx.y >> 1, par = blockIdx.y & 1, h = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 8 * g.Vh) return;
-    const int mp = idx / g.Vh, h = idx - mp * g.Vh, mu = mp >> 1, par = mp & 1;
+    if (h >= g.Vh) return;
     T c[8];
     B.load(mu, par, h, c);
+    const M3<T> u0 = U.load(mu, par, h);
 #pragma unroll
     for (int a = 0; a < 8; a++) c[a] *= s;
-    const M3<T> E = exp_alg(c);
-    M3<T> u = mul_nn(E, U.load(mu, par, h));
+    M3<T> u = mul_nn(exp_alg(c), u0);
     if (sizeof(T) == 4) reunitarize(u);
     U.store(mu, par, h, u);
 }
@@ -288,7 +288,7 @@ mgq_status force_accumulate(const mgq_lattice* lat, void* B, double coef, double
 mgq_status exp_update(const mgq_lattice* lat, void* B, double s, cudaStream_t st) {
     const Geom g = make_geom(lat->dims);
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
-        launch_pdl(k_exp_update<T, NP>, nblk(8L * g.Vh, 128), 128, st, links_of<T, NP>(lat), g,
+        launch_pdl(k_exp_update<T, NP>, dim3(nblk(g.Vh, 128), 8), 128, st, links_of<T, NP>(lat), g,
                    alg_at<T>(B, lat->dims), (T)s);
     });
     return cuda_check("exp_update");
