@@ -111,7 +111,9 @@ uint64_t mgq_workspace_bytes(const mgq_lattice* lat);
  * depend on it (one thread per link or per active bond).  FP32 12-real
  * sub-sweeps of the batched driver, and of single lattices with V/2 >= 49152,
  * stage their staple links through shared memory and always run 128 threads
- * per block; the setting applies to the other launches.  The force kernel's shape is structural (eight warps cover the
+ * per block; the setting applies to the other launches, except single-lattice
+ * FP64 sub-sweeps of too few links to fill the chip with one thread each, which
+ * run several lanes per link in blocks of 128.  The force kernel's shape is structural (eight warps cover the
  * eight (mu, parity) planes of a 32-site band) and not tuned.  Process-wide setting; change it only while no
  * call is being issued.  Set by the autotuner (paper_1510_04675_gb300/tune.py). */
 typedef enum {

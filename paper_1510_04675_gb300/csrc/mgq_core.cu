@@ -7,6 +7,7 @@
 
 #include "mgq_internal.h"
 #include "mgq_stencil.cuh"
+#include "mgq_columns.cuh"
 
 namespace mgq {
 
@@ -421,12 +422,27 @@ static int g_block[MGQ_NKERNELS][3] = {{128, 128, 128}, {128, 128, 128}, {128, 1
 
 int block_size(int kernel, int prec) { return g_block[kernel][prec]; }
 
+// FP64 sub-sweeps of too few links for one thread each (lanes_per_link), with
+// `lanes` lanes per link; returns the number of blocks
+template <bool HB>
+static int launch_columns(int lanes, mgq_lattice* lat, const Geom& g, int mu, int par, double beta, const RngKey& rk,
+                          int n_hb, uint8_t* dec, double* partials, cudaStream_t st) {
+    const int nb = nblk(g.Vh, lanes == 3 ? ColumnLane<3>::kPerBlock : ColumnLane<6>::kPerBlock);
+    launch_pdl(lanes == 3 ? k_update_columns<HB, 3> : k_update_columns<HB, 6>, nb, COL_THREADS, st, links_of<double, 9>(lat),
+               g, mu, par, beta, rk, n_hb, dec, partials);
+    return nb;
+}
+
 mgq_status heatbath_subsweep(mgq_lattice* lat, double beta, uint64_t sweep, int n_hb, int mu, int par,
                              uint8_t* dec, cudaStream_t st) {
     Trace trace("heatbath_subsweep");
     const Geom g = make_geom(lat->dims);
     const int bs = g_block[MGQ_KERNEL_HEATBATH][lat->prec];
     const RngKey rk = make_rng(lat->seed, lat->lattice_id, sweep);
+    if (const int lanes = lat->prec == MGQ_F64 ? lanes_per_link(g.Vh) : 1; lanes > 1) {
+        launch_columns<true>(lanes, lat, g, mu, par, beta, rk, n_hb, dec, nullptr, st);
+        return cuda_check("mgq_heatbath");
+    }
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
         dispatch_mu(mu, [&]<int MU>() {
             if constexpr (sizeof(T) == 4 && NP == 6) {
@@ -451,6 +467,10 @@ mgq_status overrelax_subsweep(mgq_lattice* lat, int mu, int par, cudaStream_t st
     Trace trace("overrelax_subsweep");
     const Geom g = make_geom(lat->dims);
     const int bs = g_block[MGQ_KERNEL_OVERRELAX][lat->prec];
+    if (const int lanes = lat->prec == MGQ_F64 ? lanes_per_link(g.Vh) : 1; lanes > 1) {
+        launch_columns<false>(lanes, lat, g, mu, par, 0.0, RngKey{}, 0, nullptr, nullptr, st);
+        return cuda_check("mgq_overrelax");
+    }
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
         dispatch_mu(mu, [&]<int MU>() {
             if (sizeof(T) == 4 && NP == 6 && g.Vh >= STAGED_MIN_VH)
@@ -474,8 +494,15 @@ mgq_status overrelax_sweep_plaquette(mgq_lattice* lat, double* dev_out, cudaStre
     const Geom g = make_geom(lat->dims);
     const bool staged = lat->prec == MGQ_F32_C12 && g.Vh >= STAGED_MIN_VH;
     const int bs = staged ? STAGED_THREADS : g_block[MGQ_KERNEL_OVERRELAX][lat->prec];
-    const int nb = nblk(g.Vh, bs);
     double* partials = reinterpret_cast<double*>(ws_alg(lat));  // free during sweeps; >= 2 nb doubles
+    if (const int lanes = lat->prec == MGQ_F64 ? lanes_per_link(g.Vh) : 1; lanes > 1) {
+        int n = 0;
+        for (int par = 0; par < 2; par++)
+            n += launch_columns<false>(lanes, lat, g, 3, par, 0.0, RngKey{}, 0, nullptr, partials + n, st);
+        launch_final_sum(partials, n, 1.0 / (18.0 * (double)g.V), dev_out, st);
+        return cuda_check("overrelax_sweep_plaquette");
+    }
+    const int nb = nblk(g.Vh, bs);
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
         for (int par = 0; par < 2; par++) {
             if (staged)

@@ -114,6 +114,64 @@ template <class T> __device__ __forceinline__ M3<T> mul_dd(const M3<T>& a, const
             r.e[i][j] = conjg(b.e[j][0] * a.e[0][i] + b.e[j][1] * a.e[1][i] + b.e[j][2] * a.e[2][i]);
     return r;
 }
+// FP64 products as chains of fused multiply-adds, four per complex term: 108
+// operations for a 3x3 product where separately added complex products take 144
+// (an FP64 warp instruction occupies its sub-partition for 64 cycles here, so the
+// operation count is the time).
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+// a b, and acc + a b
+__device__ __forceinline__ Cx<double> cmul0(Cx<double> a, Cx<double> b) {
+    return mk(fma_rn(-a.im, b.im, __dmul_rn(a.re, b.re)), fma_rn(a.im, b.re, __dmul_rn(a.re, b.im)));
+}
+__device__ __forceinline__ void cmac(Cx<double>& acc, Cx<double> a, Cx<double> b) {
+    acc.re = fma_rn(-a.im, b.im, fma_rn(a.re, b.re, acc.re));
+    acc.im = fma_rn(a.im, b.re, fma_rn(a.re, b.im, acc.im));
+}
+// a0 b0 + a1 b1 + a2 b2
+__device__ __forceinline__ Cx<double> dot3(Cx<double> a0, Cx<double> b0, Cx<double> a1, Cx<double> b1, Cx<double> a2,
+                                           Cx<double> b2) {
+    Cx<double> r = cmul0(a0, b0);
+    cmac(r, a1, b1);
+    cmac(r, a2, b2);
+    return r;
+}
+// element (i, k) of op(m), the conjugate transpose for D
+template <bool D> __device__ __forceinline__ Cx<double> op_at(const M3<double>& m, int i, int k) {
+    return D ? conjg(m.e[k][i]) : m.e[i][k];
+}
+template <bool DA, bool DB> __device__ __forceinline__ M3<double> chain_product(const M3<double>& a, const M3<double>& b) {
+    M3<double> r;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++)
+            r.e[i][j] = dot3(op_at<DA>(a, i, 0), op_at<DB>(b, 0, j), op_at<DA>(a, i, 1), op_at<DB>(b, 1, j),
+                             op_at<DA>(a, i, 2), op_at<DB>(b, 2, j));
+    return r;
+}
+// r += op(a) op(b)
+template <bool DA, bool DB>
+__device__ __forceinline__ void chain_product_add(M3<double>& r, const M3<double>& a, const M3<double>& b) {
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++)
+#pragma unroll
+            for (int k = 0; k < 3; k++) cmac(r.e[i][j], op_at<DA>(a, i, k), op_at<DB>(b, k, j));
+}
+template <> __device__ __forceinline__ M3<double> mul_nn<double>(const M3<double>& a, const M3<double>& b) {
+    return chain_product<false, false>(a, b);
+}
+template <> __device__ __forceinline__ M3<double> mul_nd<double>(const M3<double>& a, const M3<double>& b) {
+    return chain_product<false, true>(a, b);
+}
+template <> __device__ __forceinline__ M3<double> mul_dn<double>(const M3<double>& a, const M3<double>& b) {
+    return chain_product<true, false>(a, b);
+}
+template <> __device__ __forceinline__ M3<double> mul_dd<double>(const M3<double>& a, const M3<double>& b) {
+    return chain_product<true, true>(a, b);
+}
+
 // FP32 products on the packed f32x2 FMA of sm_100+: a complex product is
 // a.re * (b.re, b.im) + a.im * (-b.im, b.re), two paired FMAs instead of four.
 // ROWS = 2 computes rows 0 and 1 of the result only; DA / DB take the
@@ -211,6 +269,21 @@ template <class T> __device__ __forceinline__ void rebuild_row2(M3<T>& u) {
     u.e[2][2] = conjg(u.e[0][0] * u.e[1][1] - u.e[0][1] * u.e[1][0]);
 }
 
+// FP64: the same entries as chains (one definition for the kernels that hold a
+// link in one thread and those that hold a column of it per lane).
+__device__ __forceinline__ Cx<double> cross_conj(Cx<double> r0p, Cx<double> r0q, Cx<double> r1p, Cx<double> r1q) {
+    Cx<double> v = cmul0(r0p, r1q);
+    cmac(v, mk(-r0q.re, -r0q.im), r1p);
+    return conjg(v);
+}
+template <> __device__ __forceinline__ void rebuild_row2<double>(M3<double>& u) {
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const int p = (k + 1) % 3, q = (k + 2) % 3;
+        u.e[2][k] = cross_conj(u.e[0][p], u.e[0][q], u.e[1][p], u.e[1][q]);
+    }
+}
+
 // FP32: conj(a b - c d) per entry on the packed FMA, row 1 entries paired.
 template <> __device__ __forceinline__ void rebuild_row2<float>(M3<float>& u) {
     float2 B[3], iB[3];
@@ -249,6 +322,26 @@ template <class T> __device__ __forceinline__ void reunitarize(M3<T>& u) {
     for (int k = 0; k < 3; k++) u.e[1][k] = u.e[1][k] - ip * u.e[0][k];
     T n1 = norm2(u.e[1][0]) + norm2(u.e[1][1]) + norm2(u.e[1][2]);
     T inv1 = inv_norm(n1);
+#pragma unroll
+    for (int k = 0; k < 3; k++) u.e[1][k] = scale(u.e[1][k], inv1);
+    rebuild_row2(u);
+}
+
+// FP64, with the order of every operation fixed (see cross_conj).
+__device__ __forceinline__ double sum3(double a, double b, double c) { return __dadd_rn(__dadd_rn(a, b), c); }
+__device__ __forceinline__ double norm2_rn(Cx<double> a) { return fma_rn(a.im, a.im, __dmul_rn(a.re, a.re)); }
+template <> __device__ __forceinline__ void reunitarize<double>(M3<double>& u) {
+    const double inv0 = inv_norm(sum3(norm2_rn(u.e[0][0]), norm2_rn(u.e[0][1]), norm2_rn(u.e[0][2])));
+    Cx<double> q[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        u.e[0][k] = scale(u.e[0][k], inv0);
+        q[k] = cmul0(u.e[1][k], conjg(u.e[0][k]));
+    }
+    const Cx<double> mip = mk(-sum3(q[0].re, q[1].re, q[2].re), -sum3(q[0].im, q[1].im, q[2].im));
+#pragma unroll
+    for (int k = 0; k < 3; k++) cmac(u.e[1][k], mip, u.e[0][k]);
+    const double inv1 = inv_norm(sum3(norm2_rn(u.e[1][0]), norm2_rn(u.e[1][1]), norm2_rn(u.e[1][2])));
 #pragma unroll
     for (int k = 0; k < 3; k++) u.e[1][k] = scale(u.e[1][k], inv1);
     rebuild_row2(u);

@@ -238,15 +238,18 @@ __device__ __forceinline__ M3<float> staple_staged(const Links<float, 6>& U, con
     return A;
 }
 
-// Full products in the oracle's order (the FP64 parity path).
-template <class T, int NP>
-__device__ __forceinline__ M3<T> staple_full(const Links<T, NP>& U, const Geom& g, const int x[4], int h, int mu,
-                                             int par) {
-    M3<T> A;
+// Full products, no use of unitarity (the FP64 parity path): the upper terms
+// a (b^+ c^+) summed over nu, the lower terms d^+ (e^+ f) summed over nu, then
+// added; the second product of each term accumulates onto the sum directly.
+// Column k of every term needs column k of c^+ or f alone, which the kernels with
+// one column per lane use (mgq_columns.cuh; same operations, same bits).
+__device__ __forceinline__ M3<double> staple_full(const Links<double, 9>& U, const Geom& g, const int x[4], int h, int mu,
+                                                  int par) {
+    M3<double> A, D;
 #pragma unroll
     for (int i = 0; i < 3; i++)
 #pragma unroll
-        for (int j = 0; j < 3; j++) A.e[i][j] = mk(T(0), T(0));
+        for (int j = 0; j < 3; j++) A.e[i][j] = D.e[i][j] = mk(0.0, 0.0);
     const int op = par ^ 1;
     const Hops H = make_hops(g, x);
     const int fmu = pick(H.fwd, mu);
@@ -255,29 +258,23 @@ __device__ __forceinline__ M3<T> staple_full(const Links<T, NP>& U, const Geom& 
     for (int nu = 0; nu < 4; nu++) {
         if (nu == mu) continue;
         const int hpn = (H.lex + H.fwd[nu]) >> 1;
+        const M3<double> v = mul_dd(U.load(mu, op, hpn), U.load(nu, par, h));  // U_mu(x+nu)^+ U_nu(x)^+
+        chain_product_add<false, false>(A, U.load(nu, op, hpm), v);            // U_nu(x+mu)
+    }
+#pragma unroll
+    for (int nu = 0; nu < 4; nu++) {
+        if (nu == mu) continue;
         const int hmn = (H.lex + H.bwd[nu]) >> 1;
         const int hpm_mn = (H.lex + fmu + H.bwd[nu]) >> 1;
-        M3<T> up, dn;
-        {
-            const M3<T> a = U.load(nu, op, hpm);   // U_nu(x+mu)
-            const M3<T> b = U.load(mu, op, hpn);   // U_mu(x+nu)
-            const M3<T> c = U.load(nu, par, h);    // U_nu(x)
-            up = mul_nd(mul_nd(a, b), c);
-        }
-        {
-            const M3<T> d = U.load(nu, par, hpm_mn);  // U_nu(x+mu-nu)
-            const M3<T> e = U.load(mu, op, hmn);      // U_mu(x-nu)
-            const M3<T> f = U.load(nu, op, hmn);      // U_nu(x-nu)
-            dn = mul_nn(mul_dd(d, e), f);
-        }
-        acc_add(up, dn);
-        acc_add(A, up);
+        const M3<double> w = mul_dn(U.load(mu, op, hmn), U.load(nu, op, hmn));  // U_mu(x-nu)^+ U_nu(x-nu)
+        chain_product_add<true, false>(D, U.load(nu, par, hpm_mn), w);          // U_nu(x+mu-nu)^+
     }
+    acc_add(A, D);
     return A;
 }
 
 // FP32 (both formats): products of SU(3) factors in two-row form; FP64: full
-// products in the oracle's order.
+// products.
 template <class T, int NP>
 __device__ __forceinline__ M3<T> staple(const Links<T, NP>& U, const Geom& g, const int x[4], int h, int mu, int par) {
     if constexpr (sizeof(T) == 4) return staple_two_row<T>(U, g, x, h, mu, par);
@@ -383,6 +380,26 @@ __device__ __forceinline__ void su2_rows(M3<T>& m, int i, int j, const T r[4], b
     }
 }
 
+// FP64: one column of the two rows as chains.
+__device__ __forceinline__ void su2_pair(Cx<double>& mi, Cx<double>& mj, const double r[4]) {
+    Cx<double> ni = cmul0(mk(r[0], r[3]), mi), nj = cmul0(mk(-r[2], r[1]), mi);
+    cmac(ni, mk(r[2], r[1]), mj);
+    cmac(nj, mk(r[0], -r[3]), mj);
+    mi = ni;
+    mj = nj;
+}
+template <>
+__device__ __forceinline__ void su2_rows<double>(M3<double>& m, int i, int j, const double r[4], bool do_i, bool do_j,
+                                                 int ci, int cj) {
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        Cx<double> mi = m.e[i][k], mj = m.e[j][k];
+        su2_pair(mi, mj, r);
+        if (do_i && ((ci >> k) & 1)) m.e[i][k] = mi;
+        if (do_j && ((cj >> k) & 1)) m.e[j][k] = mj;
+    }
+}
+
 // FP32: a m_i + b m_j with a = r0 + i r3, b = r2 + i r1 (and c = -r2 + i r1,
 // d = r0 - i r3 for row j) as packed FMAs on (re, im) pairs.
 template <>
@@ -461,10 +478,17 @@ __device__ __forceinline__ void creutz_phi(float u3, float* s, float* c) {
 // direction cos(theta) = 2 u2 - 1, phi = 2 pi u3; R = X (w/|w|), U <- R U,
 // V <- R V; reunitarise at the end.  dec[s] = accepted attempt or 255.
 
-// One Creutz attempt on subgroup s with the four words r; on acceptance
-// applies R = X (w/|w|) to u and v and returns true.
+// |w|^2 of a subgroup's quaternion (FP64: a fixed chain)
+template <class T> __device__ __forceinline__ T quat_norm2(const T w[4]) {
+    return w[0] * w[0] + w[1] * w[1] + w[2] * w[2] + w[3] * w[3];
+}
+template <> __device__ __forceinline__ double quat_norm2<double>(const double w[4]) {
+    return fma_rn(w[3], w[3], fma_rn(w[2], w[2], fma_rn(w[1], w[1], __dmul_rn(w[0], w[0]))));
+}
+
+// One Creutz attempt with the four words r: R = X (w/|w|) and true on acceptance.
 template <class T>
-__device__ __forceinline__ bool creutz_attempt(M3<T>& u, M3<T>& v, int s, const T w[4], T xi, T k, T em, uint4 r) {
+__device__ __forceinline__ bool creutz_draw(const T w[4], T xi, T k, T em, uint4 r, T R[4]) {
     const T u0 = u01<T>(r.x), u1 = u01<T>(r.y), u2 = u01<T>(r.z), u3 = u01<T>(r.w);
     const T a0 = creutz_a0(k, em, u0);
     const T rest = sub_rn(T(1), mul_rn(a0, a0));
@@ -477,8 +501,15 @@ __device__ __forceinline__ bool creutz_attempt(M3<T>& u, M3<T>& v, int s, const 
     const T X[4] = {a0, rad * st * cp, rad * st * sp, rad * ct};
     const T inv = recip(xi);
     const T wh[4] = {w[0] * inv, w[1] * inv, w[2] * inv, w[3] * inv};
-    T R[4];
     qmul(X, wh, R);
+    return true;
+}
+
+// the attempt on subgroup s, applied to u and v when accepted
+template <class T>
+__device__ __forceinline__ bool creutz_attempt(M3<T>& u, M3<T>& v, int s, const T w[4], T xi, T k, T em, uint4 r) {
+    T R[4];
+    if (!creutz_draw(w, xi, k, em, r, R)) return false;
     apply_subgroup(u, v, s, R);
     return true;
 }
@@ -492,7 +523,7 @@ __device__ __forceinline__ void hb_link(M3<T>& u, const M3<T>& A, T beta, int n_
         const int i = (s == 2) ? 1 : 0, j = (s == 0) ? 1 : 2;
         T w[4];
         block_w(v, i, j, w);
-        const T xi = m_sqrt(w[0] * w[0] + w[1] * w[1] + w[2] * w[2] + w[3] * w[3]);
+        const T xi = m_sqrt(quat_norm2(w));
         uint8_t d = 255;
         if (xi >= tiny_norm<T>()) {
             const T k = creutz_k(beta, xi);
@@ -519,13 +550,38 @@ __device__ __forceinline__ void hb_link_drawn(M3<T>& u, const M3<T>& A, T beta, 
         const int i = (s == 2) ? 1 : 0, j = (s == 0) ? 1 : 2;
         T w[4];
         block_w(v, i, j, w);
-        const T xi = m_sqrt(w[0] * w[0] + w[1] * w[1] + w[2] * w[2] + w[3] * w[3]);
+        const T xi = m_sqrt(quat_norm2(w));
         if (xi >= tiny_norm<T>()) {
             const T k = creutz_k(beta, xi);
             creutz_attempt(u, v, s, w, xi, k, creutz_em(k), r[s]);
         }
     }
     reunitarize(u);
+}
+
+// Overrelaxation's rotation (w/|w|)^2 = (w0^2 - |w_vec|^2, 2 w0 w_vec) / |w|^2;
+// false when |w| is too small to divide by
+template <class T> __device__ __forceinline__ bool or_rotation(const T w[4], T R[4]) {
+    const T n2 = quat_norm2(w);
+    if (!(m_sqrt(n2) >= tiny_norm<T>())) return false;
+    const T inv2 = recip(n2);
+    R[0] = (w[0] * w[0] - w[1] * w[1] - w[2] * w[2] - w[3] * w[3]) * inv2;
+    R[1] = T(2) * w[0] * w[1] * inv2;
+    R[2] = T(2) * w[0] * w[2] * inv2;
+    R[3] = T(2) * w[0] * w[3] * inv2;
+    return true;
+}
+// FP64, in fixed operations; |w| >= 1e-300 holds for every |w|^2 > 0
+template <> __device__ __forceinline__ bool or_rotation<double>(const double w[4], double R[4]) {
+    const double n2 = quat_norm2(w);
+    if (!(n2 > 0.0)) return false;
+    const double inv2 = 1.0 / n2, t = __dmul_rn(__dadd_rn(w[0], w[0]), inv2);
+    const double v2 = fma_rn(w[3], w[3], fma_rn(w[2], w[2], __dmul_rn(w[1], w[1])));
+    R[0] = __dmul_rn(fma_rn(w[0], w[0], -v2), inv2);
+    R[1] = __dmul_rn(t, w[1]);
+    R[2] = __dmul_rn(t, w[2]);
+    R[3] = __dmul_rn(t, w[3]);
+    return true;
 }
 
 // Overrelaxation of one link: per subgroup R = (w/|w|)^2; reunitarise.
@@ -535,15 +591,9 @@ __device__ __forceinline__ void or_link(M3<T>& u, const M3<T>& A) {
 #pragma unroll
     for (int s = 0; s < 3; s++) {
         const int i = (s == 2) ? 1 : 0, j = (s == 0) ? 1 : 2;
-        T w[4];
+        T w[4], R[4];
         block_w(v, i, j, w);
-        const T n2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2] + w[3] * w[3];
-        if (!(m_sqrt(n2) >= tiny_norm<T>())) continue;
-        const T inv2 = recip(n2);
-        // (w/|w|)^2 = (w0^2 - |w_vec|^2, 2 w0 w_vec) / |w|^2
-        const T R[4] = {(w[0] * w[0] - w[1] * w[1] - w[2] * w[2] - w[3] * w[3]) * inv2, T(2) * w[0] * w[1] * inv2,
-                        T(2) * w[0] * w[2] * inv2, T(2) * w[0] * w[3] * inv2};
-        apply_subgroup(u, v, s, R);
+        if (or_rotation(w, R)) apply_subgroup(u, v, s, R);
     }
     reunitarize(u);
 }
