@@ -8,10 +8,13 @@
 //   E = (1/V) sum_x 1/2 sum_p |g_p|^2           -> c_p = g_p / V
 //   Q = 1/(8 pi^2) sum_x (g01.g23 - g02.g13 + g03.g12) -> c01 = g23/(8 pi^2), ...
 // and dg = t(TA(dQ))/4, c . t(TA(N)) = -2 Re Tr(C N) (C = sum c_a X_a), so
-// dO = -1/2 sum Re Tr(C_p(x) dQ_p(x)).  A leaf F1 F2 F3 F4 varied in factor k
-// (F_k = U_m or U_m^+, variation U_m -> exp(e) U_m) contributes to the link's
-// cotangent +1/4 TA(F_k R_k) for an undaggered and -1/4 TA(R_k F_k) for a
-// daggered factor, R_k = F_{k+1} .. F_4 C F_1 .. F_{k-1}.
+// dO = -1/2 sum Re Tr(C_p(x) dQ_p(x)).  Each plaquette is a leaf of the clovers at
+// its four corners, so it carries the four C of its corners, each inserted once.
+// For a link m = U_rho(y) of it, traced from m as m X1 X2 X3 past the corners
+// y, y1, y2, y3, the link's cotangent gets (variation U_m -> exp(e) U_m)
+//   s/4 TA(m R),  R = C(y1) X1 X2 X3 + X1 C(y2) X2 X3 + X1 X2 C(y3) X3 + X1 X2 X3 C(y),
+// s = +1 when that is the leaf's sense (a then b for plane a < b), -1 when it is
+// the reverse, as C^+ = -C and TA(M^+) = -TA(M).
 #include "mgq_internal.h"
 #include "mgq_stencil.cuh"
 
@@ -20,18 +23,6 @@ namespace mgq {
 // plane index of (a, b), a < b: 01 02 03 12 13 23
 __host__ __device__ constexpr int plane_of(int a, int b) { return a == 0 ? b - 1 : (a == 1 ? b + 1 : 5); }
 
-// clover leaves of plane (a, b) at x: factor j of leaf l is the link in
-// direction (kDir ? b : a) at x + oa e_a + ob e_b, daggered if kDag
-struct LeafFactor {
-    int8_t dir_b, oa, ob, dag;
-};
-__constant__ LeafFactor c_leaves[4][4] = {
-    {{0, 0, 0, 0}, {1, 1, 0, 0}, {0, 0, 1, 1}, {1, 0, 0, 1}},        // l1 = U_a(x) U_b(x+a) U_a(x+b)^+ U_b(x)^+
-    {{1, 0, 0, 0}, {0, -1, 1, 1}, {1, -1, 0, 1}, {0, -1, 0, 0}},     // l2 = U_b(x) U_a(x-a+b)^+ U_b(x-a)^+ U_a(x-a)
-    {{0, -1, 0, 1}, {1, -1, -1, 1}, {0, -1, -1, 0}, {1, 0, -1, 0}},  // l3 = U_a(x-a)^+ U_b(x-a-b)^+ U_a(x-a-b) U_b(x-b)
-    {{1, 0, -1, 1}, {0, 0, -1, 0}, {1, 1, -1, 0}, {0, 0, 0, 1}},     // l4 = U_b(x-b)^+ U_a(x-b) U_b(x+a-b) U_a(x)^+
-};
-
 template <class T>
 struct Planes6 {  // c_p(x): [p][parity][a][h] (scratch of this file only)
     T* p;
@@ -39,106 +30,97 @@ struct Planes6 {  // c_p(x): [p][parity][a][h] (scratch of this file only)
     __device__ __forceinline__ T* at(int pl, int par, int h) const { return p + (size_t)(pl * 2 + par) * 8 * S + h; }
 };
 
-// Pass 1: c_p(x) for every site and plane.
+// Pass 1: c_p(x) for every site and plane, one thread per site and dual pair of
+// planes (block row y).
 template <class T, int NP>
-__global__ void __launch_bounds__(128) k_clover_cotangent(Links<T, NP> U, Geom g, int obs, Planes6<T> C) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 1 : 4) k_clover_cotangent(Links<T, NP> U, Geom g, int obs, Planes6<T> C) {
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x, p = blockIdx.y;
     if (idx >= g.V) return;
     const int par = idx >= g.Vh, h = idx - par * g.Vh;
     int x[4];
     cb_coords(g, par, h, x);
-    T G[6][8];
-    const int pl[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
-#pragma unroll 1
-    for (int p = 0; p < 6; p++) clover_coeffs(U, g, x, par, h, pl[p][0], pl[p][1], G[p]);
-    const T invV = T(1) / (T)g.V, q = T(1.0 / (8.0 * 9.869604401089358));
+    const Hops H = make_hops(g, x);
+    T Ga[8], Gb[8];
+    clover_coeffs(U, H, par, par ^ 1, 0, p + 1, Ga);
+    clover_coeffs(U, H, par, par ^ 1, dual_mu(p), dual_nu(p), Gb);
+    // E: c = g / V; Q: c of a plane is +- g of its dual plane / (8 pi^2): 01<->23 (+), 02<->13 (-), 03<->12 (+)
+    const T f = obs == 0 ? T(1) / (T)g.V : (p == 1 ? T(-1.0 / (8.0 * 9.869604401089358)) : T(1.0 / (8.0 * 9.869604401089358)));
+    T* oa = C.at(p, par, h);
+    T* ob = C.at(5 - p, par, h);
 #pragma unroll
-    for (int p = 0; p < 6; p++) {
-        T* out = C.at(p, par, h);
-#pragma unroll
-        for (int a = 0; a < 8; a++) {
-            T v;
-            if (obs == 0) v = G[p][a] * invV;
-            else {
-                // partner planes: 01<->23 (+), 02<->13 (-), 03<->12 (+)
-                const int partner = 5 - p;
-                const T sgn = (p == 1 || p == 4) ? T(-1) : T(1);
-                v = sgn * q * G[partner][a];
-            }
-            out[(size_t)a * C.S] = v;
-        }
+    for (int a = 0; a < 8; a++) {
+        oa[(size_t)a * C.S] = f * (obs == 0 ? Ga[a] : Gb[a]);
+        ob[(size_t)a * C.S] = f * (obs == 0 ? Gb[a] : Ga[a]);
     }
 }
 
-template <class T, int NP>
-__device__ __forceinline__ M3<T> factor(const Links<T, NP>& U, const Geom& g, const int x[4], int a, int b,
-                                        const LeafFactor& f) {
-    int y[4];
+// the antihermitian C of plane pl at site (par, h)
+template <class T> __device__ __forceinline__ M3<T> corner(const Planes6<T>& C, int pl, int par, int h) {
+    T c[8];
+    const T* p = C.at(pl, par, h);
 #pragma unroll
-    for (int d = 0; d < 4; d++) y[d] = wrap(x[d] + (d == a ? f.oa : 0) + (d == b ? f.ob : 0), g.L[d]);
-    const int lex = lex_of(g, y);
-    const M3<T> u = U.load(f.dir_b ? b : a, (y[0] + y[1] + y[2] + y[3]) & 1, lex >> 1);
-    return f.dag ? dagger(u) : u;
+    for (int q = 0; q < 8; q++) c[q] = p[(size_t)q * C.S];
+    return alg_matrix(c);
 }
 
-// Pass 2: lam_m += scale * dO/de_m for every link m = U_rho(y).
+// Pass 2: lam_m += scale * dO/de_m for every link m = U_rho(y): two plaquettes in each
+// of three planes.  The product rule runs along the loop: with P = X1 X2 and
+// S = P X3, R = C(y1) S + (X1 C(y2) X2 + P C(y3)) X3 + S C(y), and since every
+// plaquette of a plane has the same C(y), the sum of s S takes it once per plane:
+// 15 products a plane, where a gather over the 8 leaves of a plane that hold the
+// link, each multiplied out on its own, took about 44 and as many link loads.  A
+// plane's two sides run one after the other and the planes in a rolled loop, which
+// keeps the live matrices in registers (16^4, FP32 12-real: 296 -> 70 us).
 template <class T, int NP>
-__global__ void __launch_bounds__(128) k_clover_vjp(Links<T, NP> U, Geom g, Planes6<T> C, T scl, Alg<T> Lam) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 8 * g.Vh) return;
-    const int mp = idx / g.Vh, h = idx - mp * g.Vh, rho = mp >> 1, par = mp & 1;
+__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 1 : 3) k_clover_vjp(Links<T, NP> U, Geom g, Planes6<T> C, T scl, Alg<T> Lam) {
+    const int rho = blockIdx.y >> 1, par = blockIdx.y & 1, op = par ^ 1, h = blockIdx.x * blockDim.x + threadIdx.x;
+    if (h >= g.Vh) return;
     int y[4];
     cb_coords(g, par, h, y);
-    T acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    const Hops H = make_hops(g, y);
+    const int frho = pick(H.fwd, rho), h1 = (H.lex + frho) >> 1;  // y + rho (op)
+    M3<T> R;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) R.e[i][j] = mk(T(0), T(0));
 #pragma unroll 1
-    for (int s = 0; s < 4; s++) {
-        if (s == rho) continue;
-        const int a = s < rho ? s : rho, b = s < rho ? rho : s;
-        const int pl = plane_of(a, b);
-        const bool rho_is_b = (rho == b);
-#pragma unroll 1
-        for (int l = 0; l < 4; l++) {
-#pragma unroll 1
-            for (int k = 0; k < 4; k++) {
-                const LeafFactor fk = c_leaves[l][k];
-                if ((fk.dir_b != 0) != rho_is_b) continue;
-                // clover centre x with x + offset_k = y
-                int x[4];
-#pragma unroll
-                for (int d = 0; d < 4; d++) x[d] = wrap(y[d] - (d == a ? fk.oa : 0) - (d == b ? fk.ob : 0), g.L[d]);
-                const int xpar = (x[0] + x[1] + x[2] + x[3]) & 1;
-                T c[8];
-                const T* cp = C.at(pl, xpar, lex_of(g, x) >> 1);
-#pragma unroll
-                for (int q = 0; q < 8; q++) c[q] = cp[(size_t)q * C.S];
-                const M3<T> cq = herm_from_coeffs(c);  // C = i Q
-                M3<T> Cm;
-#pragma unroll
-                for (int i = 0; i < 3; i++)
-#pragma unroll
-                    for (int j = 0; j < 3; j++) Cm.e[i][j] = mk(-cq.e[i][j].im, cq.e[i][j].re);
-                // R_k = F_{k+1} .. F_4 C F_1 .. F_{k-1}
-                M3<T> R = unit3<T>();
-                for (int j = k + 1; j < 4; j++) R = mul_nn(R, factor(U, g, x, a, b, c_leaves[l][j]));
-                R = mul_nn(R, Cm);
-                for (int j = 0; j < k; j++) R = mul_nn(R, factor(U, g, x, a, b, c_leaves[l][j]));
-                const M3<T> Fk = factor(U, g, x, a, b, fk);
-                T t[8];
-                if (!fk.dag) {
-                    ta_coeffs(mul_nn(Fk, R), t);
-#pragma unroll
-                    for (int q = 0; q < 8; q++) acc[q] += T(0.25) * t[q];
-                } else {
-                    ta_coeffs(mul_nn(R, Fk), t);
-#pragma unroll
-                    for (int q = 0; q < 8; q++) acc[q] -= T(0.25) * t[q];
-                }
-            }
+    for (int K = 0; K < 3; K++) {
+        const int nu = K < rho ? K : K + 1;
+        const int pl = rho < nu ? plane_of(rho, nu) : plane_of(nu, rho);
+        M3<T> Sd;  // s (S_up - S_dn) summed over the sides, and R's part of the plane
+        M3<T> Rp;
+        {
+            const int h3 = (H.lex + pick(H.fwd, nu)) >> 1, h2 = (H.lex + frho + pick(H.fwd, nu)) >> 1;  // y + nu (op), y + rho + nu (par)
+            const M3<T> X1 = U.load(nu, op, h1), X2d = U.load(rho, op, h3);
+            const M3<T> P = mul_nd(X1, X2d);
+            M3<T> Q = mul_nd(mul_nn(X1, corner(C, pl, par, h2)), X2d);
+            acc_add(Q, mul_nn(P, corner(C, pl, op, h3)));
+            const M3<T> X3d = U.load(nu, par, h);
+            Rp = mul_nd(Q, X3d);
+            Sd = mul_nd(P, X3d);
         }
+        {
+            const int bnu = pick(H.bwd, nu), h3 = (H.lex + bnu) >> 1, h2 = (H.lex + frho + bnu) >> 1;  // y - nu (op), y + rho - nu (par)
+            const M3<T> Y1d = U.load(nu, par, h2), Y2d = U.load(rho, op, h3);
+            const M3<T> P = mul_dd(Y1d, Y2d);
+            M3<T> Q = mul_nd(mul_dn(Y1d, corner(C, pl, par, h2)), Y2d);
+            acc_add(Q, mul_nn(P, corner(C, pl, op, h3)));
+            const M3<T> Y3 = U.load(nu, op, h3);
+            acc_sub(Rp, mul_nn(Q, Y3));
+            acc_sub(Sd, mul_nn(P, Y3));
+        }
+        acc_add(Rp, mul_nn(corner(C, pl, op, h1), Sd));
+        acc_add(Rp, mul_nn(Sd, corner(C, pl, par, h)));
+        if (rho < nu) acc_add(R, Rp);
+        else acc_sub(R, Rp);
     }
+    T t[8];
+    ta_coeffs(mul_nn(U.load(rho, par, h), R), t);
     T* out = Lam.at(rho, par, h);
+    const T f = T(0.25) * scl;
 #pragma unroll
-    for (int q = 0; q < 8; q++) out[q * Alg<T>::kStep] += scl * acc[q];
+    for (int q = 0; q < 8; q++) out[q * Alg<T>::kStep] += f * t[q];
 }
 
 static inline int nblk(long n, int t) { return (int)((n + t - 1) / t); }
@@ -175,8 +157,8 @@ mgq_status mgq_clover_vjp(const mgq_lattice* lat, int observable, double scale, 
         Planes6<T> C;
         C.p = reinterpret_cast<T*>(scratch);
         C.S = g.S;
-        k_clover_cotangent<T, NP><<<nblk(g.V, 128), 128, 0, st>>>(links_of<T, NP>(lat), g, observable, C);
-        k_clover_vjp<T, NP><<<nblk(8L * g.Vh, 128), 128, 0, st>>>(links_of<T, NP>(lat), g, C, (T)scale,
+        k_clover_cotangent<T, NP><<<dim3(nblk(g.V, 128), 3), 128, 0, st>>>(links_of<T, NP>(lat), g, observable, C);
+        k_clover_vjp<T, NP><<<dim3(nblk(g.Vh, 128), 8), 128, 0, st>>>(links_of<T, NP>(lat), g, C, (T)scale,
                                                                    alg_at<T>(lambda, lat->dims));
     });
     return cuda_check("mgq_clover_vjp");

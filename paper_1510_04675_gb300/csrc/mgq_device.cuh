@@ -415,6 +415,23 @@ __device__ __forceinline__ Hops make_hops(const Geom& g, const int x[4]) {
     return H;
 }
 
+// The same for hops of m steps: lex(x + m e_d) = lex + fwd[d] (m may exceed L_d).
+__device__ __forceinline__ Hops make_hops(const Geom& g, const int x[4], int m) {
+    Hops H;
+    int st = 1;
+#pragma unroll
+    for (int d = 0; d < 4; d++) {
+        int f = x[d] + m, b = x[d] - m;
+        while (f >= g.L[d]) f -= g.L[d];
+        while (b < 0) b += g.L[d];
+        H.fwd[d] = (f - x[d]) * st;
+        H.bwd[d] = (b - x[d]) * st;
+        st *= g.L[d];
+    }
+    H.lex = lex_of(g, x);
+    return H;
+}
+
 // a[d] for a run-time d without dynamic indexing (keeps a[] in registers)
 __device__ __forceinline__ int pick(const int a[4], int d) { return d == 0 ? a[0] : d == 1 ? a[1] : d == 2 ? a[2] : a[3]; }
 
@@ -632,6 +649,17 @@ template <class T> __device__ __forceinline__ M3<T> herm_from_coeffs(const T c[8
     q.e[1][2] = mk(h * c[5], -h * c[6]);
     q.e[2][1] = mk(h * c[5], h * c[6]);
     return q;
+}
+
+// i Q for hermitian Q: the antihermitian matrix sum_a c_a X_a
+template <class T> __device__ __forceinline__ M3<T> alg_matrix(const T c[8]) {
+    const M3<T> q = herm_from_coeffs(c);
+    M3<T> r;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) r.e[i][j] = mk(-q.e[i][j].im, q.e[i][j].re);
+    return r;
 }
 
 // Coefficients of exp(i Q) = f0 + f1 Q + f2 Q^2, Q hermitian and traceless with

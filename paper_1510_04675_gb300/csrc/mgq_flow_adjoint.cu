@@ -24,17 +24,6 @@ namespace mgq {
 mgq_status force_accumulate(const mgq_lattice* lat, void* B, double coef, double alpha, cudaStream_t st);
 mgq_status exp_update(const mgq_lattice* lat, void* B, double s, cudaStream_t st);
 
-// i Q for hermitian Q: the antihermitian matrix sum_a c_a X_a
-template <class T> __device__ __forceinline__ M3<T> alg_matrix(const T c[8]) {
-    const M3<T> q = herm_from_coeffs(c);
-    M3<T> r;
-#pragma unroll
-    for (int i = 0; i < 3; i++)
-#pragma unroll
-        for (int j = 0; j < 3; j++) r.e[i][j] = mk(-q.e[i][j].im, q.e[i][j].re);
-    return r;
-}
-
 // [a, b] for antihermitian a, b: b a = (a b)^+, so [a, b] = a b - (a b)^+ from
 // one product; the result is antihermitian entry by entry (r_ji = -conj(r_ij)
 // exactly, the diagonal purely imaginary).

@@ -73,9 +73,14 @@ mgq_status heatbath_subsweep(mgq_lattice* lat, double beta, uint64_t sweep, int 
 mgq_status overrelax_subsweep(mgq_lattice* lat, int mu, int par, cudaStream_t st);
 // E (site average) and Q of the clover field strength into dev_out[0], dev_out[1]
 mgq_status clover_into(const mgq_lattice* lat, double* partials, double* dev_out, cudaStream_t st);
-// Per-block E and Q partial sums (E at partials[0..nb), Q at partials[nb..2nb));
-// skipped when gate != nullptr and *gate == 0.  Returns nb.
-int clover_partials(const mgq_lattice* lat, double* partials, const int* gate, cudaStream_t st);
+// Per-block E and Q partial sums (E at partials[0..nb), Q at partials[nb..2nb)) of
+// the clover with lines of m links a side at `lines` (the links, or line_field's
+// products); skipped when gate != nullptr and *gate == 0.  Returns nb.
+int clover_partials(const mgq_lattice* lat, const void* lines, int m, double* partials, const int* gate, cudaStream_t st);
+// lines_out <- the products of m links in every direction, lines_out(x) =
+// lines_in(x) U(x + m - 1): lines_in holds those of m - 1 links (the links for
+// m = 2) and may be lines_out itself
+void line_field(const mgq_lattice* lat, const void* lines_in, void* lines_out, int m, cudaStream_t st);
 
 inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 

@@ -7,93 +7,106 @@
 
 namespace mgq {
 
-// Product of the links along the straight path of `len` steps in direction
-// mu starting at x (coordinates updated in place to the end point).
+// P <- P times the `len` links in direction mu from the site (lexicographic index
+// lex, coordinate c along mu, parity par) on, which move along.  FP32: rows 0, 1
+// of P (a left factor throughout).
 template <class T, int NP>
-__device__ __forceinline__ M3<T> line(const Links<T, NP>& U, const Geom& g, int x[4], int mu, int len) {
-    M3<T> L = unit3<T>();
+__device__ __forceinline__ void extend_line(M3<T>& P, const Links<T, NP>& U, int mu, int len, int L, int stride, int& lex,
+                                            int& c, int& par) {
     for (int k = 0; k < len; k++) {
-        const int lex = lex_of(g, x);
-        const int par = (x[0] + x[1] + x[2] + x[3]) & 1;
-        L = mul_nn(L, U.load(mu, par, lex >> 1));
-#pragma unroll
-        for (int d = 0; d < 4; d++)
-            if (d == mu) x[d] = wrap(x[d] + 1, g.L[d]);
+        const M3<T> u = U.load(mu, par, lex >> 1);
+        if constexpr (sizeof(T) == 4) P = mul_nn_2(P, u);
+        else P = mul_nn(P, u);
+        const bool last = ++c == L;
+        lex += last ? stride * (1 - L) : stride;
+        if (last) c = 0;
+        par ^= 1;
     }
-    return L;
 }
 
-// (1/3) Re Tr L^m_mu(x) L^n_nu(x+m mu) [L^n_nu(x) L^m_mu(x+n nu)]^+
+// L^m_mu(x) L^n_nu(x + m mu): the path along mu, then nu
 template <class T, int NP>
-__device__ __forceinline__ double loop_mn(const Links<T, NP>& U, const Geom& g, const int x[4], int mu, int nu, int m, int n) {
-    int y[4] = {x[0], x[1], x[2], x[3]};
-    const M3<T> a1 = line(U, g, y, mu, m);
-    const M3<T> a2 = line(U, g, y, nu, n);
-    int z[4] = {x[0], x[1], x[2], x[3]};
-    const M3<T> b1 = line(U, g, z, nu, n);
-    const M3<T> b2 = line(U, g, z, mu, m);
-    return (double)retr_nd(mul_nn(a1, a2), mul_nn(b1, b2)) / 3.0;
+__device__ __forceinline__ M3<T> corner_path(const Links<T, NP>& U, const Geom& g, const int x[4], int par, int mu, int m, int nu,
+                                             int n) {
+    const int st[4] = {1, g.L[0], g.L[0] * g.L[1], g.L[0] * g.L[1] * g.L[2]};
+    const int smu = pick(st, mu), Lmu = pick(g.L, mu);
+    int lex = lex_of(g, x), c = pick(x, mu);
+    M3<T> P = load_left(U, mu, par, lex >> 1);
+    const bool last = ++c == Lmu;
+    lex += last ? smu * (1 - Lmu) : smu;
+    if (last) c = 0;
+    par ^= 1;
+    extend_line(P, U, mu, m - 1, Lmu, smu, lex, c, par);
+    c = pick(x, nu);
+    extend_line(P, U, nu, n, pick(g.L, nu), pick(st, nu), lex, c, par);
+    return P;
 }
 
+__device__ __forceinline__ int plane_mu(int p) { return p < 3 ? 0 : (p < 5 ? 1 : 2); }
+__device__ __forceinline__ int plane_nu(int p) { return p < 3 ? p + 1 : (p < 5 ? p - 1 : 3); }
+
+// Re Tr L^m_mu(x) L^n_nu(x+m mu) [L^n_nu(x) L^m_mu(x+n nu)]^+, one thread per site
+// and plane (block row y): two paths of m + n links, FP32 in two rows throughout
+// (2x3 loops of 24^3x48, FP32 12-real: 355 -> 176 us)
 template <class T, int NP>
 __global__ void __launch_bounds__(128) k_wilson_loop(Links<T, NP> U, Geom g, int m, int n, double* __restrict__ partials) {
+    const int mu = plane_mu(blockIdx.y), nu = plane_nu(blockIdx.y);
     double acc = 0.0;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < g.V; idx += gridDim.x * blockDim.x) {
         const int par = idx >= g.Vh, h = idx - par * g.Vh;
         int x[4];
         cb_coords(g, par, h, x);
-#pragma unroll 1
-        for (int mu = 0; mu < 3; mu++)
-#pragma unroll 1
-            for (int nu = mu + 1; nu < 4; nu++) acc += loop_mn(U, g, x, mu, nu, m, n);
+        const M3<T> a = corner_path(U, g, x, par, mu, m, nu, n), b = corner_path(U, g, x, par, nu, n, mu, m);
+        if constexpr (sizeof(T) == 4) acc += (double)retr_two_row(a, b);
+        else acc += retr_nd(a, b);
     }
     acc = block_sum(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = acc;
+    if (threadIdx.x == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = acc;
 }
 
-// 8 class sums (W1x1 by chi_munu = 0..2, W2x2 by chi = 0..4) and max s_p:
-// partials[q * gridDim.x + block] for q = 0..7, maxima in partials[8 * gridDim.x + block]
+// 8 class sums of Re Tr (1x1 loops by chi_munu = 0..2, 2x2 loops by chi = 0..4) and
+// the least Re Tr of the 1x1 loops: partials[q * nb + block] for q = 0..7, minima in
+// partials[8 * nb + block], nb = gridDim.x * 6.  One thread per site and plane
+// (block row y); U2 holds the lines of two links.  24^3x48, FP32 12-real: 571 us
+// with the 2x2 loops multiplied out link by link and thirds taken in FP64 per loop,
+// now 177 us after 40 us for the lines.
 template <class T, int NP>
-__global__ void __launch_bounds__(128) k_partial_loops(Links<T, NP> U, Geom g, double* __restrict__ partials) {
+__global__ void __launch_bounds__(128) k_partial_loops(Links<T, NP> U, Links<T, NP> U2, Geom g, double* __restrict__ partials) {
+    const int mu = plane_mu(blockIdx.y), nu = plane_nu(blockIdx.y);
     double a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    double hmax = 0.0;
+    T least = T(3);
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < g.V; idx += gridDim.x * blockDim.x) {
         const int par = idx >= g.Vh, h = idx - par * g.Vh;
         int x[4];
         cb_coords(g, par, h, x);
         const int chi = (x[0] & 1) + (x[1] & 1) + (x[2] & 1) + (x[3] & 1);
-#pragma unroll 1
-        for (int mu = 0; mu < 3; mu++)
-#pragma unroll 1
-            for (int nu = mu + 1; nu < 4; nu++) {
-                int cmn = 0;
+        const int cmn = chi - (pick(x, mu) & 1) - (pick(x, nu) & 1);
+        const T w1 = loop_retr(U, make_hops(g, x), par, par ^ 1, mu, nu);
+        const T w2 = loop_retr(U2, make_hops(g, x, 2), par, par, mu, nu);
+        least = w1 < least ? w1 : least;
+        // the sites of a warp mostly share their classes: one branch taken
 #pragma unroll
-                for (int r = 0; r < 4; r++)
-                    if (r != mu && r != nu) cmn += x[r] & 1;
-                const double w1 = loop_mn(U, g, x, mu, nu, 1, 1);
-                const double w2 = loop_mn(U, g, x, mu, nu, 2, 2);
+        for (int d = 0; d < 3; d++)
+            if (d == cmn) a[d] += (double)w1;
 #pragma unroll
-                for (int d = 0; d < 3; d++)
-                    if (d == cmn) a[d] += w1;
-#pragma unroll
-                for (int d = 0; d < 5; d++)
-                    if (d == chi) a[3 + d] += w2;
-                hmax = fmax(hmax, 3.0 * (1.0 - w1));
-            }
+        for (int d = 0; d < 5; d++)
+            if (d == chi) a[3 + d] += (double)w2;
     }
+    const int nb = gridDim.x * gridDim.y, b = blockIdx.y * gridDim.x + blockIdx.x;
 #pragma unroll
     for (int q = 0; q < 8; q++) {
         const double s = block_sum(a[q]);
-        if (threadIdx.x == 0) partials[q * gridDim.x + blockIdx.x] = s;
+        if (threadIdx.x == 0) partials[q * nb + b] = s;
     }
+    // h's part 3 (1 - W) of a loop, W = Re Tr / 3, is largest where Re Tr is least
     __shared__ double smax[128];
-    smax[threadIdx.x] = hmax;
+    smax[threadIdx.x] = 3.0 * (1.0 - (double)least / 3.0);
     __syncthreads();
     for (int o = blockDim.x / 2; o > 0; o >>= 1) {
         if ((int)threadIdx.x < o) smax[threadIdx.x] = fmax(smax[threadIdx.x], smax[threadIdx.x + o]);
         __syncthreads();
     }
-    if (threadIdx.x == 0) partials[8 * gridDim.x + blockIdx.x] = smax[0];
+    if (threadIdx.x == 0) partials[8 * nb + b] = smax[0];
 }
 
 __global__ void k_max_final(const double* __restrict__ partials, int n, double* out) {
@@ -129,12 +142,12 @@ mgq_status mgq_wilson_loop(const mgq_lattice* lat, int m, int n, double* out, vo
     if (!out) return fail(MGQ_EINVAL, "mgq_wilson_loop: out is NULL");
     const Geom g = make_geom(lat->dims);
     cudaStream_t st = as_stream(stream);
-    const int nb = reduction_blocks(g.V, 128);
+    const int nb = reduction_blocks(g.V, 128);  // at most 1184: 6 x 1184 partial sums
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
-        k_wilson_loop<T, NP><<<nb, 128, 0, st>>>(links_of<T, NP>(lat), g, m, n, ws_partials(lat));
+        k_wilson_loop<T, NP><<<dim3(nb, 6), 128, 0, st>>>(links_of<T, NP>(lat), g, m, n, ws_partials(lat));
     });
     double* sc = ws_scalars(lat);
-    launch_final_sum(ws_partials(lat), nb, 1.0 / (6.0 * (double)g.V), sc + 24, st);
+    launch_final_sum(ws_partials(lat), 6 * nb, 1.0 / (18.0 * (double)g.V), sc + 24, st);
     if ((s = cuda_check("mgq_wilson_loop"))) return s;
     return deliver(sc + 24, out, 1, st, "mgq_wilson_loop");
 }
@@ -146,18 +159,21 @@ mgq_status mgq_partial_loops(const mgq_lattice* lat, double* out, void* stream) 
     if (!out) return fail(MGQ_EINVAL, "mgq_partial_loops: out is NULL");
     const Geom g = make_geom(lat->dims);
     cudaStream_t st = as_stream(stream);
-    int nb = reduction_blocks(g.V, 128);
-    if (nb > (int)(WS_NPARTIALS / 9)) nb = (int)(WS_NPARTIALS / 9);
+    int nbx = reduction_blocks(g.V, 128);
+    if (nbx > (int)(WS_NPARTIALS / 54)) nbx = (int)(WS_NPARTIALS / 54);
+    const int nb = 6 * nbx;
+    line_field(lat, lat->links, ws_links(lat), 2, st);
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
-        k_partial_loops<T, NP><<<nb, 128, 0, st>>>(links_of<T, NP>(lat), g, ws_partials(lat));
+        k_partial_loops<T, NP><<<dim3(nbx, 6), 128, 0, st>>>(links_of<T, NP>(lat), links_at<T, NP>(ws_links(lat), lat->dims), g,
+                                                             ws_partials(lat));
     });
     double* sc = ws_scalars(lat);
     const double V = (double)g.V;
     for (int d = 0; d < 3; d++)
-        launch_final_sum(ws_partials(lat) + d * nb, nb, 1.0 / (2.0 * (4 - d) * (3 - d) * binom(4, d) * V / 16.0),
+        launch_final_sum(ws_partials(lat) + d * nb, nb, 1.0 / (6.0 * (4 - d) * (3 - d) * binom(4, d) * V / 16.0),
                          sc + 24 + d, st);
     for (int d = 0; d < 5; d++)
-        launch_final_sum(ws_partials(lat) + (3 + d) * nb, nb, 1.0 / (6.0 * binom(4, d) * V / 16.0), sc + 27 + d, st);
+        launch_final_sum(ws_partials(lat) + (3 + d) * nb, nb, 1.0 / (18.0 * binom(4, d) * V / 16.0), sc + 27 + d, st);
     k_max_final<<<1, 256, 0, st>>>(ws_partials(lat) + 8 * nb, nb, sc + 32);
     if ((s = cuda_check("mgq_partial_loops"))) return s;
     return deliver(sc + 24, out, 9, st, "mgq_partial_loops");

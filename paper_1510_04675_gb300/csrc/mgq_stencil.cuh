@@ -329,40 +329,102 @@ __device__ __forceinline__ double site_plaquettes(const Links<T, NP>& U, const G
 }
 
 // =============================================================== clover
+// The three loops around the unit square of lines with sides A_mu, A_nu are
+// written for a line field A_d(x) (the links, or products of m links) whose hops H
+// are the lines' lengths; op is the parity one line away.
+
+// a b^+ c^+ and (e d)^+ f of lines in SU(3).  FP32: rows 0, 1 of every partial
+// product, row 2 rebuilt.
+template <class T> __device__ __forceinline__ M3<T> up_term(const M3<T>& a_rows, const M3<T>& b, const M3<T>& c) {
+    if constexpr (sizeof(T) == 4) {
+        M3<T> r = mul_nd_2(mul_nd_2(a_rows, b), c);
+        rebuild_row2(r);
+        return r;
+    } else {
+        return mul_nd(mul_nd(a_rows, b), c);
+    }
+}
+template <class T> __device__ __forceinline__ M3<T> down_term(const M3<T>& e_rows, const M3<T>& d, const M3<T>& f) {
+    if constexpr (sizeof(T) == 4) {
+        M3<T> t = mul_nn_2(e_rows, d);
+        rebuild_row2(t);
+        M3<T> r = mul_dn_2(t, f);
+        rebuild_row2(r);
+        return r;
+    } else {
+        return mul_dn(mul_nn(e_rows, d), f);
+    }
+}
+// a link that enters as a left factor: FP32 needs its rows 0, 1 only
+template <class T, int NP> __device__ __forceinline__ M3<T> load_left(const Links<T, NP>& U, int mu, int par, int h) {
+    if constexpr (sizeof(T) == 4) return U.load_rows(mu, par, h);
+    else return U.load(mu, par, h);
+}
+template <class T> __device__ __forceinline__ void acc_sub(M3<T>& a, const M3<T>& b) {
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) a.e[i][j] = a.e[i][j] - b.e[i][j];
+}
+
 // Clover leaves around x in the (mu,nu) plane, all starting and ending at x,
-// counterclockwise; returns the algebra coefficients g of
-// G = traceless part of (Q - Q^+)/8, i.e. g = t(TA(Q))/4.
+// counterclockwise; the algebra coefficients g of G = traceless part of
+// (Q - Q^+)/8, i.e. g = t(TA(Q))/4.  TA(M^+) = -TA(M), so the leaves l1 and l4 that
+// hold U_mu(x), and l2 and l3 that hold U_mu(x-mu), come in pairs with one product
+// for that link:
+//   l1 - l4^+ = U_mu(x) [U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+ - U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu)]
+//   l2 - l3^+ = [U_nu(x) U_mu(x-mu+nu)^+ U_nu(x-mu)^+ - U_nu(x-nu)^+ U_mu(x-mu-nu)^+ U_nu(x-mu-nu)] U_mu(x-mu)
+// ten products, eight of them in two-row form in FP32, where four separate leaves
+// take twelve full ones.
 template <class T, int NP>
-__device__ __forceinline__ void clover_coeffs(const Links<T, NP>& U, const Geom& g, const int x[4], int par, int h, int mu,
-                                              int nu, T out[8]) {
-    const int op = par ^ 1;
-    const int lpm = lex_hop(g, x, mu, +1), lpn = lex_hop(g, x, nu, +1);
-    const int lmm = lex_hop(g, x, mu, -1), lmn = lex_hop(g, x, nu, -1);
-    const int lmm_pn = lex_hop(g, x, mu, -1, nu, +1);
-    const int lmm_mn = lex_hop(g, x, mu, -1, nu, -1);
-    const int lpm_mn = lex_hop(g, x, mu, +1, nu, -1);
-    const M3<T> umu = U.load(mu, par, h), unu = U.load(nu, par, h);
-    // l1 = U_mu(x) U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+
-    M3<T> Q = mul_nd(mul_nn(umu, U.load(nu, op, lpm >> 1)), mul_nn(unu, U.load(mu, op, lpn >> 1)));
-    // l2 = U_nu(x) U_mu(x-mu+nu)^+ U_nu(x-mu)^+ U_mu(x-mu)
+__device__ __forceinline__ void clover_coeffs(const Links<T, NP>& U, const Hops& H, int par, int op, int mu, int nu, T out[8]) {
+    const int fm = pick(H.fwd, mu), fn = pick(H.fwd, nu), bm = pick(H.bwd, mu), bn = pick(H.bwd, nu);
+    const int x = H.lex;
+    M3<T> Q;
     {
-        const M3<T> a = U.load(mu, par, lmm_pn >> 1), b = U.load(nu, op, lmm >> 1), c = U.load(mu, op, lmm >> 1);
-        acc_add(Q, mul_nn(mul_nd(unu, a), mul_dn(b, c)));
+        M3<T> D = up_term(load_left(U, nu, op, (x + fm) >> 1), U.load(mu, op, (x + fn) >> 1), U.load(nu, par, x >> 1));
+        acc_sub(D, down_term(load_left(U, mu, op, (x + bn) >> 1), U.load(nu, par, (x + fm + bn) >> 1), U.load(nu, op, (x + bn) >> 1)));
+        Q = mul_nn(U.load(mu, par, x >> 1), D);
     }
-    // l3 = U_mu(x-mu)^+ U_nu(x-mu-nu)^+ U_mu(x-mu-nu) U_nu(x-nu)
     {
-        const M3<T> a = U.load(mu, op, lmm >> 1), b = U.load(nu, par, lmm_mn >> 1), c = U.load(mu, par, lmm_mn >> 1),
-                    d = U.load(nu, op, lmn >> 1);
-        acc_add(Q, mul_nn(mul_dd(a, b), mul_nn(c, d)));
-    }
-    // l4 = U_nu(x-nu)^+ U_mu(x-nu) U_nu(x+mu-nu) U_mu(x)^+
-    {
-        const M3<T> a = U.load(nu, op, lmn >> 1), b = U.load(mu, op, lmn >> 1), c = U.load(nu, par, lpm_mn >> 1);
-        acc_add(Q, mul_nd(mul_nn(mul_dn(a, b), c), umu));
+        M3<T> D = up_term(load_left(U, nu, par, x >> 1), U.load(mu, par, (x + bm + fn) >> 1), U.load(nu, op, (x + bm) >> 1));
+        acc_sub(D, down_term(load_left(U, mu, par, (x + bm + bn) >> 1), U.load(nu, op, (x + bn) >> 1),
+                             U.load(nu, par, (x + bm + bn) >> 1)));
+        acc_add(Q, mul_nn(D, U.load(mu, op, (x + bm) >> 1)));
     }
     ta_coeffs(Q, out);
 #pragma unroll
     for (int a = 0; a < 8; a++) out[a] *= T(0.25);
+}
+
+// The dual pairs of planes (01, 23), (02, 13), (03, 12): pair p's second plane.
+__device__ __forceinline__ int dual_mu(int p) { return p == 0 ? 2 : 1; }
+__device__ __forceinline__ int dual_nu(int p) { return p == 2 ? 2 : 3; }
+
+// Re Tr of the loop A_mu(x) A_nu(x+mu) (A_nu(x) A_mu(x+nu))^+ of SU(3) lines.  FP32:
+// a = A_mu(x) A_nu(x+mu) and b = A_nu(x) A_mu(x+nu) are in SU(3), so rows 0, 1 of
+// each suffice: with s_ij = row_i(a) . conj(row_j(b)), Tr(a b^+) = s00 + s11 +
+// conj(s00 s11 - s01 s10) (row 2 = conj(row0 x row1); Binet-Cauchy).
+__device__ __forceinline__ float retr_two_row(const M3<float>& a, const M3<float>& b) {
+    Cx<float> sij[2][2];
+#pragma unroll
+    for (int i = 0; i < 2; i++)
+#pragma unroll
+        for (int j = 0; j < 2; j++)
+            sij[i][j] = mulc(a.e[i][0], b.e[j][0]) + mulc(a.e[i][1], b.e[j][1]) + mulc(a.e[i][2], b.e[j][2]);
+    const Cx<float> d = sij[0][0] * sij[1][1] - sij[0][1] * sij[1][0];
+    return sij[0][0].re + sij[1][1].re + d.re;
+}
+template <class T, int NP>
+__device__ __forceinline__ T loop_retr(const Links<T, NP>& U, const Hops& H, int par, int op, int mu, int nu) {
+    const int x = H.lex >> 1, xm = (H.lex + pick(H.fwd, mu)) >> 1, xn = (H.lex + pick(H.fwd, nu)) >> 1;
+    if constexpr (sizeof(T) == 4) {
+        const M3<T> a = mul_nn_2(U.load_rows(mu, par, x), U.load(nu, op, xm));
+        return retr_two_row(a, mul_nn_2(U.load_rows(nu, par, x), U.load(mu, op, xn)));
+    } else {
+        const M3<T> a = mul_nn(U.load(mu, par, x), U.load(nu, op, xm));
+        return retr_nd(a, mul_nn(U.load(nu, par, x), U.load(mu, op, xn)));
+    }
 }
 
 // =============================================================== SU(2) steps
