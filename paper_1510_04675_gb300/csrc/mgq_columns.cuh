@@ -15,7 +15,9 @@
 //     exchange the four entries of V's block, and the rotation's scalars are
 //     computed by all lanes of a link;
 //   - the reunitarisation exchanges norms, inner products and row entries.
-// One compound sweep (1 heat bath + 4 overrelaxation) of 8^4: 3.76 -> 1.66 ms.
+// One compound sweep (1 heat bath + 4 overrelaxation) of 8^4: 3.77 -> 0.94 ms (an
+// overrelaxation launch 94 -> 21 us, a heat bath 118 -> 40 us); the force of 8^3x12
+// 95 -> 83 us.
 // Every operation and its order are those of the one-thread form (staple_full,
 // hb_link, or_link), so both agree bit for bit.
 #pragma once
@@ -116,7 +118,7 @@ __device__ __forceinline__ void left_column(const Cx<double>* link, const Cx<dou
     }
 }
 
-// block_w of V's (i, j) block, V held by columns
+// block_w of V's (i, j) block, V held by columns in the lanes from base on
 __device__ __forceinline__ void column_block_w(const Cx<double> v[3], int i, int j, int base, double w[4]) {
     const Cx<double> vii = shfl_cx(v[i], base + i), vji = shfl_cx(v[j], base + i);
     const Cx<double> vij = shfl_cx(v[i], base + j), vjj = shfl_cx(v[j], base + j);
@@ -150,10 +152,9 @@ template <bool HB, int LPL>
 __global__ void __launch_bounds__(COL_THREADS) k_update_columns(Links<double, 9> U, Geom g, int mu, int par, double beta,
                                                                 RngKey rk, int n_hb, uint8_t* __restrict__ dec,
                                                                 double* __restrict__ partials) {
-    pdl_launch_dependents();
     const ColumnLane<LPL> c;
     const int h0 = c.item();
-    const bool live = c.active && h0 < g.Vh && c.half == 0;
+    const bool live = c.active && h0 < g.Vh && c.half == (LPL == 6 ? 1 : 0);  // the lanes that end with U
     const int h = h0 < g.Vh ? h0 : g.Vh - 1;
     int x[4];
     cb_coords(g, par, h, x);
@@ -164,11 +165,17 @@ __global__ void __launch_bounds__(COL_THREADS) k_update_columns(Links<double, 9>
     double acc = 0.0;
     if (!HB && par == 1) acc = c.k == 0 ? v[0].re : (c.k == 1 ? v[1].re : v[2].re);  // Re Tr(U A), kept by the update
     const int lex = lex_of(g, x);
+    // six lanes: the lower half carries V through the rotations, the upper half U
+    if (LPL == 6 && c.half == 0) {
+#pragma unroll
+        for (int i = 0; i < 3; i++) u[i] = v[i];
+    }
+    const int vbase = c.base - 3 * c.half;
 #pragma unroll
     for (int s = 0; s < 3; s++) {
         const int i = (s == 2) ? 1 : 0, j = (s == 0) ? 1 : 2;
         double w[4], R[4];
-        column_block_w(v, i, j, c.base, w);
+        column_block_w(LPL == 6 ? u : v, i, j, vbase, w);
         bool turn = false;
         if constexpr (HB) {
             const double xi = m_sqrt(quat_norm2(w));
@@ -186,10 +193,13 @@ __global__ void __launch_bounds__(COL_THREADS) k_update_columns(Links<double, 9>
         }
         if (turn) {
             su2_pair(u[i], u[j], R);
-            if (s < 2) su2_pair(v[i], v[j], R);
+            if (LPL == 3 && s < 2) su2_pair(v[i], v[j], R);
         }
     }
     column_reunitarize(u, c.k, c.base);
+    // only now: blocks of the next launch that settle while these run find their
+    // places on the idle SMs, two and three deep, and then run at half the rate
+    pdl_launch_dependents();
     if (live) {
         Cx<double>* b = U.base(mu, par, h);
 #pragma unroll
@@ -209,15 +219,55 @@ __global__ void __launch_bounds__(COL_THREADS) k_update_columns(Links<double, 9>
     }
 }
 
-// Lanes per link for a launch over n links: 1 (one thread per link), 3 or 6, by
-// the FP64 operations of the longest chain (a link's operations per lane, times
-// the warps that share a sub-partition).  Operation counts: 2000 for a whole link,
-// 800 for a column, 580 for a column with half the staple terms.
-inline int lanes_per_link(long n) {
+// B <- alpha B + coef t(TA(U A)) on every link (as k_force), block row y the (mu,
+// parity) plane.  With M = U A by columns, lane k holds M_nk of the pair (k, n),
+// n = k + 1 mod 3, and gets M_kn: two coefficients each, the diagonal ones by all.
+template <int LPL>
+__global__ void __launch_bounds__(COL_THREADS) k_force_columns(Links<double, 9> U, Geom g, Alg<double> B, double coef, double alpha) {
+    const ColumnLane<LPL> c;
+    const int mu = blockIdx.y >> 1, par = blockIdx.y & 1, h0 = c.item(), h = h0 < g.Vh ? h0 : g.Vh - 1;
+    int x[4];
+    cb_coords(g, par, h, x);
+    pdl_wait();
+    Cx<double> A[3], u[3], v[3];
+    staple_column<LPL>(U, g, x, h, mu, par, c, A);
+    left_column(U.base(mu, par, h), A, c.k, u, v);
+    // v = column k of M.  Entry (k, n) sits in lane n, row k; lane n serves its
+    // predecessor k = n - 1, so each lane offers the entry of that row
+    const Cx<double> offer = c.k == 0 ? v[2] : (c.k == 1 ? v[0] : v[1]);
+    const Cx<double> got = shfl_cx(offer, c.base + (c.k + 1) % 3);
+    const Cx<double> has = c.k == 0 ? v[1] : (c.k == 1 ? v[2] : v[0]);
+    const double dk = c.k == 0 ? v[0].im : (c.k == 1 ? v[1].im : v[2].im);
+    const double d0 = __shfl_sync(0xffffffffu, dk, c.base), d1 = __shfl_sync(0xffffffffu, dk, c.base + 1),
+                 d2 = __shfl_sync(0xffffffffu, dk, c.base + 2);
+    pdl_launch_dependents();
+    if (!c.active || h0 >= g.Vh || c.half) return;
+    const double re = c.k == 2 ? has.re - got.re : got.re - has.re;  // t_1, t_6, t_4 = Re(M_ij - M_ji), i < j
+    const double diag = c.k == 0 ? d0 - d1 : (d0 + d1 - 2.0 * d2) * 0.57735026918962576451;
+    double* b = B.at(mu, par, h);
+    auto put = [&](int a, double t) {
+        double& o = b[a * Alg<double>::kStep];
+        o = alpha == 0.0 ? coef * t : alpha * o + coef * t;
+    };
+    const int a = c.k == 0 ? 0 : (c.k == 1 ? 5 : 3);  // pairs 01, 12, 02
+    put(a, has.im + got.im);
+    put(a + 1, re);
+    if (c.k < 2) put(c.k == 0 ? 2 : 7, diag);
+}
+
+// Lanes per link (1: a thread for each; 3; 6) of a launch over n links, from the
+// FP64 operations of a link's chain per lane and the warps that share one of the
+// 608 sub-partitions: whichever ends first.
+inline int lanes_per_link(long n, long ops1, long ops3, long ops6) {
     constexpr long kPartitions = 152 * 4;
     auto cost = [](long warps, long ops) { return (warps + kPartitions - 1) / kPartitions * ops; };
-    const long one = cost((n + 31) / 32, 2000), three = cost((n + 9) / 10, 800), six = cost((n + 4) / 5, 580);
+    const long one = cost((n + 31) / 32, ops1), three = cost((n + 9) / 10, ops3), six = cost((n + 4) / 5, ops6);
     return one <= three && one <= six ? 1 : (three <= six ? 3 : 6);
 }
+// a sub-sweep's link: staple 1296 and 108 of products, about 500 for V, the rotations
+// and the reunitarisation; by columns about 300 of those, half the rotations' in six lanes
+inline int update_lanes(long n) { return lanes_per_link(n, 1900, 740, 450); }
+// the force's link: staple and product
+inline int force_lanes(long n) { return lanes_per_link(n, 1420, 490, 275); }
 
 }  // namespace mgq

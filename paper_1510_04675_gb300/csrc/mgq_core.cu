@@ -368,6 +368,23 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 2) k_plaquette(Links
     if (threadIdx.x == 0) partials[blockIdx.x] = acc;
 }
 
+// FP64: one thread per site and plane (block row y).  A plaquette is two products
+// of 108 FP64 operations, so a thread per site is a chain of six of them and a
+// small lattice fills few sub-partitions (8^3x12: 99 us with a thread per site, 20 us
+// with this).
+__global__ void __launch_bounds__(128) k_plaquette_planes(Links<double, 9> U, Geom g, double* __restrict__ partials) {
+    const int p = blockIdx.y, mu = p < 3 ? 0 : (p < 5 ? 1 : 2), nu = p < 3 ? p + 1 : (p < 5 ? p - 1 : 3);
+    double acc = 0.0;
+    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < g.V; idx += gridDim.x * blockDim.x) {
+        const int par = idx >= g.Vh, h = idx - par * g.Vh;
+        int x[4];
+        cb_coords(g, par, h, x);
+        acc += loop_retr(U, make_hops(g, x), par, par ^ 1, mu, nu);
+    }
+    acc = block_sum(acc);
+    if (threadIdx.x == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = acc;
+}
+
 // =============================================================== unitarity
 template <class T, int NP>
 __global__ void k_unitarity(Links<T, NP> U, Geom g, double* __restrict__ partials) {
@@ -422,7 +439,7 @@ static int g_block[MGQ_NKERNELS][3] = {{128, 128, 128}, {128, 128, 128}, {128, 1
 
 int block_size(int kernel, int prec) { return g_block[kernel][prec]; }
 
-// FP64 sub-sweeps of too few links for one thread each (lanes_per_link), with
+// FP64 sub-sweeps of too few links for one thread each (update_lanes), with
 // `lanes` lanes per link; returns the number of blocks
 template <bool HB>
 static int launch_columns(int lanes, mgq_lattice* lat, const Geom& g, int mu, int par, double beta, const RngKey& rk,
@@ -439,7 +456,7 @@ mgq_status heatbath_subsweep(mgq_lattice* lat, double beta, uint64_t sweep, int 
     const Geom g = make_geom(lat->dims);
     const int bs = g_block[MGQ_KERNEL_HEATBATH][lat->prec];
     const RngKey rk = make_rng(lat->seed, lat->lattice_id, sweep);
-    if (const int lanes = lat->prec == MGQ_F64 ? lanes_per_link(g.Vh) : 1; lanes > 1) {
+    if (const int lanes = lat->prec == MGQ_F64 ? update_lanes(g.Vh) : 1; lanes > 1) {
         launch_columns<true>(lanes, lat, g, mu, par, beta, rk, n_hb, dec, nullptr, st);
         return cuda_check("mgq_heatbath");
     }
@@ -467,7 +484,7 @@ mgq_status overrelax_subsweep(mgq_lattice* lat, int mu, int par, cudaStream_t st
     Trace trace("overrelax_subsweep");
     const Geom g = make_geom(lat->dims);
     const int bs = g_block[MGQ_KERNEL_OVERRELAX][lat->prec];
-    if (const int lanes = lat->prec == MGQ_F64 ? lanes_per_link(g.Vh) : 1; lanes > 1) {
+    if (const int lanes = lat->prec == MGQ_F64 ? update_lanes(g.Vh) : 1; lanes > 1) {
         launch_columns<false>(lanes, lat, g, mu, par, 0.0, RngKey{}, 0, nullptr, nullptr, st);
         return cuda_check("mgq_overrelax");
     }
@@ -495,7 +512,7 @@ mgq_status overrelax_sweep_plaquette(mgq_lattice* lat, double* dev_out, cudaStre
     const bool staged = lat->prec == MGQ_F32_C12 && g.Vh >= STAGED_MIN_VH;
     const int bs = staged ? STAGED_THREADS : g_block[MGQ_KERNEL_OVERRELAX][lat->prec];
     double* partials = reinterpret_cast<double*>(ws_alg(lat));  // free during sweeps; >= 2 nb doubles
-    if (const int lanes = lat->prec == MGQ_F64 ? lanes_per_link(g.Vh) : 1; lanes > 1) {
+    if (const int lanes = lat->prec == MGQ_F64 ? update_lanes(g.Vh) : 1; lanes > 1) {
         int n = 0;
         for (int par = 0; par < 2; par++)
             n += launch_columns<false>(lanes, lat, g, 3, par, 0.0, RngKey{}, 0, nullptr, partials + n, st);
@@ -519,10 +536,10 @@ mgq_status overrelax_sweep_plaquette(mgq_lattice* lat, double* dev_out, cudaStre
 // plaquette of `links` into dev_out[0] (device)
 mgq_status plaquette_into(const mgq_lattice* lat, double* partials, double* dev_out, cudaStream_t st) {
     const Geom g = make_geom(lat->dims);
-    const int nb = reduction_blocks(g.V, 256);
-    dispatch_prec(lat->prec, [&]<class T, int NP>() {
-        k_plaquette<T, NP><<<nb, 256, 0, st>>>(links_of<T, NP>(lat), g, partials);
-    });
+    const int nb = lat->prec == MGQ_F64 ? 6 * reduction_blocks(g.V, 128) : reduction_blocks(g.V, 256);  // at most 7104
+    if (lat->prec == MGQ_F64) k_plaquette_planes<<<dim3(nb / 6, 6), 128, 0, st>>>(links_of<double, 9>(lat), g, partials);
+    else if (lat->prec == MGQ_F32) k_plaquette<float, 9><<<nb, 256, 0, st>>>(links_of<float, 9>(lat), g, partials);
+    else k_plaquette<float, 6><<<nb, 256, 0, st>>>(links_of<float, 6>(lat), g, partials);
     launch_final_sum(partials, nb, 1.0 / (18.0 * (double)g.V), dev_out, st);
     return cuda_check("mgq_plaquette");
 }

@@ -304,9 +304,9 @@ template <> __device__ __forceinline__ void rebuild_row2<float>(M3<float>& u) {
     }
 }
 
-// 1/sqrt(n): the correctly rounded quotient in FP64 (the oracle's operations),
-// the hardware reciprocal square root in FP32.
-__device__ __forceinline__ double inv_norm(double n) { return 1.0 / sqrt(n); }
+// 1/sqrt(n): CUDA's reciprocal square roots (FP64: within 1 ulp, as 1.0 / sqrt(n) is,
+// in less than half the operations).
+__device__ __forceinline__ double inv_norm(double n) { return rsqrt(n); }
 __device__ __forceinline__ float inv_norm(float n) { return rsqrtf(n); }
 
 // Gram-Schmidt reunitarisation: normalise row 0, orthogonalise and
@@ -709,22 +709,31 @@ __device__ __noinline__ void exp_coeffs_trig(T c0, T c1, Cx<T>& f0, Cx<T>& f1, C
     }
 }
 
-// The same coefficients by the exponential's own series, N terms, in Horner form:
-// E <- 1 + (i Q / k) E for k = N .. 1 with E = f0 + f1 Q + f2 Q^2 and
-// Q^3 = c1 Q + c0.  The eigenvalues of Q are at most rho = sqrt(4 c1 / 3), the
-// remainder below rho^(N+1) / (N+1)!.
+// The same coefficients by the exponential's own series up to Q^N, with the powers
+// reduced by Q^3 = c1 Q + c0: Q^n = p + q Q + r Q^2 with real p, q, r, and
+// Q^(n+1) = c0 r + (p + c1 r) Q + q Q^2.  The eigenvalues of Q are at most
+// rho = sqrt(4 c1 / 3), the remainder below rho^(N+1) / (N+1)!.
 template <int N, class T>
 __device__ __forceinline__ void exp_coeffs_series(T c0, T c1, Cx<T>& f0, Cx<T>& f1, Cx<T>& f2) {
     f0 = mk(T(1), T(0));
-    f1 = mk(T(0), T(0));
-    f2 = mk(T(0), T(0));
+    f1 = mk(T(0), T(1));
+    f2 = mk(T(-0.5), T(0));
+    T p = T(0), q = T(0), r = T(1);
+    double fact = 2.0;
 #pragma unroll
-    for (int k = N; k >= 1; k--) {
-        const T r = T(1) / T(k);
-        const Cx<T> t = mk(r * (f0.re + c1 * f2.re), r * (f0.im + c1 * f2.im));
-        f0 = mk(T(1) - r * c0 * f2.im, r * c0 * f2.re);
-        f2 = mk(-r * f1.im, r * f1.re);
-        f1 = mk(-t.im, t.re);
+    for (int n = 3; n <= N; n++) {
+        const T p1 = c0 * r, q1 = p + c1 * r, r1 = q;
+        p = p1;
+        q = q1;
+        r = r1;
+        fact *= n;
+        const T c = T(((n & 3) < 2 ? 1.0 : -1.0) / fact);  // i^n / n! without its factor i for odd n
+        T& a0 = (n & 1) ? f0.im : f0.re;
+        T& a1 = (n & 1) ? f1.im : f1.re;
+        T& a2 = (n & 1) ? f2.im : f2.re;
+        a0 += c * p;
+        a1 += c * q;
+        a2 += c * r;
     }
 }
 

@@ -5,6 +5,7 @@
 // with the Wilson flow (its generator is the force at beta = 6).
 #include "mgq_internal.h"
 #include "mgq_stencil.cuh"
+#include "mgq_columns.cuh"
 
 namespace mgq {
 
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(STAGED_THREADS, 5) k_force_staged(Links<float,
 // per link, block row y of the grid holding the links of one (mu, parity).
 template <class T, int NP>
 __global__ void __launch_bounds__(128) k_exp_update(Links<T, NP> U, Geom g, Alg<T> B, T s) {
-    pdl_launch_dependents();
+    if constexpr (sizeof(T) == 4) pdl_launch_dependents();  // FP64: at the end, see k_update_columns
     const int mu = blockIdx.y >> 1, par = blockIdx.y & 1, h = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();
     if (h >= g.Vh) return;
@@ -194,6 +195,7 @@ __global__ void __launch_bounds__(128) k_exp_update(Links<T, NP> U, Geom g, Alg<
     for (int a = 0; a < 8; a++) c[a] *= s;
     M3<T> u = mul_nn(exp_alg(c), u0);
     if (sizeof(T) == 4) reunitarize(u);
+    else pdl_launch_dependents();
     U.store(mu, par, h, u);
 }
 
@@ -274,6 +276,12 @@ static inline int nblk(long n, int t) { return (int)((n + t - 1) / t); }
 // B <- alpha B + coef TA-coefficients, on `links` with the lattice's format
 mgq_status force_accumulate(const mgq_lattice* lat, void* B, double coef, double alpha, cudaStream_t st) {
     const Geom g = make_geom(lat->dims);
+    if (const int lanes = lat->prec == MGQ_F64 ? force_lanes(8L * g.Vh) : 1; lanes > 1) {
+        const int per = lanes == 3 ? ColumnLane<3>::kPerBlock : ColumnLane<6>::kPerBlock;
+        launch_pdl(lanes == 3 ? k_force_columns<3> : k_force_columns<6>, dim3(nblk(g.Vh, per), 8), COL_THREADS, st,
+                   links_of<double, 9>(lat), g, alg_at<double>(B, lat->dims), coef, alpha);
+        return cuda_check("force");
+    }
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
         if constexpr (sizeof(T) == 4 && NP == 6)
             launch_pdl_smem(k_force_staged, 2 * nblk(g.Vh, 32), STAGED_THREADS, STAGED_SMEM, st, links_of<T, NP>(lat), g,

@@ -514,7 +514,7 @@ __device__ __forceinline__ float creutz_a0(float k, float em, float u0) {
     const float y = (1.f - u0) * em;
     return 1.f + (y < -0.1f ? __logf(1.f + y) : log1pf(y)) * __frcp_rn(k);
 }
-__device__ __forceinline__ double creutz_k(double beta, double xi) { return 2.0 * beta * xi / 3.0; }
+__device__ __forceinline__ double creutz_k(double beta, double xi) { return xi * (beta * (2.0 / 3.0)); }
 __device__ __forceinline__ float creutz_k(float beta, float xi) { return xi * (beta * 0.666666667f); }
 __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }

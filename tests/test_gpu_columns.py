@@ -26,3 +26,23 @@ def test_columns_equal_one_thread_per_link(gpu, dims, n_hb):
     # sums of at most 6 V terms of O(1), each to 2^-53 relative
     assert abs(rec.cpu().numpy()[:, 0] - plaq).max() < 1e-14
     assert abs(gpu.mgq_plaquette(a) - plaq[-1]) < 1e-13
+
+
+@pytest.mark.parametrize("dims", [[2, 2, 2, 2], [4, 2, 6, 8], [6, 6, 6, 6], [8, 8, 8, 12], [12, 12, 12, 14]])
+def test_force_and_plaquette_by_columns(gpu, orc, dims):
+    """Force (written and accumulated) and plaquette around the limits of the lane counts, against the oracle."""
+    import numpy as np
+
+    U = orc.init_links(dims, 1, seed=5)
+    orc.update_chain(U, dims, 5.8, 5, 0, 0, 1, 1, 1)
+    lat = gpu.Lattice(dims, "f64", with_mom=True)
+    lat.from_numpy(U)
+    ref = orc.force(U, dims, 6.0)
+    F = lat.new_alg_field()
+    gpu.mgq_hmc_force(lat, 6.0, F)
+    assert np.max(np.abs(gpu.alg_to_numpy(lat, F) - ref)) < 1e-13
+    P = np.random.default_rng(3).standard_normal(ref.shape)
+    lat.mom.view(torch.float64).copy_(gpu.alg_from_numpy(lat, P))
+    gpu.mgq_hmc_momentum_step(lat, 6.0, 0.25)
+    assert np.max(np.abs(lat.mom_numpy() - (P + 0.25 * ref))) < 1e-13
+    assert abs(gpu.mgq_plaquette(lat) - orc.plaquette(U, dims)) < 1e-14
