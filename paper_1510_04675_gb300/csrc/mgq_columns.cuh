@@ -22,6 +22,7 @@
 // hb_link, or_link), so both agree bit for bit.
 #pragma once
 
+#include "mgq_force_out.cuh"
 #include "mgq_stencil.cuh"
 
 namespace mgq {
@@ -219,16 +220,16 @@ __global__ void __launch_bounds__(COL_THREADS) k_update_columns(Links<double, 9>
     }
 }
 
-// B <- alpha B + coef t(TA(U A)) on every link (as k_force), block row y the (mu,
-// parity) plane.  With M = U A by columns, lane k holds M_nk of the pair (k, n),
+// The force of every link (as k_force), block row y the (mu, parity) plane.  With M = U A by columns, lane k holds M_nk of the pair (k, n),
 // n = k + 1 mod 3, and gets M_kn: two coefficients each, the diagonal ones by all.
-template <int LPL>
-__global__ void __launch_bounds__(COL_THREADS) k_force_columns(Links<double, 9> U, Geom g, Alg<double> B, double coef, double alpha) {
+template <int LPL, class Out>
+__global__ void __launch_bounds__(COL_THREADS) k_force_columns(Links<double, 9> U, Geom g, Out out) {
     const ColumnLane<LPL> c;
     const int mu = blockIdx.y >> 1, par = blockIdx.y & 1, h0 = c.item(), h = h0 < g.Vh ? h0 : g.Vh - 1;
     int x[4];
     cb_coords(g, par, h, x);
     pdl_wait();
+    if (out.idle()) return;
     Cx<double> A[3], u[3], v[3];
     staple_column<LPL>(U, g, x, h, mu, par, c, A);
     left_column(U.base(mu, par, h), A, c.k, u, v);
@@ -244,15 +245,10 @@ __global__ void __launch_bounds__(COL_THREADS) k_force_columns(Links<double, 9> 
     if (!c.active || h0 >= g.Vh || c.half) return;
     const double re = c.k == 2 ? has.re - got.re : got.re - has.re;  // t_1, t_6, t_4 = Re(M_ij - M_ji), i < j
     const double diag = c.k == 0 ? d0 - d1 : (d0 + d1 - 2.0 * d2) * 0.57735026918962576451;
-    double* b = B.at(mu, par, h);
-    auto put = [&](int a, double t) {
-        double& o = b[a * Alg<double>::kStep];
-        o = alpha == 0.0 ? coef * t : alpha * o + coef * t;
-    };
     const int a = c.k == 0 ? 0 : (c.k == 1 ? 5 : 3);  // pairs 01, 12, 02
-    put(a, has.im + got.im);
-    put(a + 1, re);
-    if (c.k < 2) put(c.k == 0 ? 2 : 7, diag);
+    out.put_one(mu, par, h, a, has.im + got.im);
+    out.put_one(mu, par, h, a + 1, re);
+    if (c.k < 2) out.put_one(mu, par, h, c.k == 0 ? 2 : 7, diag);
 }
 
 // Lanes per link (1: a thread for each; 3; 6) of a launch over n links, from the

@@ -5,9 +5,6 @@
 
 namespace mgq {
 
-mgq_status force_accumulate(const mgq_lattice* lat, void* B, double coef, double alpha, cudaStream_t st);
-mgq_status exp_update(const mgq_lattice* lat, void* B, double s, cudaStream_t st);
-
 // Per site: E(x) = -1/2 sum_{mu,nu} Tr G^2 = 1/2 sum_{mu<nu} |g_munu|^2 and
 // q(x) = -1/(32 pi^2) eps Tr(G G) = 1/(8 pi^2) (g01.g23 - g02.g13 + g03.g12),
 // using Tr(X_a X_b) = -delta_ab / 2, with G from the leaves of the line field A of

@@ -18,18 +18,6 @@
 
 namespace mgq {
 
-struct FlowCtl {
-    double t, eps, h, t_next;
-    unsigned long long dbits;  // max error estimate: bits of a non-negative double
-    int active;                // the current trial runs
-    int hits;                  // the trial lands on the next measurement time
-    int restore;               // the trial was rejected: links <- backup
-    int meas;                  // measure E, Q now
-    int m, steps, rejects;
-    int status;                // 0 running, 1 finished, 2 step size underflow
-};
-static_assert(sizeof(FlowCtl) <= 16 * sizeof(double), "control block must fit 16 scalar slots");
-
 __global__ void k_adapt_init(FlowCtl* c, double eps0) {
     c->t = 0.0;
     c->eps = eps0;
@@ -46,9 +34,9 @@ __global__ void k_adapt_init(FlowCtl* c, double eps0) {
     c->status = 0;
 }
 
-__global__ void k_adapt_begin(FlowCtl* c, double t_end, double eps_max, double dt_meas, int max_meas) {
-    pdl_launch_dependents();
-    pdl_wait();
+// Sets up the next trial: its size, capped by the maximal step and the next
+// measurement time, or the end of the flow.
+__device__ __forceinline__ void adapt_begin(FlowCtl* c, double t_end, double eps_max, double dt_meas, int max_meas) {
     c->active = 0;
     c->restore = 0;
     c->meas = 0;
@@ -92,102 +80,56 @@ __global__ void k_adapt_end(FlowCtl* c, double tol, double eps_max) {
     }
 }
 
-// Stage generator z = -h TA(W A(W)) coefficients, then
-//   B <- aB B + cB z   (aB == 0: write only)
-//   Y <- aY Y + cY z   (cY == 0: Y untouched; aY == 0: write only)
-// Same 8-warp plane layout as the HMC force kernel: a block covers 32 sites in
-// all eight (mu, parity) planes.
-template <class T, int NP>
-__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 2)
-    k_flow_stage(Links<T, NP> U, Geom g, Alg<T> B, Alg<T> Y, const FlowCtl* c, T cB, T aB, T cY, T aY) {
+// W <- exp(s B) W, block row y the (mu, parity) plane.  SAVE: the old W goes to
+// `start` first (the start of the trial, restored on rejection).  ERROR (the
+// trial's last stage): also d = max over links of |W3 - exp(Y) W0|_F / 3, Y = 2 Z1 -
+// Z0, with W3 at hand and W0 from `start`.
+template <class T, int NP, bool SAVE, bool ERROR>
+__global__ void __launch_bounds__(128) k_flow_exp(Links<T, NP> U, Geom g, Alg<T> B, T s, FlowCtl* c, Links<T, NP> start,
+                                                  Alg<T> Y) {
     pdl_launch_dependents();
+    const int mu = blockIdx.y >> 1, par = blockIdx.y & 1, h = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();
     if (!c->active) return;
-    const int w = threadIdx.x >> 5;
-    const int mu = w >> 1, par = w & 1;
-    const int h = blockIdx.x * 32 + (threadIdx.x & 31);
-    if (h >= g.Vh) return;
-    int x[4];
-    cb_coords(g, par, h, x);
-    const M3<T> A = staple(U, g, x, h, mu, par);
-    T t[8];
-    ta_coeffs(mul_nn(U.load(mu, par, h), A), t);
-    const T mh = (T)(-c->h);
-    T* b = B.at(mu, par, h);
+    double d = 0.0;
+    if (h < g.Vh) {
+        T q[8];
+        B.load(mu, par, h, q);
+        const M3<T> u0 = U.load(mu, par, h);
 #pragma unroll
-    for (int a = 0; a < 8; a++) {
-        const T z = mh * t[a];
-        b[a * Alg<T>::kStep] = aB == T(0) ? cB * z : aB * b[a * Alg<T>::kStep] + cB * z;
-    }
-    if (cY != T(0)) {
-        T* y = Y.at(mu, par, h);
+        for (int a = 0; a < 8; a++) q[a] *= s;
+        if (SAVE) start.store(mu, par, h, u0);
+        M3<T> u = mul_nn(exp_alg(q), u0);
+        if (sizeof(T) == 4) reunitarize(u);
+        U.store(mu, par, h, u);
+        if constexpr (ERROR) {
+            Y.load(mu, par, h, q);
+            const M3<T> w2 = mul_nn(exp_alg(q), start.load(mu, par, h));
+            // in the link precision: an FP32 estimate steers the step as well as
+            // an FP64 one, and FP64 arithmetic is slow on this part
+            T s2 = T(0);
 #pragma unroll
-        for (int a = 0; a < 8; a++) {
-            const T z = mh * t[a];
-            y[a * Alg<T>::kStep] = aY == T(0) ? cY * z : aY * y[a * Alg<T>::kStep] + cY * z;
+            for (int i = 0; i < 3; i++)
+#pragma unroll
+                for (int j = 0; j < 3; j++) {
+                    const T dr = u.e[i][j].re - w2.e[i][j].re;
+                    const T di = u.e[i][j].im - w2.e[i][j].im;
+                    s2 += dr * dr + di * di;
+                }
+            d = (double)(m_sqrt(s2) / T(3));
         }
     }
-}
-
-// W <- exp(s B) W; with backup, the old W is saved there first (the start
-// of the trial, restored on rejection).
-template <class T, int NP>
-__global__ void __launch_bounds__(128) k_flow_exp(Links<T, NP> U, Geom g, Alg<T> B, T s, const FlowCtl* c,
-                                                  Links<T, NP> backup, int save) {
-    pdl_launch_dependents();
-    pdl_wait();
-    if (!c->active) return;
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 8 * g.Vh) return;
-    const int mp = idx / g.Vh, h = idx - mp * g.Vh, mu = mp >> 1, par = mp & 1;
-    T q[8];
-    B.load(mu, par, h, q);
+    if constexpr (ERROR) {
+        // Non-negative doubles order like their bit patterns, and a NaN compares
+        // above every number, so a broken step is rejected.
+        unsigned long long bits = (unsigned long long)__double_as_longlong(d);
 #pragma unroll
-    for (int a = 0; a < 8; a++) q[a] *= s;
-    const M3<T> u0 = U.load(mu, par, h);
-    if (save) backup.store(mu, par, h, u0);
-    M3<T> u = mul_nn(exp_alg(q), u0);
-    if (sizeof(T) == 4) reunitarize(u);
-    U.store(mu, par, h, u);
-}
-
-// d = max over links of |W3 - exp(Y) W0|_F / 3, Y = 2 Z1 - Z0.
-template <class T, int NP>
-__global__ void __launch_bounds__(128) k_flow_error(Links<T, NP> U, Links<T, NP> U0, Geom g, Alg<T> Y,
-                                                    FlowCtl* c) {
-    pdl_launch_dependents();
-    pdl_wait();
-    if (!c->active) return;
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    double d = 0.0;
-    if (idx < 8 * g.Vh) {
-        const int mp = idx / g.Vh, h = idx - mp * g.Vh, mu = mp >> 1, par = mp & 1;
-        T y[8];
-        Y.load(mu, par, h, y);
-        const M3<T> w2 = mul_nn(exp_alg(y), U0.load(mu, par, h));
-        const M3<T> w3 = U.load(mu, par, h);
-        // in the link precision: an FP32 estimate steers the step as well as
-        // an FP64 one, and FP64 arithmetic is slow on this part
-        T s2 = T(0);
-#pragma unroll
-        for (int i = 0; i < 3; i++)
-#pragma unroll
-            for (int j = 0; j < 3; j++) {
-                const T dr = w3.e[i][j].re - w2.e[i][j].re;
-                const T di = w3.e[i][j].im - w2.e[i][j].im;
-                s2 += dr * dr + di * di;
-            }
-        d = (double)(m_sqrt(s2) / T(3));
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long other = __shfl_down_sync(0xffffffffu, bits, o);
+            bits = other > bits ? other : bits;
+        }
+        if ((threadIdx.x & 31) == 0 && bits) atomicMax(&c->dbits, bits);
     }
-    // Non-negative doubles order like their bit patterns, and a NaN compares
-    // above every number, so a broken step is rejected.
-    unsigned long long bits = (unsigned long long)__double_as_longlong(d);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long other = __shfl_down_sync(0xffffffffu, bits, o);
-        bits = other > bits ? other : bits;
-    }
-    if ((threadIdx.x & 31) == 0 && bits) atomicMax(&c->dbits, bits);
 }
 
 __global__ void k_flow_restore(uint4* links, const uint4* backup, size_t nwords,
@@ -199,24 +141,29 @@ __global__ void k_flow_restore(uint4* links, const uint4* backup, size_t nwords,
         links[i] = backup[i];
 }
 
-// meas[2m] = E (site average), meas[2m+1] = Q from the clover partials; m++.
-__global__ void k_adapt_meas(FlowCtl* c, const double* partials, int nb, double invV, double* meas) {
+// After a trial (and before the first): the measurement it asked for, meas[2m] = E
+// (site average), meas[2m+1] = Q from the clover partials, m++; then the next trial
+// is set up.
+__global__ void k_adapt_next(FlowCtl* c, const double* partials, int nb, double invV, double* meas, double t_end, double eps_max,
+                             double dt_meas, int max_meas) {
     pdl_launch_dependents();
     pdl_wait();
-    if (!c->meas) return;
-    double e = 0.0, q = 0.0;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-        e += partials[i];
-        q += partials[nb + i];
+    if (c->meas) {
+        double e = 0.0, q = 0.0;
+        for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+            e += partials[i];
+            q += partials[nb + i];
+        }
+        e = block_sum(e);
+        q = block_sum(q);
+        if (threadIdx.x == 0) {
+            meas[2 * c->m] = e * invV;
+            meas[2 * c->m + 1] = q;
+            c->m++;
+        }
     }
-    e = block_sum(e);
-    q = block_sum(q);
-    if (threadIdx.x == 0) {
-        meas[2 * c->m] = e * invV;
-        meas[2 * c->m + 1] = q;
-        c->m++;
-        c->meas = 0;
-    }
+    __syncthreads();
+    if (threadIdx.x == 0) adapt_begin(c, t_end, eps_max, dt_meas, max_meas);
 }
 
 static inline int nblk(long n, int t) { return (int)((n + t - 1) / t); }
@@ -270,35 +217,33 @@ mgq_status mgq_wilson_flow_adaptive(mgq_lattice* lat, double t_end, double tol, 
     void* backup = ws_links(lat);
     const size_t nwords = links_bytes(lat) / 16;
 
-    auto measure = [&]() {
+    auto next = [&]() {
         const int nb = clover_partials(lat, lat->links, 1, partials, &c->meas, st);
-        launch_pdl(k_adapt_meas, 1, 512, st, c, partials, nb, invV, meas);
+        launch_pdl(k_adapt_next, 1, 512, st, c, partials, nb, invV, meas, t_end, eps_max, dt_meas, nm);
     };
     auto trial = [&]() {
-        launch_pdl(k_adapt_begin, 1, 1, st, c, t_end, eps_max, dt_meas, nm);
         dispatch_prec(lat->prec, [&]<class T, int NP>() {
             const Links<T, NP> U = links_of<T, NP>(lat), U0 = links_at<T, NP>(backup, lat->dims);
             const Alg<T> B = alg_at<T>(Bp, lat->dims), Y = alg_at<T>(scratch, lat->dims);
-            const int fb = nblk(g.Vh, 32), eb = nblk(8L * g.Vh, 128);
+            const dim3 eb(nblk(g.Vh, 128), 8);
             // Z0: B = Z0, Y = -Z0
-            launch_pdl(k_flow_stage<T, NP>, fb, 256, st, U, g, B, Y, c, T(1), T(0), T(-1), T(0));
-            launch_pdl(k_flow_exp<T, NP>, eb, 128, st, U, g, B, T(0.25), c, U0, 1);
+            flow_stage(lat, Bp, 1.0, 0.0, scratch, -1.0, 0.0, c, st);
+            launch_pdl(k_flow_exp<T, NP, true, false>, eb, 128, st, U, g, B, T(0.25), c, U0, Y);
             // Z1: B = 8/9 Z1 - 17/36 B, Y = 2 Z1 + Y
-            launch_pdl(k_flow_stage<T, NP>, fb, 256, st, U, g, B, Y, c, T(8.0 / 9.0), T(-17.0 / 36.0), T(2), T(1));
-            launch_pdl(k_flow_exp<T, NP>, eb, 128, st, U, g, B, T(1), c, U0, 0);
+            flow_stage(lat, Bp, 8.0 / 9.0, -17.0 / 36.0, scratch, 2.0, 1.0, c, st);
+            launch_pdl(k_flow_exp<T, NP, false, false>, eb, 128, st, U, g, B, T(1), c, U0, Y);
             // Z2: B = 3/4 Z2 - B
-            launch_pdl(k_flow_stage<T, NP>, fb, 256, st, U, g, B, Y, c, T(0.75), T(-1), T(0), T(0));
-            launch_pdl(k_flow_exp<T, NP>, eb, 128, st, U, g, B, T(1), c, U0, 0);
-            launch_pdl(k_flow_error<T, NP>, eb, 128, st, U, U0, g, Y, c);
+            flow_stage(lat, Bp, 0.75, -1.0, scratch, 0.0, 0.0, c, st);
+            launch_pdl(k_flow_exp<T, NP, false, true>, eb, 128, st, U, g, B, T(1), c, U0, Y);
         });
         launch_pdl(k_adapt_end, 1, 1, st, c, tol, eps_max);
         launch_pdl(k_flow_restore, 1184, 256, st, reinterpret_cast<uint4*>(lat->links),
                    reinterpret_cast<const uint4*>(backup), nwords, (const FlowCtl*)c);
-        measure();
+        next();
     };
 
     k_adapt_init<<<1, 1, 0, st>>>(c, eps0);
-    measure();
+    next();
     if ((s = cuda_check("mgq_wilson_flow_adaptive"))) return s;
     // Trials run in chunks between reads of the status word; a chunk that
     // finishes early leaves its remaining trials as gated no-op launches.

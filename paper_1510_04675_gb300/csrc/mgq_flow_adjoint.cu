@@ -21,9 +21,6 @@
 
 namespace mgq {
 
-mgq_status force_accumulate(const mgq_lattice* lat, void* B, double coef, double alpha, cudaStream_t st);
-mgq_status exp_update(const mgq_lattice* lat, void* B, double s, cudaStream_t st);
-
 // [a, b] for antihermitian a, b: b a = (a b)^+, so [a, b] = a b - (a b)^+ from
 // one product; the result is antihermitian entry by entry (r_ji = -conj(r_ij)
 // exactly, the diagonal purely imaginary).

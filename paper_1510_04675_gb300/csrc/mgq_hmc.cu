@@ -5,17 +5,17 @@
 // with the Wilson flow (its generator is the force at beta = 6).
 #include "mgq_internal.h"
 #include "mgq_stencil.cuh"
+#include "mgq_force_out.cuh"
 #include "mgq_columns.cuh"
 
 namespace mgq {
 
-// B <- alpha B + coef t(TA(U A)), t the algebra coefficients of TA(U A);
-// alpha == 0 writes without reading B.  A block of 8 warps covers 32
-// consecutive sites in all eight (mu, parity) planes (warp w: mu = w/2,
-// parity = w%2), so the neighbour links of a site band are used by all
-// directions while they are still in cache.
-template <class T, int NP>
-__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 2) k_force(Links<T, NP> U, Geom g, Alg<T> B, T coef, T alpha) {
+// FP64 force, one thread per link.  A block of 8 warps covers 32 consecutive sites
+// in all eight (mu, parity) planes (warp w: mu = w/2, parity = w%2), so the
+// neighbour links of a site band are used by all directions while they are still
+// in cache.
+template <class Out>
+__global__ void __launch_bounds__(256, 1) k_force(Links<double, 9> U, Geom g, Out out) {
     pdl_launch_dependents();
     const int w = threadIdx.x >> 5;
     const int mu = w >> 1, par = w & 1;
@@ -23,19 +23,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 2) k_force(Links<T, 
     int x[4];
     cb_coords(g, par, h, x);
     pdl_wait();
-    if (h >= g.Vh) return;
-    const M3<T> A = staple(U, g, x, h, mu, par);
-    const M3<T> M = mul_nn(U.load(mu, par, h), A);
-    T t[8];
-    ta_coeffs(M, t);
-    T* b = B.at(mu, par, h);
-    if (alpha == T(0)) {
-#pragma unroll
-        for (int a = 0; a < 8; a++) b[a * Alg<T>::kStep] = coef * t[a];
-    } else {
-#pragma unroll
-        for (int a = 0; a < 8; a++) b[a * Alg<T>::kStep] = alpha * b[a * Alg<T>::kStep] + coef * t[a];
-    }
+    if (h >= g.Vh || out.idle()) return;
+    const M3<double> A = staple(U, g, x, h, mu, par);
+    double t[8];
+    ta_coeffs(mul_nn(U.load(mu, par, h), A), t);
+    out.put(mu, par, h, t);
 }
 
 // FP32 12-real force with the staple's links staged through shared memory (the
@@ -71,8 +63,8 @@ __device__ __forceinline__ void staged_ta_sub(const float4* sm, int col, int j, 
     t[4] -= b.x, t[5] -= b.y, t[6] -= b.z, t[7] -= b.w;
 }
 
-__global__ void __launch_bounds__(STAGED_THREADS, 5) k_force_staged(Links<float, 6> U, Geom g, Alg<float> B, float coef,
-                                                                  float alpha) {
+template <class Out>
+__global__ void __launch_bounds__(STAGED_THREADS, 5) k_force_staged(Links<float, 6> U, Geom g, Out out) {
     extern __shared__ float4 sm[];
     pdl_launch_dependents();
     const int mu = threadIdx.x >> 5, par = blockIdx.x & 1, op = par ^ 1, lane = threadIdx.x & 31;
@@ -100,6 +92,7 @@ __global__ void __launch_bounds__(STAGED_THREADS, 5) k_force_staged(Links<float,
         own_hpn[j] = (H.lex + pick(H.fwd, own_nu[j])) >> 1;
     }
     pdl_wait();
+    if (out.idle()) return;
     // half-term k < 3: dn = (e d)^+ f, d = U_nu(x+mu-nu), e = U_mu(x-nu), f = U_nu(x-nu)
     // for the k-th direction nu != mu; k >= 3: up = (a b^+) c^+ for owned plane
     // j = k - 3, a = U_nu(x+mu), b = U_mu(x+nu), c = U_nu(x) (shared)
@@ -169,15 +162,68 @@ __global__ void __launch_bounds__(STAGED_THREADS, 5) k_force_staged(Links<float,
     // for mu >= 2, nu = mu - 2 (its second)
     staged_ta_sub(sm, ((mu + 3) & 3) * 32 + lane, 0, t);
     if (mu >= 2) staged_ta_sub(sm, (mu - 2) * 32 + lane, 1, t);
-    if (h >= g.Vh) return;
-    float* b = B.at(mu, par, h);
-    if (alpha == 0.f) {
+    if (h < g.Vh) out.put(mu, par, h, t);
+}
+
+// FP32 18-real force, with the plaquettes shared in the same way and the links read
+// straight into registers (32^4: 260 us, where one thread per link with its own six
+// upper and lower terms took 279 us; eight warps for both parities of a band take
+// 279 us too, and copies of single 8-byte planes staged as above do not pay).
+template <class Out>
+__global__ void __launch_bounds__(128, 4) k_force_shared(Links<float, 9> U, Geom g, Out out) {
+    __shared__ float2 own[4][9][32];    // U_mu(x)
+    __shared__ float ta[4][2][8][32];   // TA coefficients of the owned plaquettes
+    pdl_launch_dependents();
+    const int mu = threadIdx.x >> 5, par = blockIdx.x & 1, op = par ^ 1, lane = threadIdx.x & 31;
+    const int h = (blockIdx.x >> 1) * 32 + lane;
+    const int hc = h < g.Vh ? h : g.Vh - 1;  // lanes past the end compute a copy and store nothing
+    int x[4];
+    cb_coords(g, par, hc, x);
+    const Hops H = make_hops(g, x);
+    const int fmu = pick(H.fwd, mu), hpm = (H.lex + fmu) >> 1;
+    pdl_wait();
+    if (out.idle()) return;
+    M3<float> A;
 #pragma unroll
-        for (int a = 0; a < 8; a++) b[a * Alg<float>::kStep] = coef * t[a];
-    } else {
+    for (int i = 0; i < 3; i++)
 #pragma unroll
-        for (int a = 0; a < 8; a++) b[a * Alg<float>::kStep] = alpha * b[a * Alg<float>::kStep] + coef * t[a];
+        for (int j = 0; j < 3; j++) A.e[i][j] = mk(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const int nu = k < mu ? k : k + 1, b = pick(H.bwd, nu), hmn = (H.lex + b) >> 1;
+        acc_add(A, down_term(U.load_rows(mu, op, hmn), U.load(nu, par, (H.lex + fmu + b) >> 1), U.load(nu, op, hmn)));
     }
+    const M3<float> u = U.load(mu, par, hc);
+#pragma unroll
+    for (int e = 0; e < 9; e++) own[mu][e][lane] = make_float2(u.e[e / 3][e % 3].re, u.e[e / 3][e % 3].im);
+    float t[8];
+    ta_coeffs(mul_nn(u, A), t);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+        if (j == 1 && mu >= 2) break;  // owned planes: nu = mu + 1, and mu + 2 for mu < 2 (mod 4)
+        const int nu = (mu + 1 + j) & 3;
+        M3<float> c;
+#pragma unroll
+        for (int e = 0; e < 9; e++) c.e[e / 3][e % 3] = from_f2(own[nu][e][lane]);
+        const M3<float> up = up_term(U.load_rows(nu, op, hpm), U.load(mu, op, (H.lex + pick(H.fwd, nu)) >> 1), c);
+        M3<float> P = mul_nn_2(u, up);
+        rebuild_row2(P);
+        float tp[8];
+        ta_coeffs(P, tp);
+#pragma unroll
+        for (int a = 0; a < 8; a++) {
+            t[a] += tp[a];
+            ta[mu][j][a][lane] = tp[a];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < 8; a++) {
+        t[a] -= ta[(mu + 3) & 3][0][a][lane];
+        if (mu >= 2) t[a] -= ta[mu - 2][1][a][lane];
+    }
+    if (h < g.Vh) out.put(mu, par, h, t);
 }
 
 // U <- exp(s B) U on every link; the FP32 formats are reunitarised.  One thread
@@ -273,24 +319,43 @@ __global__ void k_restore(uint4* __restrict__ links, const uint4* __restrict__ b
 
 static inline int nblk(long n, int t) { return (int)((n + t - 1) / t); }
 
-// B <- alpha B + coef TA-coefficients, on `links` with the lattice's format
-mgq_status force_accumulate(const mgq_lattice* lat, void* B, double coef, double alpha, cudaStream_t st) {
+// the force kernel of the lattice's format and size, with epilogue `out`
+template <class T, template <class> class Out> static void launch_force(const mgq_lattice* lat, const Out<T>& out, cudaStream_t st) {
     const Geom g = make_geom(lat->dims);
-    if (const int lanes = lat->prec == MGQ_F64 ? force_lanes(8L * g.Vh) : 1; lanes > 1) {
+    if constexpr (sizeof(T) == 8) {
+        const Links<double, 9> U = links_of<double, 9>(lat);
+        const int lanes = force_lanes(8L * g.Vh);
         const int per = lanes == 3 ? ColumnLane<3>::kPerBlock : ColumnLane<6>::kPerBlock;
-        launch_pdl(lanes == 3 ? k_force_columns<3> : k_force_columns<6>, dim3(nblk(g.Vh, per), 8), COL_THREADS, st,
-                   links_of<double, 9>(lat), g, alg_at<double>(B, lat->dims), coef, alpha);
-        return cuda_check("force");
-    }
-    dispatch_prec(lat->prec, [&]<class T, int NP>() {
-        if constexpr (sizeof(T) == 4 && NP == 6)
-            launch_pdl_smem(k_force_staged, 2 * nblk(g.Vh, 32), STAGED_THREADS, STAGED_SMEM, st, links_of<T, NP>(lat), g,
-                            alg_at<T>(B, lat->dims), (T)coef, (T)alpha);
+        if (lanes == 1) launch_pdl(k_force<Out<double>>, nblk(g.Vh, 32), 256, st, U, g, out);
         else
-            launch_pdl(k_force<T, NP>, nblk(g.Vh, 32), 256, st, links_of<T, NP>(lat), g, alg_at<T>(B, lat->dims),
-                       (T)coef, (T)alpha);
+            launch_pdl(lanes == 3 ? k_force_columns<3, Out<double>> : k_force_columns<6, Out<double>>, dim3(nblk(g.Vh, per), 8),
+                       COL_THREADS, st, U, g, out);
+    } else if (lat->prec == MGQ_F32) {
+        launch_pdl(k_force_shared<Out<float>>, 2 * nblk(g.Vh, 32), 128, st, links_of<float, 9>(lat), g, out);
+    } else {
+        launch_pdl_smem(k_force_staged<Out<float>>, 2 * nblk(g.Vh, 32), STAGED_THREADS, STAGED_SMEM, st, links_of<float, 6>(lat), g,
+                        out);
+    }
+}
+
+// calls f.template operator()<T>() for the arithmetic type of a precision
+template <class F> static void dispatch_real(int prec, F&& f) {
+    if (prec == MGQ_F64) f.template operator()<double>();
+    else f.template operator()<float>();
+}
+
+mgq_status force_accumulate(const mgq_lattice* lat, void* B, double coef, double alpha, cudaStream_t st) {
+    dispatch_real(lat->prec, [&]<class T>() {
+        launch_force(lat, ForceOut<T>{alg_at<T>(B, lat->dims), (T)coef, (T)alpha}, st);
     });
     return cuda_check("force");
+}
+
+void flow_stage(const mgq_lattice* lat, void* B, double cB, double aB, void* Y, double cY, double aY, const FlowCtl* ctl,
+                cudaStream_t st) {
+    dispatch_real(lat->prec, [&]<class T>() {
+        launch_force(lat, StageOut<T>{{alg_at<T>(B, lat->dims), (T)cB, (T)aB}, {alg_at<T>(Y, lat->dims), (T)cY, (T)aY}, ctl}, st);
+    });
 }
 
 mgq_status exp_update(const mgq_lattice* lat, void* B, double s, cudaStream_t st) {

@@ -71,6 +71,28 @@ mgq_status plaquette_into(const mgq_lattice* lat, double* partials, double* dev_
 mgq_status heatbath_subsweep(mgq_lattice* lat, double beta, uint64_t sweep, int n_hb, int mu, int par, uint8_t* dec,
                              cudaStream_t st);
 mgq_status overrelax_subsweep(mgq_lattice* lat, int mu, int par, cudaStream_t st);
+// ---- adaptive flow: the device-side control block (mgq_flow_adaptive.cu)
+struct FlowCtl {
+    double t, eps, h, t_next;
+    unsigned long long dbits;  // max error estimate: bits of a non-negative double
+    int active;                // the current trial runs
+    int hits;                  // the trial lands on the next measurement time
+    int restore;               // the trial was rejected: links <- backup
+    int meas;                  // measure E, Q now
+    int m, steps, rejects;
+    int status;                // 0 running, 1 finished, 2 step size underflow
+};
+static_assert(sizeof(FlowCtl) <= 16 * sizeof(double), "control block must fit 16 scalar slots");
+
+// With t the algebra coefficients of TA(U A) at the lattice's links:
+// B <- alpha B + coef t (alpha == 0 writes without reading B)
+mgq_status force_accumulate(const mgq_lattice* lat, void* B, double coef, double alpha, cudaStream_t st);
+// A stage of an adaptive-flow trial, z = -h t with h of the control block: B <- aB B +
+// cB z and, if cY != 0, Y <- aY Y + cY z; nothing when the trial is not active.
+void flow_stage(const mgq_lattice* lat, void* B, double cB, double aB, void* Y, double cY, double aY, const FlowCtl* ctl,
+                cudaStream_t st);
+// U <- exp(s B) U on every link
+mgq_status exp_update(const mgq_lattice* lat, void* B, double s, cudaStream_t st);
 // E (site average) and Q of the clover field strength into dev_out[0], dev_out[1]
 mgq_status clover_into(const mgq_lattice* lat, double* partials, double* dev_out, cudaStream_t st);
 // Per-block E and Q partial sums (E at partials[0..nb), Q at partials[nb..2nb)) of
