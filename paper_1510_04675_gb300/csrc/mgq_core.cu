@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(STAGED_THREADS, 5) k_heatbath_staged(Links<flo
     uint4 r[3];
     const uint32_t lex = (uint32_t)lex_of(g, x);
     // the three Philox draws while the first staged loads are in flight
-    const M3<float> A = staple_staged(U, g, x, h, MU, par, sm, u, [&]() {
+    const M3<float> A = staple_staged<true>(U, g, x, h, MU, par, sm, u, [&]() {
 #pragma unroll
         for (int s = 0; s < 3; s++) r[s] = draw(rk, lex, (uint32_t)MU, (uint32_t)s, 0u, KIND_HB);
     });

@@ -172,10 +172,40 @@ template <> __device__ __forceinline__ M3<double> mul_dd<double>(const M3<double
     return chain_product<true, true>(a, b);
 }
 
-// FP32 products on the packed f32x2 FMA of sm_100+: a complex product is
-// a.re * (b.re, b.im) + a.im * (-b.im, b.re), two paired FMAs instead of four.
+// FP32 products come in two forms with the same operations per entry, in the same
+// order, and so the same bits:
+//   fma_product   single FMAs, re += a.re b.re, im += a.re b.im, re -= a.im b.im,
+//                 im += a.im b.re, signs free;
+//   x2_product    the packed f32x2 FMA of sm_100+: a.re * (b.re, b.im) + a.im *
+//                 (-b.im, b.re), half the issue slots for the arithmetic but as many
+//                 again to build the pairs, and more registers.
+// Which is the faster is the kernel's matter (measured on 32^4, 12-real): the force
+// 249 -> 232 us and the flow's vector-Jacobian product 1263 -> 1104 us with single
+// FMAs; the sub-sweeps, whose issue slots compete with six staged loads a term, 45.5
+// -> 50.3 us, and the prolongation's iterations 21.8 -> 22.9 ms a batch the other way.
 // ROWS = 2 computes rows 0 and 1 of the result only; DA / DB take the
 // conjugate transpose of a / b.
+template <int ROWS, bool DA, bool DB>
+__device__ __forceinline__ M3<float> fma_product(const M3<float>& a, const M3<float>& b) {
+    M3<float> r;
+#pragma unroll
+    for (int i = 0; i < ROWS; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            float re = 0.f, im = 0.f;
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const float are = DA ? a.e[k][i].re : a.e[i][k].re, aim = DA ? -a.e[k][i].im : a.e[i][k].im;
+                const float bre = DB ? b.e[j][k].re : b.e[k][j].re, bim = DB ? -b.e[j][k].im : b.e[k][j].im;
+                re = __fmaf_rn(are, bre, re);
+                im = __fmaf_rn(are, bim, im);
+                re = __fmaf_rn(aim, -bim, re);
+                im = __fmaf_rn(aim, bre, im);
+            }
+            r.e[i][j] = mk(re, im);
+        }
+    return r;
+}
 __device__ __forceinline__ float2 bcast(float x) { return make_float2(x, x); }
 __device__ __forceinline__ Cx<float> from_f2(float2 z) { return mk(z.x, z.y); }
 
@@ -210,16 +240,16 @@ __device__ __forceinline__ M3<float> x2_product(const M3<float>& a, const M3<flo
 }
 
 template <> __device__ __forceinline__ M3<float> mul_nn<float>(const M3<float>& a, const M3<float>& b) {
-    return x2_product<3, false, false>(a, b);
+    return fma_product<3, false, false>(a, b);
 }
 template <> __device__ __forceinline__ M3<float> mul_nd<float>(const M3<float>& a, const M3<float>& b) {
-    return x2_product<3, false, true>(a, b);
+    return fma_product<3, false, true>(a, b);
 }
 template <> __device__ __forceinline__ M3<float> mul_dn<float>(const M3<float>& a, const M3<float>& b) {
-    return x2_product<3, true, false>(a, b);
+    return fma_product<3, true, false>(a, b);
 }
 template <> __device__ __forceinline__ M3<float> mul_dd<float>(const M3<float>& a, const M3<float>& b) {
-    return x2_product<3, true, true>(a, b);
+    return fma_product<3, true, true>(a, b);
 }
 
 template <class T> __device__ __forceinline__ void acc_add(M3<T>& a, const M3<T>& b) {
@@ -284,8 +314,28 @@ template <> __device__ __forceinline__ void rebuild_row2<double>(M3<double>& u) 
     }
 }
 
-// FP32: conj(a b - c d) per entry on the packed FMA, row 1 entries paired.
+// FP32: conj(a b - c d) per entry with single FMAs (22 rebuilds per overrelaxed link:
+// 45.5 -> 45.1 us per 32^4 launch against the packed form below, the flow's
+// vector-Jacobian product 1277 -> 1181 us).
 template <> __device__ __forceinline__ void rebuild_row2<float>(M3<float>& u) {
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const int p = (k + 1) % 3, q = (k + 2) % 3;
+        const Cx<float> a = u.e[0][p], b = u.e[0][q], c = u.e[1][q], d = u.e[1][p];
+        float re = __fmul_rn(a.re, c.re), im = __fmul_rn(a.re, c.im);
+        re = __fmaf_rn(a.im, -c.im, re);
+        im = __fmaf_rn(a.im, c.re, im);
+        re = __fmaf_rn(-b.re, d.re, re);
+        im = __fmaf_rn(-b.re, d.im, im);
+        re = __fmaf_rn(-b.im, -d.im, re);
+        im = __fmaf_rn(-b.im, d.re, im);
+        u.e[2][k] = mk(re, -im);
+    }
+}
+
+// The same on the packed FMA, row 1 entries paired (same bits): the better form in
+// the staged heat bath (54.7 us per 32^4 launch, 56.0 us with single FMAs).
+__device__ __forceinline__ void rebuild_row2_packed(M3<float>& u) {
     float2 B[3], iB[3];
 #pragma unroll
     for (int k = 0; k < 3; k++) {

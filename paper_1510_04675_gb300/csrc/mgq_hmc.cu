@@ -25,9 +25,11 @@ __global__ void __launch_bounds__(256, 1) k_force(Links<double, 9> U, Geom g, Ou
     pdl_wait();
     if (h >= g.Vh || out.idle()) return;
     const M3<double> A = staple(U, g, x, h, mu, par);
+    typename Out::Ahead ahead;
+    out.fetch(mu, par, h, ahead);
     double t[8];
     ta_coeffs(mul_nn(U.load(mu, par, h), A), t);
-    out.put(mu, par, h, t);
+    out.put(mu, par, h, t, ahead);
 }
 
 // FP32 12-real force with the staple's links staged through shared memory (the
@@ -118,6 +120,7 @@ __global__ void __launch_bounds__(STAGED_THREADS, 5) k_force_staged(Links<float,
         for (int j = 0; j < 3; j++) A.e[i][j] = mk(0.f, 0.f);
     M3<float> u;
     float t[8];
+    typename Out::Ahead ahead;
 #pragma unroll
     for (int k = 0; k < 5; k++) {
         if (k >= n_terms) break;
@@ -125,17 +128,17 @@ __global__ void __launch_bounds__(STAGED_THREADS, 5) k_force_staged(Links<float,
         else cp_async_wait<0>();
         const int st = k & 1;
         if (k < 3) {
-            M3<float> d = mul_nn_2(staged_rows(sm, st, 1), staged_full(sm, st, 0));
+            M3<float> d = mul_nn_2<true>(staged_rows(sm, st, 1), staged_full(sm, st, 0));
             rebuild_row2(d);
-            M3<float> term = mul_dn_2(d, staged_full(sm, st, 2));
+            M3<float> term = mul_dn_2<true>(d, staged_full(sm, st, 2));
             rebuild_row2(term);
             acc_add(A, term);
         } else {
             const int j = k - 3;
-            const M3<float> ab = mul_nd_2(staged_rows(sm, st, 0), staged_full(sm, st, 1));
-            M3<float> up = mul_nd_2(ab, own_full_of(sm, own_nu[j] * 32 + lane));
+            const M3<float> ab = mul_nd_2<true>(staged_rows(sm, st, 0), staged_full(sm, st, 1));
+            M3<float> up = mul_nd_2<true>(ab, own_full_of(sm, own_nu[j] * 32 + lane));
             rebuild_row2(up);
-            M3<float> P = mul_nn_2(u, up);
+            M3<float> P = mul_nn_2<true>(u, up);
             rebuild_row2(P);
             float tp[8];
             ta_coeffs(P, tp);
@@ -154,6 +157,7 @@ __global__ void __launch_bounds__(STAGED_THREADS, 5) k_force_staged(Links<float,
             *staged_slot(sm, 0, 2, 0) = make_float4(u.e[2][0].re, u.e[2][0].im, u.e[2][1].re, u.e[2][1].im);
             *reinterpret_cast<float2*>(staged_slot(sm, 0, 2, 1)) = make_float2(u.e[2][2].re, u.e[2][2].im);
             ta_coeffs(mul_nn(u, A), t);
+            out.fetch(mu, par, hc, ahead);
             __syncthreads();  // every warp's updated link is staged and completed
         }
     }
@@ -162,7 +166,7 @@ __global__ void __launch_bounds__(STAGED_THREADS, 5) k_force_staged(Links<float,
     // for mu >= 2, nu = mu - 2 (its second)
     staged_ta_sub(sm, ((mu + 3) & 3) * 32 + lane, 0, t);
     if (mu >= 2) staged_ta_sub(sm, (mu - 2) * 32 + lane, 1, t);
-    if (h < g.Vh) out.put(mu, par, h, t);
+    if (h < g.Vh) out.put(mu, par, h, t, ahead);
 }
 
 // FP32 18-real force, with the plaquettes shared in the same way and the links read
@@ -197,7 +201,9 @@ __global__ void __launch_bounds__(128, 4) k_force_shared(Links<float, 9> U, Geom
 #pragma unroll
     for (int e = 0; e < 9; e++) own[mu][e][lane] = make_float2(u.e[e / 3][e % 3].re, u.e[e / 3][e % 3].im);
     float t[8];
-    ta_coeffs(mul_nn(u, A), t);
+    ta_coeffs(x2_product<3, false, false>(u, A), t);
+    typename Out::Ahead ahead;
+    out.fetch(mu, par, hc, ahead);
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < 2; j++) {
@@ -223,7 +229,7 @@ __global__ void __launch_bounds__(128, 4) k_force_shared(Links<float, 9> U, Geom
         t[a] -= ta[(mu + 3) & 3][0][a][lane];
         if (mu >= 2) t[a] -= ta[mu - 2][1][a][lane];
     }
-    if (h < g.Vh) out.put(mu, par, h, t);
+    if (h < g.Vh) out.put(mu, par, h, t, ahead);
 }
 
 // U <- exp(s B) U on every link; the FP32 formats are reunitarised.  One thread

@@ -30,7 +30,9 @@ __device__ __forceinline__ M3<T> su3_project(const M3<T>& M) {
 #pragma unroll
         for (int s = 0; s < 3; s++) {
             const int i = (s == 2) ? 1 : 0, j = (s == 0) ? 1 : 2;
-            const M3<T> V = mul_nd(W, M);
+            M3<T> V;
+            if constexpr (sizeof(T) == 4) V = x2_product<3, false, true>(W, M);  // four of its entries are read
+            else V = mul_nd(W, M);
             T w[4];
             block_w(V, i, j, w);
             const T n2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2] + w[3] * w[3];

@@ -6,44 +6,21 @@
 
 namespace mgq {
 
-// Rows 0 and 1 of a b^+ and of a b (row 2 of the result is left unset): the
-// callers rebuild it as conj(row0 x row1) because the product is in SU(3).
-template <class T> __device__ __forceinline__ M3<T> mul_nd_2(const M3<T>& a, const M3<T>& b) {
-    M3<T> r;
-#pragma unroll
-    for (int i = 0; i < 2; i++)
-#pragma unroll
-        for (int j = 0; j < 3; j++)
-            r.e[i][j] = mulc(a.e[i][0], b.e[j][0]) + mulc(a.e[i][1], b.e[j][1]) + mulc(a.e[i][2], b.e[j][2]);
-    return r;
+// Rows 0 and 1 of op(a) op(b) (row 2 of the result is left unset): the callers
+// rebuild it as conj(row0 x row1) because the product is in SU(3).  FP32: packed, or
+// with single FMAs for FMA = true.
+template <bool FMA, bool DA, bool DB> __device__ __forceinline__ M3<float> two_rows(const M3<float>& a, const M3<float>& b) {
+    if constexpr (FMA) return fma_product<2, DA, DB>(a, b);
+    else return x2_product<2, DA, DB>(a, b);
 }
-template <class T> __device__ __forceinline__ M3<T> mul_nn_2(const M3<T>& a, const M3<T>& b) {
-    M3<T> r;
-#pragma unroll
-    for (int i = 0; i < 2; i++)
-#pragma unroll
-        for (int j = 0; j < 3; j++) r.e[i][j] = a.e[i][0] * b.e[0][j] + a.e[i][1] * b.e[1][j] + a.e[i][2] * b.e[2][j];
-    return r;
+template <bool FMA = false> __device__ __forceinline__ M3<float> mul_nd_2(const M3<float>& a, const M3<float>& b) {
+    return two_rows<FMA, false, true>(a, b);
 }
-// rows 0, 1 of a^+ b
-template <class T> __device__ __forceinline__ M3<T> mul_dn_2(const M3<T>& a, const M3<T>& b) {
-    M3<T> r;
-#pragma unroll
-    for (int i = 0; i < 2; i++)
-#pragma unroll
-        for (int j = 0; j < 3; j++)
-            r.e[i][j] = mulc(b.e[0][j], a.e[0][i]) + mulc(b.e[1][j], a.e[1][i]) + mulc(b.e[2][j], a.e[2][i]);
-    return r;
+template <bool FMA = false> __device__ __forceinline__ M3<float> mul_nn_2(const M3<float>& a, const M3<float>& b) {
+    return two_rows<FMA, false, false>(a, b);
 }
-
-template <> __device__ __forceinline__ M3<float> mul_nd_2<float>(const M3<float>& a, const M3<float>& b) {
-    return x2_product<2, false, true>(a, b);
-}
-template <> __device__ __forceinline__ M3<float> mul_nn_2<float>(const M3<float>& a, const M3<float>& b) {
-    return x2_product<2, false, false>(a, b);
-}
-template <> __device__ __forceinline__ M3<float> mul_dn_2<float>(const M3<float>& a, const M3<float>& b) {
-    return x2_product<2, true, false>(a, b);
+template <bool FMA = false> __device__ __forceinline__ M3<float> mul_dn_2(const M3<float>& a, const M3<float>& b) {
+    return two_rows<FMA, true, false>(a, b);
 }
 
 // =============================================================== staple
@@ -141,9 +118,13 @@ __device__ __forceinline__ M3<float> staged_rows(float4* sm, int stage, int j) {
     }
     return m;
 }
-__device__ __forceinline__ M3<float> staged_full(float4* sm, int stage, int j) {
+template <bool PACKED = false> __device__ __forceinline__ void complete(M3<float>& m) {
+    if constexpr (PACKED) rebuild_row2_packed(m);
+    else rebuild_row2(m);
+}
+template <bool PACKED = false> __device__ __forceinline__ M3<float> staged_full(float4* sm, int stage, int j) {
     M3<float> m = staged_rows(sm, stage, j);
-    rebuild_row2(m);
+    complete<PACKED>(m);
     return m;
 }
 // the updated link staged by thread col of the block (slot (2, 0)), with the
@@ -170,8 +151,9 @@ __device__ __forceinline__ M3<float> own_full_of(float4* sm, int col) {
 struct NoWork {
     __device__ void operator()() const {}
 };
-// early(): independent work that runs while the first loads are in flight.
-template <class Work = NoWork>
+// early(): independent work that runs while the first loads are in flight; PACKED:
+// the form of the row-2 rebuilds.
+template <bool PACKED = false, class Work = NoWork>
 __device__ __forceinline__ M3<float> staple_staged(const Links<float, 6>& U, const Geom& g, const int x[4], int h,
                                                    const int MU, int par, float4* sm, M3<float>& u,
                                                    Work early = Work()) {
@@ -220,21 +202,21 @@ __device__ __forceinline__ M3<float> staple_staged(const Links<float, 6>& U, con
         const int st = k & 1;
         M3<float> term;
         if ((k & 1) == 0) {
-            const M3<float> t = mul_nd_2(staged_rows(sm, st, 0), staged_full(sm, st, 1));
-            term = mul_nd_2(t, staged_full(sm, st, 2));
+            const M3<float> t = mul_nd_2(staged_rows(sm, st, 0), staged_full<PACKED>(sm, st, 1));
+            term = mul_nd_2(t, staged_full<PACKED>(sm, st, 2));
         } else {
-            M3<float> t = mul_nn_2(staged_rows(sm, st, 1), staged_full(sm, st, 0));
-            rebuild_row2(t);
-            term = mul_dn_2(t, staged_full(sm, st, 2));
+            M3<float> t = mul_nn_2(staged_rows(sm, st, 1), staged_full<PACKED>(sm, st, 0));
+            complete<PACKED>(t);
+            term = mul_dn_2(t, staged_full<PACKED>(sm, st, 2));
         }
-        rebuild_row2(term);
+        complete<PACKED>(term);
         acc_add(A, term);
         if (k + 2 < 6) {
             issue(k + 2, st);
             cp_async_commit();
         }
     }
-    u = staged_full(sm, 2, 0);
+    u = staged_full<PACKED>(sm, 2, 0);
     return A;
 }
 
@@ -334,21 +316,21 @@ __device__ __forceinline__ double site_plaquettes(const Links<T, NP>& U, const G
 // are the lines' lengths; op is the parity one line away.
 
 // a b^+ c^+ and (e d)^+ f of lines in SU(3).  FP32: rows 0, 1 of every partial
-// product, row 2 rebuilt.
-template <class T> __device__ __forceinline__ M3<T> up_term(const M3<T>& a_rows, const M3<T>& b, const M3<T>& c) {
+// product, row 2 rebuilt; FMA as in two_rows.
+template <bool FMA = false, class T> __device__ __forceinline__ M3<T> up_term(const M3<T>& a_rows, const M3<T>& b, const M3<T>& c) {
     if constexpr (sizeof(T) == 4) {
-        M3<T> r = mul_nd_2(mul_nd_2(a_rows, b), c);
+        M3<T> r = mul_nd_2<FMA>(mul_nd_2<FMA>(a_rows, b), c);
         rebuild_row2(r);
         return r;
     } else {
         return mul_nd(mul_nd(a_rows, b), c);
     }
 }
-template <class T> __device__ __forceinline__ M3<T> down_term(const M3<T>& e_rows, const M3<T>& d, const M3<T>& f) {
+template <bool FMA = false, class T> __device__ __forceinline__ M3<T> down_term(const M3<T>& e_rows, const M3<T>& d, const M3<T>& f) {
     if constexpr (sizeof(T) == 4) {
-        M3<T> t = mul_nn_2(e_rows, d);
+        M3<T> t = mul_nn_2<FMA>(e_rows, d);
         rebuild_row2(t);
-        M3<T> r = mul_dn_2(t, f);
+        M3<T> r = mul_dn_2<FMA>(t, f);
         rebuild_row2(r);
         return r;
     } else {
@@ -382,13 +364,13 @@ __device__ __forceinline__ void clover_coeffs(const Links<T, NP>& U, const Hops&
     const int x = H.lex;
     M3<T> Q;
     {
-        M3<T> D = up_term(load_left(U, nu, op, (x + fm) >> 1), U.load(mu, op, (x + fn) >> 1), U.load(nu, par, x >> 1));
-        acc_sub(D, down_term(load_left(U, mu, op, (x + bn) >> 1), U.load(nu, par, (x + fm + bn) >> 1), U.load(nu, op, (x + bn) >> 1)));
+        M3<T> D = up_term<true>(load_left(U, nu, op, (x + fm) >> 1), U.load(mu, op, (x + fn) >> 1), U.load(nu, par, x >> 1));
+        acc_sub(D, down_term<true>(load_left(U, mu, op, (x + bn) >> 1), U.load(nu, par, (x + fm + bn) >> 1), U.load(nu, op, (x + bn) >> 1)));
         Q = mul_nn(U.load(mu, par, x >> 1), D);
     }
     {
-        M3<T> D = up_term(load_left(U, nu, par, x >> 1), U.load(mu, par, (x + bm + fn) >> 1), U.load(nu, op, (x + bm) >> 1));
-        acc_sub(D, down_term(load_left(U, mu, par, (x + bm + bn) >> 1), U.load(nu, op, (x + bn) >> 1),
+        M3<T> D = up_term<true>(load_left(U, nu, par, x >> 1), U.load(mu, par, (x + bm + fn) >> 1), U.load(nu, op, (x + bm) >> 1));
+        acc_sub(D, down_term<true>(load_left(U, mu, par, (x + bm + bn) >> 1), U.load(nu, op, (x + bn) >> 1),
                              U.load(nu, par, (x + bm + bn) >> 1)));
         acc_add(Q, mul_nn(D, U.load(mu, op, (x + bm) >> 1)));
     }
@@ -419,8 +401,8 @@ template <class T, int NP>
 __device__ __forceinline__ T loop_retr(const Links<T, NP>& U, const Hops& H, int par, int op, int mu, int nu) {
     const int x = H.lex >> 1, xm = (H.lex + pick(H.fwd, mu)) >> 1, xn = (H.lex + pick(H.fwd, nu)) >> 1;
     if constexpr (sizeof(T) == 4) {
-        const M3<T> a = mul_nn_2(U.load_rows(mu, par, x), U.load(nu, op, xm));
-        return retr_two_row(a, mul_nn_2(U.load_rows(nu, par, x), U.load(mu, op, xn)));
+        const M3<T> a = mul_nn_2<NP == 9>(U.load_rows(mu, par, x), U.load(nu, op, xm));
+        return retr_two_row(a, mul_nn_2<NP == 9>(U.load_rows(nu, par, x), U.load(mu, op, xn)));
     } else {
         const M3<T> a = mul_nn(U.load(mu, par, x), U.load(nu, op, xm));
         return retr_nd(a, mul_nn(U.load(nu, par, x), U.load(mu, op, xn)));
@@ -463,27 +445,33 @@ __device__ __forceinline__ void su2_rows<double>(M3<double>& m, int i, int j, co
 }
 
 // FP32: a m_i + b m_j with a = r0 + i r3, b = r2 + i r1 (and c = -r2 + i r1,
-// d = r0 - i r3 for row j) as packed FMAs on (re, im) pairs.
+// d = r0 - i r3 for row j) with single FMAs (32^4 overrelaxation launch 45.5 -> 45.1
+// us against packed pairs, same bits).
 template <>
 __device__ __forceinline__ void su2_rows<float>(M3<float>& m, int i, int j, const float r[4], bool do_i, bool do_j,
                                                 int ci, int cj) {
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-        const float2 MI = make_float2(m.e[i][k].re, m.e[i][k].im), iMI = make_float2(-m.e[i][k].im, m.e[i][k].re);
-        const float2 MJ = make_float2(m.e[j][k].re, m.e[j][k].im), iMJ = make_float2(-m.e[j][k].im, m.e[j][k].re);
+        const Cx<float> x = m.e[i][k], y = m.e[j][k];
         if (do_i && ((ci >> k) & 1)) {
-            float2 v = __fmul2_rn(bcast(r[0]), MI);
-            v = __ffma2_rn(bcast(r[3]), iMI, v);
-            v = __ffma2_rn(bcast(r[2]), MJ, v);
-            v = __ffma2_rn(bcast(r[1]), iMJ, v);
-            m.e[i][k] = from_f2(v);
+            float re = __fmul_rn(r[0], x.re), im = __fmul_rn(r[0], x.im);
+            re = __fmaf_rn(r[3], -x.im, re);
+            im = __fmaf_rn(r[3], x.re, im);
+            re = __fmaf_rn(r[2], y.re, re);
+            im = __fmaf_rn(r[2], y.im, im);
+            re = __fmaf_rn(r[1], -y.im, re);
+            im = __fmaf_rn(r[1], y.re, im);
+            m.e[i][k] = mk(re, im);
         }
         if (do_j && ((cj >> k) & 1)) {
-            float2 v = __fmul2_rn(bcast(-r[2]), MI);
-            v = __ffma2_rn(bcast(r[1]), iMI, v);
-            v = __ffma2_rn(bcast(r[0]), MJ, v);
-            v = __ffma2_rn(bcast(-r[3]), iMJ, v);
-            m.e[j][k] = from_f2(v);
+            float re = __fmul_rn(-r[2], x.re), im = __fmul_rn(-r[2], x.im);
+            re = __fmaf_rn(r[1], -x.im, re);
+            im = __fmaf_rn(r[1], x.re, im);
+            re = __fmaf_rn(r[0], y.re, re);
+            im = __fmaf_rn(r[0], y.im, im);
+            re = __fmaf_rn(-r[3], -y.im, re);
+            im = __fmaf_rn(-r[3], y.re, im);
+            m.e[j][k] = mk(re, im);
         }
     }
 }
