@@ -107,10 +107,10 @@ class FlowedObservable(torch.autograd.Function):
         for start, links in reversed(ctx.ckpts):
             m = min(ctx.n - start, ctx.k)
             seg.links.copy_(links)
-            starts = []
-            for _ in range(m):
-                starts.append(seg.links.clone())
+            starts = [links]
+            for _ in range(m - 1):  # the field after the segment's last step is not needed
                 _flow_steps(seg, ctx.eps, 1)
+                starts.append(seg.links.clone())
             for w0 in reversed(starts):
                 seg.links.copy_(w0)
                 api.mgq_wilson_flow_step_adjoint(seg, ctx.eps, lam, scratch)

@@ -34,23 +34,26 @@ template <class T> __device__ __forceinline__ M3<T> commutator_ah(const M3<T>& a
     return r;
 }
 
-// Per link: X = c0 Z0 + c1 Z1 + c2 Z2; Xi = J(X)* Lam, the series summed until a
-// term drops below the precision's rounding of the partial sum (|X| is O(eps):
-// a few terms; at most 12 in FP64 and 8 in FP32, enough for |X| <= 0.5);
-// Lam <- e^{-X} Lam e^{X}.
+// Per link: X = ca Za + cb Zb; Xi = J(X)* Lam, the series summed until a term drops
+// below the precision's rounding of the partial sum (|X| is O(eps): a few terms; at
+// most 12 in FP64 and 8 in FP32, enough for |X| <= 0.5); Lam <- e^{-X} Lam e^{X};
+// Out <- s Xi + p Prev (cb == 0, p == 0: Zb, Prev not read).
 template <class T>
-__global__ void __launch_bounds__(128) k_dexp_adjoint(Geom g, Alg<T> Z0, Alg<T> Z1, Alg<T> Z2, T c0, T c1, T c2,
-                                                      Alg<T> Lam, Alg<T> Xi) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 8 * g.Vh) return;
-    const int mp = idx / g.Vh, h = idx - mp * g.Vh, mu = mp >> 1, par = mp & 1;
-    T z0[8], z1[8], z2[8], x[8], l[8];
-    Z0.load(mu, par, h, z0);
-    Z1.load(mu, par, h, z1);
-    Z2.load(mu, par, h, z2);
-    Lam.load(mu, par, h, l);
+__global__ void __launch_bounds__(128) k_dexp_adjoint(Geom g, Alg<T> Za, Alg<T> Zb, T ca, T cb, Alg<T> Lam, Alg<T> Out, Alg<T> Prev,
+                                                      T s, T p) {
+    const int mu = blockIdx.y >> 1, par = blockIdx.y & 1, h = blockIdx.x * blockDim.x + threadIdx.x;
+    if (h >= g.Vh) return;
+    T x[8], l[8];
+    Za.load(mu, par, h, x);
 #pragma unroll
-    for (int a = 0; a < 8; a++) x[a] = c0 * z0[a] + c1 * z1[a] + c2 * z2[a];
+    for (int a = 0; a < 8; a++) x[a] *= ca;
+    if (cb != T(0)) {
+        T z[8];
+        Zb.load(mu, par, h, z);
+#pragma unroll
+        for (int a = 0; a < 8; a++) x[a] += cb * z[a];
+    }
+    Lam.load(mu, par, h, l);
     const M3<T> X = alg_matrix(x);
     const M3<T> L = alg_matrix(l);
     M3<T> term = L, sum = L;
@@ -73,7 +76,16 @@ __global__ void __launch_bounds__(128) k_dexp_adjoint(Geom g, Alg<T> Z0, Alg<T> 
     }
     T xi[8];
     ta_coeffs(sum, xi);
-    Xi.store(mu, par, h, xi);
+    if (p != T(0)) {
+        T q[8];
+        Prev.load(mu, par, h, q);
+#pragma unroll
+        for (int a = 0; a < 8; a++) xi[a] = s * xi[a] + p * q[a];
+    } else {
+#pragma unroll
+        for (int a = 0; a < 8; a++) xi[a] *= s;
+    }
+    Out.store(mu, par, h, xi);
     const M3<T> E = exp_alg(x);
     const M3<T> Ln = mul_dn(E, mul_nn(L, E));
     T ln[8];
@@ -117,21 +129,6 @@ __global__ void __launch_bounds__(128) k_exp_vjp(Geom g, Alg<T> Om, Alg<T> Gin, 
     Gout.store(mu, par, h, out);
 }
 
-// P <- a0 X0 + a1 X1 + a2 X2 (algebra coefficients, elementwise)
-template <class T>
-__global__ void k_alg_combine(Geom g, Alg<T> P, Alg<T> X0, Alg<T> X1, Alg<T> X2, T a0, T a1, T a2) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 8 * g.Vh) return;
-    const int mp = idx / g.Vh, h = idx - mp * g.Vh, mu = mp >> 1, par = mp & 1;
-    T p[8], u[8], v[8], w[8];
-    X0.load(mu, par, h, u);
-    X1.load(mu, par, h, v);
-    X2.load(mu, par, h, w);
-#pragma unroll
-    for (int a = 0; a < 8; a++) p[a] = a0 * u[a] + a1 * v[a] + a2 * w[a];
-    P.store(mu, par, h, p);
-}
-
 template <class T, int NP>
 __device__ __forceinline__ M3<T> psi_at(const Alg<T>& P, int mu, int par, int h) {
     T c[8];
@@ -146,8 +143,7 @@ __device__ __forceinline__ M3<T> psi_at(const Alg<T>& P, int mu, int par, int h)
 // it, one it traverses backwards (as W^+) carries -Psi just after it.  Its
 // cotangent at m is -TA(U_m R), R the rest of the loop after m with one
 // insertion at a time, summed; the insertion at m itself is the self term
-// -TA(W_m A_m Psi_m), which the two launches below add half by half (the upper
-// and the lower staples of A_m).
+// -TA(W_m A_m Psi_m), A_m the staple.
 
 template <class T> __device__ __forceinline__ M3<T> msub(const M3<T>& a, const M3<T>& b) {
     M3<T> r;
@@ -164,18 +160,19 @@ template <class T> __device__ __forceinline__ M3<T> msub(const M3<T>& a, const M
 //         R_up = Psi_nu(y+rho) X1 X2 X3 - X1 X2 Psi_rho(y+nu) X3 - X1 X2 X3 Psi_nu(y)
 //   down: m Y1 Y2 Y3,   Y1 = U_nu(y-nu+rho)^+, Y2 = U_rho(y-nu)^+, Y3 = U_nu(y-nu)
 //         R_dn = -Y1 Psi_nu(y-nu+rho) Y2 Y3 - Y1 Y2 Psi_rho(y-nu) Y3 + Y1 Y2 Psi_nu(y-nu) Y3
-// each summed by the product rule over the running prefix; SIDE 0 adds
-// scale * (-TA(U_m (sum_nu R_up + A_up Psi_m))), SIDE 1 the same with R_dn and
-// A_dn, A_up = sum_nu X1 X2 X3 and A_dn = sum_nu Y1 Y2 Y3 the two halves of the
-// staple (one side per launch, directions in a rolled loop, keeps the live
-// state in registers).  SIDE 0 folds X1 X2 X3 Psi_m into its last insertion
-// (both Psi at y); SIDE 1 sums A_dn and multiplies by Psi_m once.
-template <class T, int NP, int SIDE>
-__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 1 : 4) k_flow_vjp_plane(Links<T, NP> U, Geom g, Alg<T> Psi, T scl, Alg<T> Lam) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 8 * g.Vh) return;
-    const int mp = idx / g.Vh, h = idx - mp * g.Vh, rho = mp >> 1, par = mp & 1;
-    const int op = par ^ 1;
+// each summed by the product rule over the running prefix, plus the staples'
+// share of the self term: scale * (-TA(U_m (sum_nu R_up + R_dn + A Psi_m))), A = sum_nu
+// (X1 X2 X3 + Y1 Y2 Y3).  X1 X2 X3 Psi_m folds into the last insertion of R_up (both
+// Psi at y); the lower staples are summed and multiplied by Psi_m once.  The planes
+// run in a rolled loop, a plane's two sides one after the other, so that the live
+// matrices stay in registers, and the four warps of a block take the four
+// directions at the same 32 sites, whose links and cotangents they share in L1.
+// 16^4, FP32 12-real: 74 us as two launches (a side each, with its own pass over
+// Lam, U_m and Psi_m), 59 us so.
+template <class T, int NP>
+__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 1 : 3) k_flow_vjp(Links<T, NP> U, Geom g, Alg<T> Psi, T scl, Alg<T> Lam) {
+    const int rho = threadIdx.x >> 5, par = blockIdx.y, op = par ^ 1, h = blockIdx.x * 32 + (threadIdx.x & 31);
+    if (h >= g.Vh) return;
     int x[4];
     cb_coords(g, par, h, x);
     const Hops H = make_hops(g, x);
@@ -187,47 +184,46 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 1 : 4) k_flow_vjp_plane(
         for (int j = 0; j < 3; j++) Rs.e[i][j] = As.e[i][j] = mk(T(0), T(0));
 #pragma unroll 1
     for (int K = 0; K < 3; K++) {
-    const int nu = K < rho ? K : K + 1;
-    M3<T> R;
-    if constexpr (SIDE == 0) {
-        const int h_pr = (H.lex + frho) >> 1;             // y + rho  (op)
-        const int h_pn = (H.lex + pick(H.fwd, nu)) >> 1;  // y + nu   (op)
-        const M3<T> X1 = U.load(nu, op, h_pr);
-        const M3<T> X2d = U.load(rho, op, h_pn);  // X2 = X2d^+
-        const M3<T> X3d = U.load(nu, par, h);     // X3 = X3d^+
-        const M3<T> P2 = mul_nd(X1, X2d);         // X1 X2
-        const M3<T> S = mul_nd(P2, X3d);          // X1 X2 X3, the upper staple
-        // the self term's X1 X2 X3 Psi_m joins the last insertion: - X1 X2 X3 (Psi_nu(y) - Psi_m)
-        T cn[8], cm[8];
-        Psi.load(nu, par, h, cn);
-        Psi.load(rho, par, h, cm);
+        const int nu = K < rho ? K : K + 1;
+        {
+            const int h_pr = (H.lex + frho) >> 1;             // y + rho  (op)
+            const int h_pn = (H.lex + pick(H.fwd, nu)) >> 1;  // y + nu   (op)
+            const M3<T> X1 = U.load(nu, op, h_pr);
+            const M3<T> X2d = U.load(rho, op, h_pn);  // X2 = X2d^+
+            const M3<T> X3d = U.load(nu, par, h);     // X3 = X3d^+
+            const M3<T> P2 = mul_nd(X1, X2d);         // X1 X2
+            const M3<T> S = mul_nd(P2, X3d);          // X1 X2 X3, the upper staple
+            // R_up + S Psi_m = Psi_nu(y+rho) S - (X1 X2 Psi_rho(y+nu)) X3 - S (Psi_nu(y) - Psi_m)
+            acc_sub(Rs, mul_nd(mul_nn(P2, psi_at<T, NP>(Psi, rho, op, h_pn)), X3d));
+            acc_add(Rs, mul_nn(psi_at<T, NP>(Psi, nu, op, h_pr), S));
+            T cn[8], cm[8];
+            Psi.load(nu, par, h, cn);
+            Psi.load(rho, par, h, cm);
 #pragma unroll
-        for (int a = 0; a < 8; a++) cn[a] -= cm[a];
-        // R_up + S Psi_m = Psi_nu(y+rho) S - (X1 X2 Psi_rho(y+nu)) X3 - S (Psi_nu(y) - Psi_m)
-        R = msub(msub(mul_nn(psi_at<T, NP>(Psi, nu, op, h_pr), S),
-                      mul_nd(mul_nn(P2, psi_at<T, NP>(Psi, rho, op, h_pn)), X3d)),
-                 mul_nn(S, alg_matrix(cn)));
-    } else {
-        const int bnu = pick(H.bwd, nu);
-        const int h_mn = (H.lex + bnu) >> 1;            // y - nu        (op)
-        const int h_mn_pr = (H.lex + bnu + frho) >> 1;  // y - nu + rho  (par)
-        const M3<T> Y1d = U.load(nu, par, h_mn_pr);  // Y1 = Y1d^+
-        const M3<T> Y2d = U.load(rho, op, h_mn);     // Y2 = Y2d^+
-        const M3<T> P2 = mul_dd(Y1d, Y2d);           // Y1 Y2
-        // R_dn = (Y1 Y2 (Psi_c - Psi_b) - Y1 Psi_a Y2) Y3, Psi_b and Psi_c both at y - nu
-        T cc[8], cb[8];
-        Psi.load(nu, op, h_mn, cc);
-        Psi.load(rho, op, h_mn, cb);
+            for (int a = 0; a < 8; a++) cn[a] -= cm[a];
+            acc_sub(Rs, mul_nn(S, alg_matrix(cn)));
+        }
+        {
+            const int bnu = pick(H.bwd, nu);
+            const int h_mn = (H.lex + bnu) >> 1;            // y - nu        (op)
+            const int h_mn_pr = (H.lex + bnu + frho) >> 1;  // y - nu + rho  (par)
+            const M3<T> Y1d = U.load(nu, par, h_mn_pr);  // Y1 = Y1d^+
+            const M3<T> Y2d = U.load(rho, op, h_mn);     // Y2 = Y2d^+
+            const M3<T> P2 = mul_dd(Y1d, Y2d);           // Y1 Y2
+            // R_dn = (Y1 Y2 (Psi_c - Psi_b) - Y1 Psi_a Y2) Y3, Psi_b and Psi_c both at y - nu
+            M3<T> Q = mul_nd(mul_dn(Y1d, psi_at<T, NP>(Psi, nu, par, h_mn_pr)), Y2d);
+            T cc[8], cb[8];
+            Psi.load(nu, op, h_mn, cc);
+            Psi.load(rho, op, h_mn, cb);
 #pragma unroll
-        for (int a = 0; a < 8; a++) cc[a] -= cb[a];
-        const M3<T> Q = msub(mul_nn(P2, alg_matrix(cc)), mul_nd(mul_dn(Y1d, psi_at<T, NP>(Psi, nu, par, h_mn_pr)), Y2d));
-        const M3<T> Y3 = U.load(nu, op, h_mn);
-        R = mul_nn(Q, Y3);
-        acc_add(As, mul_nn(P2, Y3));                 // Y1 Y2 Y3, the lower staple
+            for (int a = 0; a < 8; a++) cc[a] -= cb[a];
+            Q = msub(mul_nn(P2, alg_matrix(cc)), Q);
+            const M3<T> Y3 = U.load(nu, op, h_mn);
+            acc_add(Rs, mul_nn(Q, Y3));
+            acc_add(As, mul_nn(P2, Y3));                 // Y1 Y2 Y3, the lower staple
+        }
     }
-    acc_add(Rs, R);
-    }
-    if constexpr (SIDE == 1) acc_add(Rs, mul_nn(As, psi_at<T, NP>(Psi, rho, par, h)));  // the self term's half
+    acc_add(Rs, mul_nn(As, psi_at<T, NP>(Psi, rho, par, h)));  // the lower staples' share of the self term
     T t[8];
     ta_coeffs(mul_nn(U.load(rho, par, h), Rs), t);
     T* b = Lam.at(rho, par, h);
@@ -243,39 +239,23 @@ static mgq_status flow_vjp(const mgq_lattice* lat, const void* links, const void
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
         const Links<T, NP> W = links_at<T, NP>(const_cast<void*>(links), lat->dims);
         const Alg<T> P = alg_at<T>(const_cast<void*>(psi), lat->dims), L = alg_at<T>(lam, lat->dims);
-        const int nb = nblk(8L * g.Vh, 128);
-        k_flow_vjp_plane<T, NP, 0><<<nb, 128, 0, st>>>(W, g, P, (T)scl, L);
-        k_flow_vjp_plane<T, NP, 1><<<nb, 128, 0, st>>>(W, g, P, (T)scl, L);
+        k_flow_vjp<T, NP><<<dim3(nblk(g.Vh, 32), 2), 128, 0, st>>>(W, g, P, (T)scl, L);
     });
     return cuda_check("flow_vjp");
 }
 
-static mgq_status dexp_adjoint(const mgq_lattice* lat, void* z0, void* z1, void* z2, double c0, double c1, double c2,
-                               void* lam, void* xi, cudaStream_t st) {
+static mgq_status dexp_adjoint(const mgq_lattice* lat, void* za, void* zb, double ca, double cb, void* lam, void* out, void* prev,
+                               double s, double p, cudaStream_t st) {
     const Geom g = make_geom(lat->dims);
-    if (lat->prec == MGQ_F64)
-        k_dexp_adjoint<double><<<nblk(8L * g.Vh, 128), 128, 0, st>>>(
-            g, alg_at<double>(z0, lat->dims), alg_at<double>(z1, lat->dims), alg_at<double>(z2, lat->dims), c0, c1, c2,
-            alg_at<double>(lam, lat->dims), alg_at<double>(xi, lat->dims));
-    else
-        k_dexp_adjoint<float><<<nblk(8L * g.Vh, 128), 128, 0, st>>>(
-            g, alg_at<float>(z0, lat->dims), alg_at<float>(z1, lat->dims), alg_at<float>(z2, lat->dims), (float)c0,
-            (float)c1, (float)c2, alg_at<float>(lam, lat->dims), alg_at<float>(xi, lat->dims));
+    const dim3 grid(nblk(g.Vh, 128), 8);
+    auto launch = [&]<class T>() {
+        k_dexp_adjoint<T><<<grid, 128, 0, st>>>(g, alg_at<T>(za, lat->dims), alg_at<T>(zb, lat->dims), (T)ca, (T)cb,
+                                                alg_at<T>(lam, lat->dims), alg_at<T>(out, lat->dims), alg_at<T>(prev, lat->dims),
+                                                (T)s, (T)p);
+    };
+    if (lat->prec == MGQ_F64) launch.template operator()<double>();
+    else launch.template operator()<float>();
     return cuda_check("dexp_adjoint");
-}
-
-static mgq_status combine(const mgq_lattice* lat, void* p, void* x0, void* x1, void* x2, double a0, double a1,
-                          double a2, cudaStream_t st) {
-    const Geom g = make_geom(lat->dims);
-    if (lat->prec == MGQ_F64)
-        k_alg_combine<double><<<nblk(8L * g.Vh, 256), 256, 0, st>>>(
-            g, alg_at<double>(p, lat->dims), alg_at<double>(x0, lat->dims), alg_at<double>(x1, lat->dims),
-            alg_at<double>(x2, lat->dims), a0, a1, a2);
-    else
-        k_alg_combine<float><<<nblk(8L * g.Vh, 256), 256, 0, st>>>(
-            g, alg_at<float>(p, lat->dims), alg_at<float>(x0, lat->dims), alg_at<float>(x1, lat->dims),
-            alg_at<float>(x2, lat->dims), (float)a0, (float)a1, (float)a2);
-    return cuda_check("combine");
 }
 
 uint64_t flow_adjoint_scratch(const mgq_lattice* lat) {
@@ -318,37 +298,30 @@ mgq_status mgq_wilson_flow_step_adjoint(const mgq_lattice* lat, double eps, void
     char* p = static_cast<char*>(scratch);
     void* W1 = p;
     void* W2 = p + lb;
-    void* Z[3] = {p + 2 * lb, p + 2 * lb + ab, p + 2 * lb + 2 * ab};
-    void* Xi[3] = {p + 2 * lb + 3 * ab, p + 2 * lb + 4 * ab, p + 2 * lb + 5 * ab};
-    void* Psi = p + 2 * lb + 6 * ab;
-    const uint64_t lbytes = links_bytes(lat);
-    // forward recompute of the step from W0 = lat->links (left unchanged)
+    void* Z0 = p + 2 * lb;
+    void* X1 = p + 2 * lb + ab;
+    void* Z2 = p + 2 * lb + 2 * ab;
+    void* Xi2 = p + 2 * lb + 3 * ab;
+    void* D = p + 2 * lb + 4 * ab;     // Xi1 - Xi2
+    void* Psi0 = p + 2 * lb + 5 * ab;
+    // forward recompute of the step from W0 = lat->links (left unchanged): the force
+    // kernels write Z0 with -17/36 Z0 beside it and add 8/9 Z1 to that, the
+    // exponentials write the next field
     mgq_lattice w = *lat;
-    if ((s = force_accumulate(lat, Z[0], -eps, 0.0, st))) return s;  // Z0 = eps Z(W0)
-    if (cudaMemcpyAsync(W1, lat->links, lbytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-        return cuda_check("mgq_wilson_flow_step_adjoint");
+    if ((s = force_two(lat, Z0, -eps, X1, 17.0 / 36.0 * eps, st))) return s;       // Z0 = eps Z(W0), X1 = -17/36 Z0
     w.links = W1;
-    if ((s = exp_update(&w, Z[0], 0.25, st))) return s;                   // W1 = exp(Z0/4) W0
-    if ((s = force_accumulate(&w, Z[1], -eps, 0.0, st))) return s;        // Z1 = eps Z(W1)
-    if (cudaMemcpyAsync(W2, W1, lbytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-        return cuda_check("mgq_wilson_flow_step_adjoint");
+    if ((s = exp_update_to(lat, W1, Z0, 0.25, st))) return s;                      // W1 = exp(Z0/4) W0
+    if ((s = force_accumulate(&w, X1, -8.0 / 9.0 * eps, 1.0, st))) return s;       // X1 = 8/9 Z1 - 17/36 Z0
+    if ((s = exp_update_to(&w, W2, X1, 1.0, st))) return s;                        // W2 = exp(X1) W1
     w.links = W2;
-    if ((s = combine(lat, Psi, Z[0], Z[1], Z[1], -17.0 / 36.0, 8.0 / 9.0, 0.0, st))) return s;  // X1
-    if ((s = exp_update(&w, Psi, 1.0, st))) return s;                     // W2 = exp(X1) W1
-    if ((s = force_accumulate(&w, Z[2], -eps, 0.0, st))) return s;        // Z2 = eps Z(W2)
-    // reverse stage 2
-    if ((s = dexp_adjoint(lat, Z[0], Z[1], Z[2], 17.0 / 36.0, -8.0 / 9.0, 0.75, lambda, Xi[2], st))) return s;
-    if ((s = combine(lat, Psi, Xi[2], Xi[2], Xi[2], 0.75, 0.0, 0.0, st))) return s;
-    if ((s = flow_vjp(lat, W2, Psi, eps, lambda, st))) return s;
-    // reverse stage 1
-    if ((s = dexp_adjoint(lat, Z[0], Z[1], Z[2], -17.0 / 36.0, 8.0 / 9.0, 0.0, lambda, Xi[1], st))) return s;
-    if ((s = combine(lat, Psi, Xi[1], Xi[2], Xi[2], 8.0 / 9.0, -8.0 / 9.0, 0.0, st))) return s;
-    if ((s = flow_vjp(lat, W1, Psi, eps, lambda, st))) return s;
-    // reverse stage 0
-    if ((s = dexp_adjoint(lat, Z[0], Z[1], Z[2], 0.25, 0.0, 0.0, lambda, Xi[0], st))) return s;
-    if ((s = combine(lat, Psi, Xi[0], Xi[1], Xi[2], 0.25, -17.0 / 36.0, 17.0 / 36.0, st))) return s;
-    if ((s = flow_vjp(lat, lat->links, Psi, eps, lambda, st))) return s;
-    return MGQ_OK;
+    if ((s = force_accumulate(&w, Z2, -eps, 0.0, st))) return s;                   // Z2 = eps Z(W2)
+    // reverse stages; Psi2 = 3/4 Xi2, Psi1 = 8/9 (Xi1 - Xi2), Psi0 = Xi0/4 - 17/36 (Xi1 - Xi2)
+    if ((s = dexp_adjoint(lat, Z2, X1, 0.75, -1.0, lambda, Xi2, Xi2, 1.0, 0.0, st))) return s;
+    if ((s = flow_vjp(lat, W2, Xi2, 0.75 * eps, lambda, st))) return s;
+    if ((s = dexp_adjoint(lat, X1, X1, 1.0, 0.0, lambda, D, Xi2, 1.0, -1.0, st))) return s;
+    if ((s = flow_vjp(lat, W1, D, 8.0 / 9.0 * eps, lambda, st))) return s;
+    if ((s = dexp_adjoint(lat, Z0, Z0, 0.25, 0.0, lambda, Psi0, D, 0.25, -17.0 / 36.0, st))) return s;
+    return flow_vjp(lat, lat->links, Psi0, eps, lambda, st);
 }
 
 mgq_status mgq_exp_vjp(const mgq_lattice* lat, const void* omega, const void* g_in, void* g_out, void* stream) {

@@ -232,10 +232,10 @@ __global__ void __launch_bounds__(128, 4) k_force_shared(Links<float, 9> U, Geom
     if (h < g.Vh) out.put(mu, par, h, t, ahead);
 }
 
-// U <- exp(s B) U on every link; the FP32 formats are reunitarised.  One thread
-// per link, block row y of the grid holding the links of one (mu, parity).
+// out <- exp(s B) U on every link (out may be U); the FP32 formats are
+// reunitarised.  One thread per link, block row y of the grid holding the links of one (mu, parity).
 template <class T, int NP>
-__global__ void __launch_bounds__(128) k_exp_update(Links<T, NP> U, Geom g, Alg<T> B, T s) {
+__global__ void __launch_bounds__(128) k_exp_update(Links<T, NP> U, Links<T, NP> out, Geom g, Alg<T> B, T s) {
     if constexpr (sizeof(T) == 4) pdl_launch_dependents();  // FP64: at the end, see k_update_columns
     const int mu = blockIdx.y >> 1, par = blockIdx.y & 1, h = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(128) k_exp_update(Links<T, NP> U, Geom g, Alg<
     M3<T> u = mul_nn(exp_alg(c), u0);
     if (sizeof(T) == 4) reunitarize(u);
     else pdl_launch_dependents();
-    U.store(mu, par, h, u);
+    out.store(mu, par, h, u);
 }
 
 // Gaussian momenta p_a ~ N(0,1): two draws per link, Box-Muller pairs;
@@ -364,14 +364,21 @@ void flow_stage(const mgq_lattice* lat, void* B, double cB, double aB, void* Y, 
     });
 }
 
-mgq_status exp_update(const mgq_lattice* lat, void* B, double s, cudaStream_t st) {
+mgq_status force_two(const mgq_lattice* lat, void* B, double cB, void* Y, double cY, cudaStream_t st) {
+    flow_stage(lat, B, cB, 0.0, Y, cY, 0.0, nullptr, st);
+    return cuda_check("force");
+}
+
+mgq_status exp_update_to(const mgq_lattice* lat, void* links_out, void* B, double s, cudaStream_t st) {
     const Geom g = make_geom(lat->dims);
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
-        launch_pdl(k_exp_update<T, NP>, dim3(nblk(g.Vh, 128), 8), 128, st, links_of<T, NP>(lat), g,
-                   alg_at<T>(B, lat->dims), (T)s);
+        launch_pdl(k_exp_update<T, NP>, dim3(nblk(g.Vh, 128), 8), 128, st, links_of<T, NP>(lat),
+                   links_at<T, NP>(links_out, lat->dims), g, alg_at<T>(B, lat->dims), (T)s);
     });
     return cuda_check("exp_update");
 }
+
+mgq_status exp_update(const mgq_lattice* lat, void* B, double s, cudaStream_t st) { return exp_update_to(lat, lat->links, B, s, st); }
 
 static mgq_status kinetic_into(const mgq_lattice* lat, double* dev_out, cudaStream_t st) {
     const Geom g = make_geom(lat->dims);

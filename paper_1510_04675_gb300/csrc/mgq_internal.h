@@ -87,12 +87,16 @@ static_assert(sizeof(FlowCtl) <= 16 * sizeof(double), "control block must fit 16
 // With t the algebra coefficients of TA(U A) at the lattice's links:
 // B <- alpha B + coef t (alpha == 0 writes without reading B)
 mgq_status force_accumulate(const mgq_lattice* lat, void* B, double coef, double alpha, cudaStream_t st);
+// B <- cB t and Y <- cY t
+mgq_status force_two(const mgq_lattice* lat, void* B, double cB, void* Y, double cY, cudaStream_t st);
 // A stage of an adaptive-flow trial, z = -h t with h of the control block: B <- aB B +
 // cB z and, if cY != 0, Y <- aY Y + cY z; nothing when the trial is not active.
 void flow_stage(const mgq_lattice* lat, void* B, double cB, double aB, void* Y, double cY, double aY, const FlowCtl* ctl,
                 cudaStream_t st);
 // U <- exp(s B) U on every link
 mgq_status exp_update(const mgq_lattice* lat, void* B, double s, cudaStream_t st);
+// links_out <- exp(s B) U
+mgq_status exp_update_to(const mgq_lattice* lat, void* links_out, void* B, double s, cudaStream_t st);
 // E (site average) and Q of the clover field strength into dev_out[0], dev_out[1]
 mgq_status clover_into(const mgq_lattice* lat, double* partials, double* dev_out, cudaStream_t st);
 // Per-block E and Q partial sums (E at partials[0..nb), Q at partials[nb..2nb)) of
