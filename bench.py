@@ -773,7 +773,7 @@ def run_mgq(args, dims, world, rank, local):
         "clocks": clocks,
         "launch_shapes": {"threads_per_block": {"heatbath": tune.STAGED_THREADS, "overrelax": tune.STAGED_THREADS}
                           if args.prec == "f32c12" and V // 2 >= tune.STAGED_MIN_VH else launch_shapes,
-                          "tuned_by": "fixed: staged FP32 12-real sub-sweeps (V/2 >= 49152)"
+                          "tuned_by": f"fixed: staged FP32 12-real sub-sweeps (V/2 >= {tune.STAGED_MIN_VH})"
                           if args.prec == "f32c12" and V // 2 >= tune.STAGED_MIN_VH else "paper_1510_04675_gb300.tune"},
     }
     if clocks and clocks.get("sm_mhz"):

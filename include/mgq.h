@@ -108,14 +108,13 @@ uint64_t mgq_workspace_bytes(const mgq_lattice* lat);
  * (heat bath and overrelaxation) of the single-lattice and the batched entry
  * points and of the APE step of the prolongation: 32, 64, 96 or 128 (the
  * kernels are compiled for at most 128); 128 by default.  Results do not
- * depend on it (one thread per link or per active bond).  FP32 12-real
- * sub-sweeps of the batched driver, and of single lattices with V/2 >= 49152,
- * stage their staple links through shared memory and always run 128 threads
- * per block; the setting applies to the other launches, except single-lattice
- * FP64 sub-sweeps of too few links to fill the chip with one thread each, which
- * run several lanes per link in blocks of 128.  The force kernel's shape is structural (eight warps cover the
- * eight (mu, parity) planes of a 32-site band) and not tuned.  Process-wide setting; change it only while no
- * call is being issued.  Set by the autotuner (paper_1510_04675_gb300/tune.py). */
+ * depend on it.  It applies where a thread holds a link (or an active bond):
+ * FP32 12-real sub-sweeps, which stage their links through shared memory in blocks
+ * of 128, and single-lattice sub-sweeps of too few links to fill the chip with a
+ * thread each (FP64; FP32 below V/2 = 40960, 12-real below 65536), which run several
+ * lanes or warps per link, have shapes of their own.  The force kernels' shapes are
+ * structural and not tuned.  Process-wide setting; change it only while no call is
+ * being issued.  Set by the autotuner (paper_1510_04675_gb300/tune.py). */
 typedef enum {
     MGQ_KERNEL_HEATBATH = 0,
     MGQ_KERNEL_OVERRELAX = 1,

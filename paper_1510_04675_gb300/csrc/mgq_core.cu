@@ -8,6 +8,7 @@
 #include "mgq_internal.h"
 #include "mgq_stencil.cuh"
 #include "mgq_columns.cuh"
+#include "mgq_terms.cuh"
 
 namespace mgq {
 
@@ -450,6 +451,33 @@ static int launch_columns(int lanes, mgq_lattice* lat, const Geom& g, int mu, in
     return nb;
 }
 
+// FP32 sub-sweeps with the staple's terms shared among warps (k_update_terms): 6 or 3
+// warps per 32 links, 0 for the kernels with a thread per link.  Six warps give the
+// shortest chain, three hold more links per SM; a thread per link wins once it fills
+// the SMs, for 18-real links from about 49152 links on (one wave of its blocks: 7.8
+// against 8.3 us per overrelaxation launch), for 12-real ones, whose one-thread form
+// stages its links, from about 73728 (10.0 against 10.5 us; at 49152 9.8 against 8.3).
+// Several attempts per subgroup, or recorded decisions, run a thread per link.
+static int term_warps(const mgq_lattice* lat, const Geom& g) {
+    if (lat->prec == MGQ_F64) return 0;
+    if (g.Vh < 16384) return 6;
+    return g.Vh < (lat->prec == MGQ_F32 ? 40960 : 65536) ? 3 : 0;
+}
+
+// returns the number of blocks
+template <int KIND>
+static int launch_terms(int warps, mgq_lattice* lat, const Geom& g, int mu, int par, double beta, const RngKey& rk,
+                        double* partials, cudaStream_t st) {
+    const int nb = nblk(g.Vh, TERMS_LINKS);
+    if (lat->prec == MGQ_F32)
+        launch_pdl(warps == 6 ? k_update_terms<9, KIND, 6> : k_update_terms<9, KIND, 3>, nb, warps * TERMS_LINKS, st,
+                   links_of<float, 9>(lat), g, mu, par, (float)beta, rk, partials);
+    else
+        launch_pdl(warps == 6 ? k_update_terms<6, KIND, 6> : k_update_terms<6, KIND, 3>, nb, warps * TERMS_LINKS, st,
+                   links_of<float, 6>(lat), g, mu, par, (float)beta, rk, partials);
+    return nb;
+}
+
 mgq_status heatbath_subsweep(mgq_lattice* lat, double beta, uint64_t sweep, int n_hb, int mu, int par,
                              uint8_t* dec, cudaStream_t st) {
     Trace trace("heatbath_subsweep");
@@ -460,21 +488,19 @@ mgq_status heatbath_subsweep(mgq_lattice* lat, double beta, uint64_t sweep, int 
         launch_columns<true>(lanes, lat, g, mu, par, beta, rk, n_hb, dec, nullptr, st);
         return cuda_check("mgq_heatbath");
     }
+    if (const int warps = n_hb == 1 && !dec ? term_warps(lat, g) : 0) {
+        launch_terms<TERMS_HEATBATH>(warps, lat, g, mu, par, beta, rk, nullptr, st);
+        return cuda_check("mgq_heatbath");
+    }
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
         dispatch_mu(mu, [&]<int MU>() {
-            if constexpr (sizeof(T) == 4 && NP == 6) {
-                if (n_hb == 1 && !dec && g.Vh >= STAGED_MIN_VH) {
-                    launch_pdl_smem(k_heatbath_staged<MU>, nblk(g.Vh, STAGED_THREADS), STAGED_THREADS, STAGED_SMEM, st,
-                                    links_of<T, NP>(lat), g, par, (float)beta, rk);
-                    return;
-                }
-            }
-            if (n_hb == 1 && !dec)
-                launch_pdl(k_heatbath<T, NP, MU, true>, nblk(g.Vh, bs), bs, st, links_of<T, NP>(lat), g, par,
-                           (T)beta, rk, n_hb, dec);
+            if (n_hb != 1 || dec)
+                launch_pdl(k_heatbath<T, NP, MU, false>, nblk(g.Vh, bs), bs, st, links_of<T, NP>(lat), g, par, (T)beta, rk, n_hb, dec);
+            else if constexpr (NP == 6)
+                launch_pdl_smem(k_heatbath_staged<MU>, nblk(g.Vh, STAGED_THREADS), STAGED_THREADS, STAGED_SMEM, st,
+                                links_of<T, NP>(lat), g, par, (float)beta, rk);
             else
-                launch_pdl(k_heatbath<T, NP, MU, false>, nblk(g.Vh, bs), bs, st, links_of<T, NP>(lat), g, par,
-                           (T)beta, rk, n_hb, dec);
+                launch_pdl(k_heatbath<T, NP, MU, true>, nblk(g.Vh, bs), bs, st, links_of<T, NP>(lat), g, par, (T)beta, rk, n_hb, dec);
         });
     });
     return cuda_check("mgq_heatbath");
@@ -488,11 +514,15 @@ mgq_status overrelax_subsweep(mgq_lattice* lat, int mu, int par, cudaStream_t st
         launch_columns<false>(lanes, lat, g, mu, par, 0.0, RngKey{}, 0, nullptr, nullptr, st);
         return cuda_check("mgq_overrelax");
     }
+    if (const int warps = term_warps(lat, g)) {
+        launch_terms<TERMS_OVERRELAX>(warps, lat, g, mu, par, 0.0, RngKey{}, nullptr, st);
+        return cuda_check("mgq_overrelax");
+    }
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
         dispatch_mu(mu, [&]<int MU>() {
-            if (sizeof(T) == 4 && NP == 6 && g.Vh >= STAGED_MIN_VH)
+            if constexpr (NP == 6)
                 launch_pdl_smem(k_overrelax_staged<MU>, nblk(g.Vh, STAGED_THREADS), STAGED_THREADS, STAGED_SMEM, st,
-                                links_of<float, 6>(lat), g, par);
+                                links_of<T, NP>(lat), g, par);
             else
                 launch_pdl(k_overrelax<T, NP, MU>, nblk(g.Vh, bs), bs, st, links_of<T, NP>(lat), g, par);
         });
@@ -509,8 +539,7 @@ mgq_status overrelax_sweep_plaquette(mgq_lattice* lat, double* dev_out, cudaStre
             if ((s = overrelax_subsweep(lat, mu, par, st))) return s;
     Trace trace("overrelax_last");
     const Geom g = make_geom(lat->dims);
-    const bool staged = lat->prec == MGQ_F32_C12 && g.Vh >= STAGED_MIN_VH;
-    const int bs = staged ? STAGED_THREADS : g_block[MGQ_KERNEL_OVERRELAX][lat->prec];
+    const int bs = lat->prec == MGQ_F32_C12 ? STAGED_THREADS : g_block[MGQ_KERNEL_OVERRELAX][lat->prec];
     double* partials = reinterpret_cast<double*>(ws_alg(lat));  // free during sweeps; >= 2 nb doubles
     if (const int lanes = lat->prec == MGQ_F64 ? update_lanes(g.Vh) : 1; lanes > 1) {
         int n = 0;
@@ -519,12 +548,19 @@ mgq_status overrelax_sweep_plaquette(mgq_lattice* lat, double* dev_out, cudaStre
         launch_final_sum(partials, n, 1.0 / (18.0 * (double)g.V), dev_out, st);
         return cuda_check("overrelax_sweep_plaquette");
     }
+    if (const int warps = term_warps(lat, g)) {
+        int n = 0;
+        for (int par = 0; par < 2; par++)
+            n += launch_terms<TERMS_OVERRELAX_LAST>(warps, lat, g, 3, par, 0.0, RngKey{}, partials + n, st);
+        launch_final_sum(partials, n, 1.0 / (18.0 * (double)g.V), dev_out, st);
+        return cuda_check("overrelax_sweep_plaquette");
+    }
     const int nb = nblk(g.Vh, bs);
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
         for (int par = 0; par < 2; par++) {
-            if (staged)
+            if constexpr (NP == 6)
                 launch_pdl_smem(k_overrelax_last_staged, nb, STAGED_THREADS, STAGED_SMEM, st,
-                                links_of<float, 6>(lat), g, par, partials + par * nb);
+                                links_of<T, NP>(lat), g, par, partials + par * nb);
             else
                 launch_pdl(k_overrelax_last<T, NP>, nb, bs, st, links_of<T, NP>(lat), g, par, partials + par * nb);
         }

@@ -85,11 +85,8 @@ __device__ __forceinline__ M3<T> staple_two_row(const LinkField& U, const Geom& 
 // it completes (A += up, A += dn).  sm: (2 stages x 3 links + 1) x 3 pair-planes
 // x STAGED_THREADS float4 (STAGED_SMEM bytes per block of STAGED_THREADS
 // threads), each thread using its own column; the fixed block size keeps every
-// slot address a constant offset from one base.  Single-lattice sub-sweeps use
-// it from STAGED_MIN_VH links per launch on: below about a wave of blocks the
-// serial half-term pipeline of each thread is not hidden by other warps.
+// slot address a constant offset from one base.
 constexpr int STAGED_THREADS = 128;
-constexpr int STAGED_MIN_VH = 49152;
 constexpr int STAGED_SMEM = (2 * 3 + 1) * 3 * 16 * STAGED_THREADS;
 
 __device__ __forceinline__ void cp_async16(float4* smem, const float4* gmem) {

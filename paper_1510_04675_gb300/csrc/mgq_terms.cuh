@@ -1,0 +1,95 @@
+// FP32 sub-sweeps of small lattices with a staple term per warp.
+//
+// A thread that does a whole link runs some 2000 instructions one after the other;
+// a launch over fewer links than the chip has threads for is as slow as that chain
+// and its six dependent rounds of loads.  Here a block of WARPS = 6 or 3 warps holds
+// 32 links: the six half-terms of their staples (the upper or the lower product of
+// one direction, all of its loads at once) are shared among the warps, left in
+// shared memory, and warp 0 adds the six in staple_two_row's order and updates the
+// links.  The products, the order of the additions and the update are those of the
+// one-thread form, so both agree bit for bit.  FP32 12-real, heat bath and
+// overrelaxation per launch: 8^4 6.6 and 3.8 -> 3.6 and 2.8 us, 12^4 8.0 and 6.3 -> 5.1
+// and 4.2 us (six warps); 16^4 9.6 and 6.6 -> 7.4 and 6.5 us (three).
+#pragma once
+
+#include "mgq_stencil.cuh"
+
+namespace mgq {
+
+constexpr int TERMS_LINKS = 32;  // per block
+
+// half-term w of the staple of U_mu(x), as in staple_two_row: direction w / 2 of
+// those other than mu, upper (even w) or lower
+template <int NP>
+__device__ __forceinline__ M3<float> staple_half_term(const Links<float, NP>& U, const Hops& H, int mu, int par, int w) {
+    const int op = par ^ 1, i = w >> 1, nu = i < mu ? i : i + 1;
+    const int fmu = pick(H.fwd, mu);
+    M3<float> r;
+    if ((w & 1) == 0) {
+        r = up_term(U.load_rows(nu, op, (H.lex + fmu) >> 1), U.load(mu, op, (H.lex + pick(H.fwd, nu)) >> 1), U.load(nu, par, H.lex >> 1));
+    } else {
+        const int b = pick(H.bwd, nu), hmn = (H.lex + b) >> 1;
+        r = down_term(U.load_rows(mu, op, hmn), U.load(nu, par, (H.lex + fmu + b) >> 1), U.load(nu, op, hmn));
+    }
+    return r;
+}
+
+enum { TERMS_HEATBATH = 0, TERMS_OVERRELAX = 1, TERMS_OVERRELAX_LAST = 2 };
+
+// One (mu, par) sub-sweep: the single-attempt heat bath (a subgroup's draws taken by
+// each of warps 0 to 2 after its terms), overrelaxation, or the direction-3
+// overrelaxation that also measures plaquettes as k_overrelax_last does (the planes
+// of directions 0, 1, 2 shared among the warps from 1 on; one partial sum per block).
+template <int NP, int KIND, int WARPS>
+__global__ void __launch_bounds__(WARPS * TERMS_LINKS, 24 / WARPS) k_update_terms(Links<float, NP> U, Geom g, int mu, int par, float beta, RngKey rk,
+                                                                   double* __restrict__ partials) {
+    __shared__ float2 term[6][9][TERMS_LINKS];
+    __shared__ uint4 words[3][TERMS_LINKS];
+    pdl_launch_dependents();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int h0 = blockIdx.x * TERMS_LINKS + lane, h = h0 < g.Vh ? h0 : g.Vh - 1;
+    int x[4];
+    cb_coords(g, par, h, x);
+    const Hops H = make_hops(g, x);
+    pdl_wait();
+    M3<float> u;
+    if (w == 0) u = U.load(mu, par, h);
+#pragma unroll 1
+    for (int k = w * (6 / WARPS); k < (w + 1) * (6 / WARPS); k++) {
+        const M3<float> t = staple_half_term(U, H, mu, par, k);
+#pragma unroll
+        for (int e = 0; e < 9; e++) term[k][e][lane] = make_float2(t.e[e / 3][e % 3].re, t.e[e / 3][e % 3].im);
+    }
+    if (KIND == TERMS_HEATBATH && w < 3)
+        words[w][lane] = draw(rk, (uint32_t)H.lex, (uint32_t)mu, (uint32_t)w, 0u, KIND_HB);
+    __syncthreads();
+    double acc = 0.0;
+    if (w == 0) {
+        M3<float> A;
+#pragma unroll
+        for (int e = 0; e < 9; e++) {
+            float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 6; k++) s = __fadd2_rn(s, term[k][e][lane]);
+            A.e[e / 3][e % 3] = mk(s.x, s.y);
+        }
+        if (KIND == TERMS_OVERRELAX_LAST && par == 1 && h0 < g.Vh) acc = (double)retr_nn(u, A);
+        if constexpr (KIND == TERMS_HEATBATH) {
+            const uint4 r[3] = {words[0][lane], words[1][lane], words[2][lane]};
+            hb_link_drawn(u, A, beta, r);
+        } else {
+            or_link(u, A);
+        }
+        if (h0 < g.Vh) U.store(mu, par, h, u);
+    } else if (KIND == TERMS_OVERRELAX_LAST && h0 < g.Vh) {
+        // planes 01, 02, 12
+        for (int p = w - 1; p < 3; p += WARPS - 1)
+            acc += (double)loop_retr(U, H, par, par ^ 1, p == 2 ? 1 : 0, p == 0 ? 1 : 2);
+    }
+    if constexpr (KIND == TERMS_OVERRELAX_LAST) {
+        acc = block_sum(acc);
+        if (threadIdx.x == 0) partials[blockIdx.x] = acc;
+    }
+}
+
+}  // namespace mgq

@@ -21,7 +21,7 @@ from ._lib import MGQ_KERNEL_HEATBATH, MGQ_KERNEL_OVERRELAX, call
 
 CANDIDATES = (32, 64, 96, 128)
 STAGED_THREADS = 128  # block size of the staged FP32 12-real sub-sweeps (not tunable)
-STAGED_MIN_VH = 49152  # single-lattice FP32 12-real sub-sweeps are staged from V/2 >= this on
+STAGED_MIN_VH = 65536  # single-lattice FP32 12-real sub-sweeps are staged from V/2 >= this on
 _KERNELS = {"heatbath": MGQ_KERNEL_HEATBATH, "overrelax": MGQ_KERNEL_OVERRELAX, "heatbath_batched": 2,
             "overrelax_batched": 3, "ape": 4}
 
