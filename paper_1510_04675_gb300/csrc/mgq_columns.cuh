@@ -15,9 +15,8 @@
 //     exchange the four entries of V's block, and the rotation's scalars are
 //     computed by all lanes of a link;
 //   - the reunitarisation exchanges norms, inner products and row entries.
-// One compound sweep (1 heat bath + 4 overrelaxation) of 8^4: 3.77 -> 0.94 ms (an
-// overrelaxation launch 94 -> 21 us, a heat bath 118 -> 40 us); the force of 8^3x12
-// 95 -> 83 us.
+// One compound sweep (1 heat bath + 4 overrelaxation) of 8^4: 3.75 -> 0.90 ms (an
+// overrelaxation launch 94 -> 20 us, a heat bath 118 -> 38 us).
 // Every operation and its order are those of the one-thread form (staple_full,
 // hb_link, or_link), so both agree bit for bit.
 #pragma once
@@ -27,7 +26,11 @@
 
 namespace mgq {
 
-constexpr int COL_THREADS = 128;
+// One warp per block: the blocks then spread over the SMs one warp at a time (8^4: 410
+// warps, three to an SM, where blocks of four fill 103 SMs; four warps of an SM share
+// its FP64 rate, 76 cycles an operation each instead of 64): 8^4 compound sweep 0.94 ->
+// 0.90 ms, 10-step trajectory on 8^3x12 1.28 -> 1.18 ms.
+constexpr int COL_THREADS = 32;
 
 // the lanes of a link: k the lane's column, half its staple terms (0 upper, 1
 // lower) when LPL = 6, base the lane of column 0 in its half
@@ -159,13 +162,20 @@ __global__ void __launch_bounds__(COL_THREADS) k_update_columns(Links<double, 9>
     const int h = h0 < g.Vh ? h0 : g.Vh - 1;
     int x[4];
     cb_coords(g, par, h, x);
+    const int lex = lex_of(g, x);
+    // heat bath: lane k draws subgroup k's first attempt and its direction for all
+    uint4 words;
+    double ct, st, sp, cp;
+    if constexpr (HB) {
+        words = draw(rk, (uint32_t)lex, (uint32_t)mu, (uint32_t)c.k, 0u, KIND_HB);
+        creutz_direction(words, &ct, &st, &sp, &cp);
+    }
     pdl_wait();
     Cx<double> A[3], u[3], v[3];
     staple_column<LPL>(U, g, x, h, mu, par, c, A);
     left_column(U.base(mu, par, h), A, c.k, u, v);
     double acc = 0.0;
     if (!HB && par == 1) acc = c.k == 0 ? v[0].re : (c.k == 1 ? v[1].re : v[2].re);  // Re Tr(U A), kept by the update
-    const int lex = lex_of(g, x);
     // six lanes: the lower half carries V through the rotations, the upper half U
     if (LPL == 6 && c.half == 0) {
 #pragma unroll
@@ -180,10 +190,16 @@ __global__ void __launch_bounds__(COL_THREADS) k_update_columns(Links<double, 9>
         bool turn = false;
         if constexpr (HB) {
             const double xi = m_sqrt(quat_norm2(w));
+            const int src = vbase + s;  // the lane that drew for this subgroup
+            const uint32_t wx = __shfl_sync(0xffffffffu, words.x, src), wy = __shfl_sync(0xffffffffu, words.y, src);
+            const double cts = __shfl_sync(0xffffffffu, ct, src), sts = __shfl_sync(0xffffffffu, st, src),
+                         sps = __shfl_sync(0xffffffffu, sp, src), cps = __shfl_sync(0xffffffffu, cp, src);
             uint8_t d = 255;
             if (xi >= tiny_norm<double>()) {
                 const double k = creutz_k(beta, xi), em = creutz_em(k);
-                for (int att = 0; att < n_hb && !turn; att++) {
+                turn = creutz_rotation(w, xi, k, em, wx, wy, cts, sts, sps, cps, R);
+                if (turn) d = 0;
+                for (int att = 1; att < n_hb && !turn; att++) {
                     turn = creutz_draw(w, xi, k, em, draw(rk, (uint32_t)lex, (uint32_t)mu, (uint32_t)s, (uint32_t)att, KIND_HB), R);
                     if (turn) d = (uint8_t)att;
                 }

@@ -372,7 +372,8 @@ mgq_status force_two(const mgq_lattice* lat, void* B, double cB, void* Y, double
 mgq_status exp_update_to(const mgq_lattice* lat, void* links_out, void* B, double s, cudaStream_t st) {
     const Geom g = make_geom(lat->dims);
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
-        launch_pdl(k_exp_update<T, NP>, dim3(nblk(g.Vh, 128), 8), 128, st, links_of<T, NP>(lat),
+        constexpr int kThreads = sizeof(T) == 8 ? 32 : 128;  // FP64: spread warp by warp, see COL_THREADS
+        launch_pdl(k_exp_update<T, NP>, dim3(nblk(g.Vh, kThreads), 8), kThreads, st, links_of<T, NP>(lat),
                    links_at<T, NP>(links_out, lat->dims), g, alg_at<T>(B, lat->dims), (T)s);
     });
     return cuda_check("exp_update");

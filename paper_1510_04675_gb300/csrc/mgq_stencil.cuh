@@ -533,18 +533,41 @@ template <> __device__ __forceinline__ double quat_norm2<double>(const double w[
     return fma_rn(w[3], w[3], fma_rn(w[2], w[2], fma_rn(w[1], w[1], __dmul_rn(w[0], w[0]))));
 }
 
-// One Creutz attempt with the four words r: R = X (w/|w|) and true on acceptance.
+// The direction of X from words z, w of a draw: cos, sin of theta and of phi.
+template <class T> __device__ __forceinline__ void creutz_direction(uint4 r, T* ct, T* st, T* sp, T* cp) {
+    const T u2 = u01<T>(r.z), u3 = u01<T>(r.w);
+    *ct = T(2) * u2 - T(1);
+    *st = sampler_sqrt(sub_rn(T(1), mul_rn(*ct, *ct)));
+    creutz_phi(u3, sp, cp);
+}
+
+// One Creutz attempt from words x, y of its draw and its direction: R = X (w/|w|) and
+// true on acceptance.
 template <class T>
-__device__ __forceinline__ bool creutz_draw(const T w[4], T xi, T k, T em, uint4 r, T R[4]) {
-    const T u0 = u01<T>(r.x), u1 = u01<T>(r.y), u2 = u01<T>(r.z), u3 = u01<T>(r.w);
+__device__ __forceinline__ bool creutz_rotation(const T w[4], T xi, T k, T em, uint32_t wx, uint32_t wy, T ct, T st, T sp, T cp,
+                                                T R[4]) {
+    const T u0 = u01<T>(wx), u1 = u01<T>(wy);
     const T a0 = creutz_a0(k, em, u0);
     const T rest = sub_rn(T(1), mul_rn(a0, a0));
     if (!(mul_rn(u1, u1) <= rest)) return false;
     const T rad = sampler_sqrt(rest);
-    const T ct = T(2) * u2 - T(1);
-    const T st = sampler_sqrt(sub_rn(T(1), mul_rn(ct, ct)));
-    T sp, cp;
-    creutz_phi(u3, &sp, &cp);
+    const T X[4] = {a0, rad * st * cp, rad * st * sp, rad * ct};
+    const T inv = recip(xi);
+    const T wh[4] = {w[0] * inv, w[1] * inv, w[2] * inv, w[3] * inv};
+    qmul(X, wh, R);
+    return true;
+}
+
+// The same with the four words r.
+template <class T>
+__device__ __forceinline__ bool creutz_draw(const T w[4], T xi, T k, T em, uint4 r, T R[4]) {
+    const T u0 = u01<T>(r.x), u1 = u01<T>(r.y);
+    const T a0 = creutz_a0(k, em, u0);
+    const T rest = sub_rn(T(1), mul_rn(a0, a0));
+    if (!(mul_rn(u1, u1) <= rest)) return false;
+    const T rad = sampler_sqrt(rest);
+    T ct, st, sp, cp;
+    creutz_direction(r, &ct, &st, &sp, &cp);
     const T X[4] = {a0, rad * st * cp, rad * st * sp, rad * ct};
     const T inv = recip(xi);
     const T wh[4] = {w[0] * inv, w[1] * inv, w[2] * inv, w[3] * inv};
