@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, NHB1 ? batch_blocks<T, NP>() : 
         hb_link_drawn(u, A, d.beta, r);
     } else {
         staple_and_link<T, NP, MU>(U, g, x, h, par, A, u);
-        hb_link(u, A, d.beta, n_hb, rk, lex, (uint32_t)MU, (uint8_t*)nullptr);
+        hb_link<(NP == 9)>(u, A, d.beta, n_hb, rk, lex, (uint32_t)MU, (uint8_t*)nullptr);
     }
     U.store(MU, par, h, u);
 }
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, batch_blocks<T, NP>()) k_overre
     cb_coords(g, par, h, x);
     M3<T> A, u;
     staple_and_link<T, NP, MU>(U, g, x, h, par, A, u);
-    or_link(u, A);
+    or_link<(NP == 9)>(u, A);
     U.store(MU, par, h, u);
 }
 
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, sizeof(T) == 8 ? 2 : 4)
         M3<T> A, u;
         staple_and_link<T, NP, 3>(U, g, x, h, par, A, u);
         if (par == 1) acc = (double)retr_nn(u, A);
-        or_link(u, A);
+        or_link<(NP == 9)>(u, A);
         U.store(3, par, h, u);
         acc += site_plaquettes<T, NP, 3>(U, g, par, h);
     }

@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 4) k_heatbath(Links<
     const M3<T> A = staple(U, g, x, h, MU, par);
     M3<T> u = U.load(MU, par, h);
     const int lex = lex_of(g, x);
-    hb_link(u, A, beta, n_hb, rk, (uint32_t)lex, (uint32_t)MU, dec ? dec + ((size_t)lex * 4 + MU) * 3 : nullptr);
+    hb_link<true>(u, A, beta, n_hb, rk, (uint32_t)lex, (uint32_t)MU, dec ? dec + ((size_t)lex * 4 + MU) * 3 : nullptr);
     U.store(MU, par, h, u);
 }
 
@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 4) k_overrelax(Links
     if (h >= g.Vh) return;
     const M3<T> A = staple(U, g, x, h, MU, par);
     M3<T> u = U.load(MU, par, h);
-    or_link(u, A);
+    or_link<true>(u, A);
     U.store(MU, par, h, u);
 }
 
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 4)
         const M3<T> A = staple(U, g, x, h, 3, par);
         M3<T> u = U.load(3, par, h);
         if (par == 1) acc = (double)retr_nn(u, A);
-        or_link(u, A);
+        or_link<true>(u, A);
         U.store(3, par, h, u);
         acc += site_plaquettes<T, NP, 3>(U, g, par, h);
     }

@@ -41,7 +41,7 @@ __device__ __forceinline__ M3<T> su3_project(const M3<T>& M) {
                 const float inv = rsqrtf(n2);
                 const float r[4] = {w[0] * inv, w[1] * inv, w[2] * inv, w[3] * inv};
                 moved = moved || fabsf(r[1]) > 1e-6f || fabsf(r[2]) > 1e-6f || fabsf(r[3]) > 1e-6f;
-                su2_rows(W, i, j, r, true, true, 7, 7);
+                su2_rows_packed(W, i, j, r, true, true, 7, 7);
             } else {
                 const T xi = m_sqrt(n2);
                 if (!(xi >= tiny_norm<T>())) continue;
@@ -111,6 +111,7 @@ static_assert(sizeof(ProlongCtl) == 64, "control block layout");
 
 constexpr int PB_CHUNK = 64;       // lattices per launch (kernel-parameter table)
 constexpr int PB_THREADS = 128;
+constexpr int PB_BLOCKS = 5;       // resident per SM (FP32); six: 48 lattices 20.2 against 20.4 ms, 8^4 -> 16^4 11.5 against 11.2
 constexpr int PB_SD_LANES = 256;  // partial-action lanes per block (any block size)
 constexpr int PB_SD_MAXBLK = 512;  // partial-action blocks per lattice
 
@@ -279,10 +280,10 @@ __device__ __forceinline__ void ape_bond(const ProDesc<T>& D, T c, int k, int t,
         if constexpr (sizeof(T) == 4) {
             // products of SU(3) factors in two-row form, the third row rebuilt
             tp = mul_nd_2(mul_nn_2(Uin.load_rows(nu, par, h), Uin.load(mu, op, lpn >> 1)), Uin.load(nu, op, lpm >> 1));
-            rebuild_row2(tp);
+            rebuild_row2_packed(tp);
             tm = mul_nn_2(mul_dn_2(Uin.load(nu, op, lmn >> 1), Uin.load(mu, op, lmn >> 1)),
                           Uin.load(nu, par, lmn_pm >> 1));
-            rebuild_row2(tm);
+            rebuild_row2_packed(tm);
         } else {
             tp = mul_nd(mul_nn(Uin.load(nu, par, h), Uin.load(mu, op, lpn >> 1)), Uin.load(nu, op, lpm >> 1));
             tm = mul_nn(mul_dn(Uin.load(nu, op, lmn >> 1), Uin.load(mu, op, lmn >> 1)), Uin.load(nu, par, lmn_pm >> 1));
@@ -380,7 +381,7 @@ __device__ __forceinline__ double lanes_sum(const double* lanes) {
 // |S_d(k) - S_d(k-1)| <= rel_tol |S_d(k-1)| or k = max_iter (rel_tol <= 0:
 // exactly max_iter steps), else the step it has just taken becomes the newest.
 template <class T, int NP>
-__global__ void __launch_bounds__(PB_THREADS, sizeof(T) == 8 ? 1 : 5) k_iter_pb(const __grid_constant__ PBatch<T> B) {
+__global__ void __launch_bounds__(PB_THREADS, sizeof(T) == 8 ? 1 : PB_BLOCKS) k_iter_pb(const __grid_constant__ PBatch<T> B) {
     pdl_launch_dependents();
     pdl_wait();  // the state and the fields come from the previous launch
     const int nSall = B.sprefix[B.n];
@@ -400,15 +401,19 @@ __global__ void __launch_bounds__(PB_THREADS, sizeof(T) == 8 ? 1 : 5) k_iter_pb(
     if (sd_role) {
         const int np = n_plaqs(D.gc, d);
         for (int v = threadIdx.x; v < PB_SD_LANES; v += blockDim.x) {
+            // Re Tr summed in FP64, the thirds taken once per lane (an FP64 division per
+            // plaquette is ten FP64 operations of 64 cycles each on this part)
             double acc = 0.0;
+            int count = 0;
             for (int t = b * PB_SD_LANES + v; t < np; t += nS * PB_SD_LANES) {
                 int mu, nu, x[4];
                 plaq_of(D.gc, d, t, mu, nu, x);
                 const int par = (x[0] + x[1] + x[2] + x[3]) & 1, h = lex_of(g, x) >> 1, op = par ^ 1;
                 const int hpm = lex_hop(g, x, mu, +1) >> 1, hpn = lex_hop(g, x, nu, +1) >> 1;
-                acc += 1.0 - (double)plaq_retr(Uin, mu, nu, par, op, h, hpm, hpn) / 3.0;
+                acc += (double)plaq_retr(Uin, mu, nu, par, op, h, hpm, hpn);
+                count++;
             }
-            lanes[v] = acc;
+            lanes[v] = (double)count - acc / 3.0;
         }
         __syncthreads();
         const double sb = lanes_sum(lanes);
@@ -486,13 +491,20 @@ __global__ void __launch_bounds__(PB_THREADS) k_finish_pb(const __grid_constant_
 
 static inline int nblk(long n, int t) { return (int)((n + t - 1) / t); }
 
-// partial-action blocks of one lattice: one block per 1024 plaquettes (four per
-// lane) of the largest set (48 V_c = 3 V) for a lattice alone, up to
-// PB_SD_MAXBLK; in a call over many lattices the lattice's share of about 4096
-// blocks, so that the blocks stay large when there is parallelism across lattices
+// partial-action blocks of one lattice.  A block takes 256 lanes of plaquettes from
+// the largest set (48 V_c = 3 V), k a lane, one after the other: k = 1 while the
+// lattice's blocks and bonds leave three quarters of the chip's places free, k = 2
+// while they fit in one wave, else 4 (8^4 -> 16^4), up to PB_SD_MAXBLK; a small lattice
+// alone waits for these chains (4^4 -> 8^4 with the 0.001 % rule 7.4 -> 6.2 ms with k =
+// 1, 4x6x4x8 9.1 -> 8.4 ms).  In a call over many lattices at most the lattice's share
+// of about 2048 blocks, so that the blocks stay large when there is parallelism
+// across lattices (48 lattices of 8^3x16 to 16^4, 20 steps a stage: 21.8 ms with a
+// share of 4096, 20.4 ms).
 static int sd_blocks(const Geom& g, double total_sites) {
-    const long full = nblk(3L * g.V, 4 * PB_SD_LANES);
-    long b = (long)((4096.0 * g.V + total_sites - 1.0) / total_sites);
+    const long wave = 152L * PB_BLOCKS, bonds = nblk(3L * g.V / 2, PB_THREADS);
+    auto blocks = [&](int k) { return (long)nblk(3L * g.V, k * PB_SD_LANES); };
+    const long full = 4 * (blocks(1) + bonds) <= wave ? blocks(1) : blocks(2) + bonds <= wave ? blocks(2) : blocks(4);
+    long b = (long)((2048.0 * g.V + total_sites - 1.0) / total_sites);
     if (b > full) b = full;
     if (b > PB_SD_MAXBLK) b = PB_SD_MAXBLK;
     return b < 1 ? 1 : (int)b;

@@ -23,6 +23,12 @@ template <bool FMA = false> __device__ __forceinline__ M3<float> mul_dn_2(const 
     return two_rows<FMA, true, false>(a, b);
 }
 
+// row 2 of a product of SU(3) factors, in either form
+template <bool PACKED = false> __device__ __forceinline__ void complete(M3<float>& m) {
+    if constexpr (PACKED) rebuild_row2_packed(m);
+    else rebuild_row2(m);
+}
+
 // =============================================================== staple
 // A_mu(x) = sum_{nu != mu} [ U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+
 //                          + U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu) ]
@@ -37,14 +43,14 @@ template <bool FMA = false> __device__ __forceinline__ M3<float> mul_dn_2(const 
 // (the left factor) is never completed.
 //   up = (a b^+) c^+            a = U_nu(x+mu), b = U_mu(x+nu), c = U_nu(x)
 //   dn = (e d)^+ f              d = U_nu(x+mu-nu), e = U_mu(x-nu), f = U_nu(x-nu)
-template <class T, class LinkField>
-__device__ __forceinline__ M3<T> staple_two_row(const LinkField& U, const Geom& g, const int x[4], int h, int mu,
+template <class LinkField>
+__device__ __forceinline__ M3<float> staple_two_row(const LinkField& U, const Geom& g, const int x[4], int h, int mu,
                                                 int par) {
-    M3<T> A;
+    M3<float> A;
 #pragma unroll
     for (int i = 0; i < 3; i++)
 #pragma unroll
-        for (int j = 0; j < 3; j++) A.e[i][j] = mk(T(0), T(0));
+        for (int j = 0; j < 3; j++) A.e[i][j] = mk(0.f, 0.f);
     const int op = par ^ 1;
     const Hops H = make_hops(g, x);
     const int fmu = pick(H.fwd, mu);
@@ -55,18 +61,18 @@ __device__ __forceinline__ M3<T> staple_two_row(const LinkField& U, const Geom& 
         const int hpn = (H.lex + H.fwd[nu]) >> 1;
         const int hmn = (H.lex + H.bwd[nu]) >> 1;
         const int hpm_mn = (H.lex + fmu + H.bwd[nu]) >> 1;
-        M3<T> up, dn;
+        M3<float> up, dn;
         {
-            M3<T> t = mul_nd_2(U.load_rows(nu, op, hpm), U.load(mu, op, hpn));
-            rebuild_row2(t);
+            M3<float> t = mul_nd_2(U.load_rows(nu, op, hpm), U.load(mu, op, hpn));
+            complete<true>(t);
             up = mul_nd_2(t, U.load(nu, par, h));
-            rebuild_row2(up);
+            complete<true>(up);
         }
         {
-            M3<T> t = mul_nn_2(U.load_rows(mu, op, hmn), U.load(nu, par, hpm_mn));
-            rebuild_row2(t);
+            M3<float> t = mul_nn_2(U.load_rows(mu, op, hmn), U.load(nu, par, hpm_mn));
+            complete<true>(t);
             dn = mul_dn_2(t, U.load(nu, op, hmn));
-            rebuild_row2(dn);
+            complete<true>(dn);
         }
         acc_add(A, up);
         acc_add(A, dn);
@@ -114,10 +120,6 @@ __device__ __forceinline__ M3<float> staged_rows(float4* sm, int stage, int j) {
         m.e[(2 * k + 1) / 3][(2 * k + 1) % 3] = mk(v.z, v.w);
     }
     return m;
-}
-template <bool PACKED = false> __device__ __forceinline__ void complete(M3<float>& m) {
-    if constexpr (PACKED) rebuild_row2_packed(m);
-    else rebuild_row2(m);
 }
 template <bool PACKED = false> __device__ __forceinline__ M3<float> staged_full(float4* sm, int stage, int j) {
     M3<float> m = staged_rows(sm, stage, j);
@@ -256,7 +258,7 @@ __device__ __forceinline__ M3<double> staple_full(const Links<double, 9>& U, con
 // products.
 template <class T, int NP>
 __device__ __forceinline__ M3<T> staple(const Links<T, NP>& U, const Geom& g, const int x[4], int h, int mu, int par) {
-    if constexpr (sizeof(T) == 4) return staple_two_row<T>(U, g, x, h, mu, par);
+    if constexpr (sizeof(T) == 4) return staple_two_row(U, g, x, h, mu, par);
     else return staple_full(U, g, x, h, mu, par);
 }
 
@@ -473,20 +475,55 @@ __device__ __forceinline__ void su2_rows<float>(M3<float>& m, int i, int j, cons
     }
 }
 
+// The same as packed FMAs on (re, im) pairs.
+__device__ __forceinline__ void su2_rows_packed(M3<float>& m, int i, int j, const float r[4], bool do_i, bool do_j, int ci,
+                                                int cj) {
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const float2 MI = make_float2(m.e[i][k].re, m.e[i][k].im), iMI = make_float2(-m.e[i][k].im, m.e[i][k].re);
+        const float2 MJ = make_float2(m.e[j][k].re, m.e[j][k].im), iMJ = make_float2(-m.e[j][k].im, m.e[j][k].re);
+        if (do_i && ((ci >> k) & 1)) {
+            float2 v = __fmul2_rn(bcast(r[0]), MI);
+            v = __ffma2_rn(bcast(r[3]), iMI, v);
+            v = __ffma2_rn(bcast(r[2]), MJ, v);
+            v = __ffma2_rn(bcast(r[1]), iMJ, v);
+            m.e[i][k] = from_f2(v);
+        }
+        if (do_j && ((cj >> k) & 1)) {
+            float2 v = __fmul2_rn(bcast(-r[2]), MI);
+            v = __ffma2_rn(bcast(r[1]), iMI, v);
+            v = __ffma2_rn(bcast(r[0]), MJ, v);
+            v = __ffma2_rn(bcast(-r[3]), iMJ, v);
+            m.e[j][k] = from_f2(v);
+        }
+    }
+}
+
+template <bool PACKED, class T>
+__device__ __forceinline__ void su2_rows_as(M3<T>& m, int i, int j, const T r[4], bool do_i, bool do_j, int ci, int cj) {
+    if constexpr (PACKED && sizeof(T) == 4) su2_rows_packed(m, i, j, r, do_i, do_j, ci, cj);
+    else su2_rows(m, i, j, r, do_i, do_j, ci, cj);
+}
+// V = U A
+template <bool PACKED, class T> __device__ __forceinline__ M3<T> link_times_staple(const M3<T>& u, const M3<T>& A) {
+    if constexpr (PACKED && sizeof(T) == 4) return x2_product<3, false, false>(u, A);
+    else return mul_nn(u, A);
+}
+
 // After the update of subgroup s: U needs rows 0, 1 (the final
 // reunitarisation rebuilds row 2) and, until s = 2, row 2 as an input; V only
 // needs the entries the later subgroups read (s = 1 reads row 0 and
 // V20, V22, s = 2 reads V11, V12, V21, V22).
-template <class T>
+template <bool PACKED = false, class T>
 __device__ __forceinline__ void apply_subgroup(M3<T>& u, M3<T>& v, int s, const T R[4]) {
     if (s == 0) {
-        su2_rows(u, 0, 1, R, true, true, 7, 7);
-        su2_rows(v, 0, 1, R, true, true, 7, 6);
+        su2_rows_as<PACKED>(u, 0, 1, R, true, true, 7, 7);
+        su2_rows_as<PACKED>(v, 0, 1, R, true, true, 7, 6);
     } else if (s == 1) {
-        su2_rows(u, 0, 2, R, true, true, 7, 7);
-        su2_rows(v, 0, 2, R, false, true, 0, 6);
+        su2_rows_as<PACKED>(u, 0, 2, R, true, true, 7, 7);
+        su2_rows_as<PACKED>(v, 0, 2, R, false, true, 0, 6);
     } else {
-        su2_rows(u, 1, 2, R, true, false, 7, 0);
+        su2_rows_as<PACKED>(u, 1, 2, R, true, false, 7, 0);
     }
 }
 
@@ -576,18 +613,22 @@ __device__ __forceinline__ bool creutz_draw(const T w[4], T xi, T k, T em, uint4
 }
 
 // the attempt on subgroup s, applied to u and v when accepted
-template <class T>
+template <bool PACKED = false, class T>
 __device__ __forceinline__ bool creutz_attempt(M3<T>& u, M3<T>& v, int s, const T w[4], T xi, T k, T em, uint4 r) {
     T R[4];
     if (!creutz_draw(w, xi, k, em, r, R)) return false;
-    apply_subgroup(u, v, s, R);
+    apply_subgroup<PACKED>(u, v, s, R);
     return true;
 }
 
-template <class T>
+// PACKED: the FP32 forms of V, the rotations and the rebuilds; the kernels that read
+// their links straight into registers use it (24^4, 18-real: heat bath 24.4 us against
+// 25.1 with single FMAs, overrelaxation 19.9 against 20.8), the staged ones and those
+// with a term per warp do not.
+template <bool PACKED = false, class T>
 __device__ __forceinline__ void hb_link(M3<T>& u, const M3<T>& A, T beta, int n_hb, const RngKey& rk, uint32_t lex,
                                         uint32_t mu, uint8_t* dec) {
-    M3<T> v = mul_nn(u, A);
+    M3<T> v = link_times_staple<PACKED>(u, A);
 #pragma unroll
     for (int s = 0; s < 3; s++) {
         const int i = (s == 2) ? 1 : 0, j = (s == 0) ? 1 : 2;
@@ -599,7 +640,7 @@ __device__ __forceinline__ void hb_link(M3<T>& u, const M3<T>& A, T beta, int n_
             const T k = creutz_k(beta, xi);
             const T em = creutz_em(k);
             for (int att = 0; att < n_hb; att++) {
-                if (creutz_attempt(u, v, s, w, xi, k, em, draw(rk, lex, mu, (uint32_t)s, (uint32_t)att, KIND_HB))) {
+                if (creutz_attempt<PACKED>(u, v, s, w, xi, k, em, draw(rk, lex, mu, (uint32_t)s, (uint32_t)att, KIND_HB))) {
                     d = (uint8_t)att;
                     break;
                 }
@@ -655,15 +696,15 @@ template <> __device__ __forceinline__ bool or_rotation<double>(const double w[4
 }
 
 // Overrelaxation of one link: per subgroup R = (w/|w|)^2; reunitarise.
-template <class T>
+template <bool PACKED = false, class T>
 __device__ __forceinline__ void or_link(M3<T>& u, const M3<T>& A) {
-    M3<T> v = mul_nn(u, A);
+    M3<T> v = link_times_staple<PACKED>(u, A);
 #pragma unroll
     for (int s = 0; s < 3; s++) {
         const int i = (s == 2) ? 1 : 0, j = (s == 0) ? 1 : 2;
         T w[4], R[4];
         block_w(v, i, j, w);
-        if (or_rotation(w, R)) apply_subgroup(u, v, s, R);
+        if (or_rotation(w, R)) apply_subgroup<PACKED>(u, v, s, R);
     }
     reunitarize(u);
 }
