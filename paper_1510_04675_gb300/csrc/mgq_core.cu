@@ -132,21 +132,50 @@ mgq_status deliver_int(const int* src, int* out, size_t n, cudaStream_t st, cons
     return deliver_t(src, out, n, st, fn);
 }
 
+mgq_status deliver_pairs(const double* dev_src, double* a_out, double* b_out, size_t n, cudaStream_t st, const char* fn) {
+    double* out[2] = {a_out, b_out};
+    bool host = false;
+    for (int k = 0; k < 2 && n > 0; k++) {
+        if (!out[k]) continue;
+        if (!is_device_ptr(out[k])) {
+            host = true;
+        } else if (cudaMemcpy2DAsync(out[k], sizeof(double), dev_src + k, 2 * sizeof(double), sizeof(double), n,
+                                     cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
+            return cuda_check(fn);
+        } else {
+            out[k] = nullptr;  // done
+        }
+    }
+    if (!host) return MGQ_OK;
+    double buf[WS_NSCALARS];
+    const mgq_status s = deliver(dev_src, buf, 2 * n, st, fn);
+    if (s) return s;
+    for (int k = 0; k < 2; k++)
+        for (size_t i = 0; out[k] && i < n; i++) out[k][i] = buf[2 * i + k];
+    return MGQ_OK;
+}
+
 int reduction_blocks(int V, int threads) {
     int b = (V + threads - 1) / threads;
     return b < 1184 ? b : 1184;  // 152 SMs x 8
 }
 
 // =============================================================== reductions
-__global__ void k_final_sum(const double* __restrict__ partials, int n, double scale, double* out) {
+// block b sums set b
+__global__ void k_final_sum(const double* __restrict__ partials, int n, double scale0, double scale1, double* out) {
+    partials += (size_t)blockIdx.x * n;
     double v = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) v += partials[i];
     v = block_sum(v);
-    if (threadIdx.x == 0) out[0] = v * scale;
+    if (threadIdx.x == 0) out[blockIdx.x] = v * (blockIdx.x ? scale1 : scale0);
 }
 
 void launch_final_sum(const double* partials, int n, double scale, double* out, cudaStream_t st) {
-    k_final_sum<<<1, 512, 0, st>>>(partials, n, scale, out);
+    k_final_sum<<<1, 512, 0, st>>>(partials, n, scale, scale, out);
+}
+
+void launch_final_sum2(const double* partials, int n, double scale0, double scale1, double* out, cudaStream_t st) {
+    k_final_sum<<<2, 512, 0, st>>>(partials, n, scale0, scale1, out);
 }
 
 // =============================================================== fields

@@ -59,8 +59,7 @@ int clover_partials(const mgq_lattice* lat, const void* lines, int m, double* pa
 mgq_status clover_into(const mgq_lattice* lat, double* partials, double* dev_out, cudaStream_t st) {
     const Geom g = make_geom(lat->dims);
     const int nb = clover_partials(lat, lat->links, 1, partials, nullptr, st);
-    launch_final_sum(partials, nb, 1.0 / (double)g.V, dev_out, st);
-    launch_final_sum(partials + nb, nb, 1.0, dev_out + 1, st);
+    launch_final_sum2(partials, nb, 1.0 / (double)g.V, 1.0, dev_out, st);
     return cuda_check("clover");
 }
 
@@ -103,8 +102,7 @@ mgq_status mgq_topo_charge(const mgq_lattice* lat, double* E_out, double* Q_out,
     cudaStream_t st = as_stream(stream);
     double* sc = ws_scalars(lat);
     if ((s = clover_into(lat, ws_partials(lat), sc + 16, st))) return s;
-    if ((s = deliver(sc + 16, E_out, E_out ? 1 : 0, st, "mgq_topo_charge"))) return s;
-    return deliver(sc + 17, Q_out, Q_out ? 1 : 0, st, "mgq_topo_charge");
+    return deliver_pairs(sc + 16, E_out, Q_out, 1, st, "mgq_topo_charge");
 }
 
 mgq_status mgq_wilson_flow(mgq_lattice* lat, double eps, int n_steps, int meas_every, double* E_out, double* Q_out,
@@ -129,12 +127,7 @@ mgq_status mgq_wilson_flow(mgq_lattice* lat, double eps, int n_steps, int meas_e
         if (k == n_steps) break;
         if ((s = flow_step(lat, B, eps, st))) return s;
     }
-    // gather strided E, Q pairs
-    for (int i = 0; i < nm; i++) {
-        if (E_out && (s = deliver(meas + 2 * i, E_out + i, 1, st, "mgq_wilson_flow"))) return s;
-        if (Q_out && (s = deliver(meas + 2 * i + 1, Q_out + i, 1, st, "mgq_wilson_flow"))) return s;
-    }
-    return MGQ_OK;
+    return deliver_pairs(meas, E_out, Q_out, (size_t)nm, st, "mgq_wilson_flow");
 }
 
 mgq_status mgq_wilson_flow_times(mgq_lattice* lat, double t_end, double eps, const double* t_meas, int n_meas,
@@ -172,11 +165,7 @@ mgq_status mgq_wilson_flow_times(mgq_lattice* lat, double t_end, double eps, con
             i++;
         }
     }
-    for (int k = 0; k < n_meas; k++) {
-        if (E_out && (s = deliver(meas + 2 * k, E_out + k, 1, st, "mgq_wilson_flow_times"))) return s;
-        if (Q_out && (s = deliver(meas + 2 * k + 1, Q_out + k, 1, st, "mgq_wilson_flow_times"))) return s;
-    }
-    return MGQ_OK;
+    return deliver_pairs(meas, E_out, Q_out, (size_t)n_meas, st, "mgq_wilson_flow_times");
 }
 
 }  // extern "C"

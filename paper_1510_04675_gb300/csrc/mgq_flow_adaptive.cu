@@ -259,10 +259,7 @@ mgq_status mgq_wilson_flow_adaptive(mgq_lattice* lat, double t_end, double tol, 
         return fail(MGQ_EINVAL, "mgq_wilson_flow_adaptive: step size underflow (tolerance below the precision floor)");
     int cnt[3];
     if ((s = deliver_int(&c->m, cnt, 3, st, "mgq_wilson_flow_adaptive"))) return s;
-    for (int i = 0; i < cnt[0]; i++) {
-        if (E_out && (s = deliver(meas + 2 * i, E_out + i, 1, st, "mgq_wilson_flow_adaptive"))) return s;
-        if (Q_out && (s = deliver(meas + 2 * i + 1, Q_out + i, 1, st, "mgq_wilson_flow_adaptive"))) return s;
-    }
+    if ((s = deliver_pairs(meas, E_out, Q_out, (size_t)cnt[0], st, "mgq_wilson_flow_adaptive"))) return s;
     if (n_meas) *n_meas = cnt[0];
     if (n_steps) *n_steps = cnt[1];
     if (n_rejects) *n_rejects = cnt[2];

@@ -3,6 +3,8 @@
 // exponential link update, FP64 Hamiltonian, device-side Metropolis test and
 // restore, and the PQP leapfrog driver.  The force/update kernels are shared
 // with the Wilson flow (its generator is the force at beta = 6).
+#include <cstring>
+
 #include "mgq_internal.h"
 #include "mgq_stencil.cuh"
 #include "mgq_force_out.cuh"
@@ -466,6 +468,14 @@ mgq_status mgq_hmc_trajectory(mgq_lattice* lat, double beta, double tau, int n_s
     k_restore<<<1184, 256, 0, st>>>(reinterpret_cast<uint4*>(lat->links), reinterpret_cast<const uint4*>(ws_links(lat)),
                                     lb / 16, flag);
     if ((s = cuda_check("mgq_hmc_trajectory"))) return s;
+    if (dH_out && accepted_out && !is_device_ptr(dH_out) && !is_device_ptr(accepted_out)) {
+        // dH (slot 4) and the flag (slot 7) in one copy
+        double buf[4];
+        if ((s = deliver(sc + 4, buf, 4, st, "mgq_hmc_trajectory"))) return s;
+        *dH_out = buf[0];
+        memcpy(accepted_out, buf + 3, sizeof(int));
+        return MGQ_OK;
+    }
     if ((s = deliver(sc + 4, dH_out, dH_out ? 1 : 0, st, "mgq_hmc_trajectory"))) return s;
     return deliver_int(flag, accepted_out, accepted_out ? 1 : 0, st, "mgq_hmc_trajectory");
 }

@@ -55,6 +55,10 @@ mgq_status check_lattice(const mgq_lattice* lat, bool need_work, const char* fn)
 // destination synchronises the stream.
 mgq_status deliver(const double* dev_src, double* out, size_t n, cudaStream_t st, const char* fn);
 mgq_status deliver_int(const int* dev_src, int* out, size_t n, cudaStream_t st, const char* fn);
+// Delivers n pairs (a_i, b_i) lying at dev_src to a_out[i] and b_out[i] (host or
+// device, NULL to skip): one copy and one synchronisation for all that goes to the
+// host.  n <= WS_NSCALARS / 2.
+mgq_status deliver_pairs(const double* dev_src, double* a_out, double* b_out, size_t n, cudaStream_t st, const char* fn);
 bool is_device_ptr(const void* p);
 
 // Number of blocks used by the site-parallel reduction kernels.
@@ -65,6 +69,8 @@ int block_size(int kernel, int prec);
 
 // Sums n partials in a fixed order into out[0] * scale (device).
 void launch_final_sum(const double* partials, int n, double scale, double* out, cudaStream_t st);
+// The same for two sets of n partials at once: out[0] and out[1].
+void launch_final_sum2(const double* partials, int n, double scale0, double scale1, double* out, cudaStream_t st);
 
 // launchers shared between translation units
 mgq_status plaquette_into(const mgq_lattice* lat, double* partials, double* dev_out, cudaStream_t st);

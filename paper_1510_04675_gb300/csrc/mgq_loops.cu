@@ -109,8 +109,22 @@ __global__ void __launch_bounds__(128) k_partial_loops(Links<T, NP> U, Links<T, 
     if (threadIdx.x == 0) partials[8 * nb + b] = smax[0];
 }
 
-__global__ void k_max_final(const double* __restrict__ partials, int n, double* out) {
-    __shared__ double sm[256];
+struct LoopScales {
+    double s[8];
+};
+
+// block q < 8: the q-th class sum times its scale; block 8: the maximum of the last set
+__global__ void k_partial_final(const double* __restrict__ partials, int n, LoopScales sc, double* out) {
+    const int q = blockIdx.x;
+    partials += (size_t)q * n;
+    if (q < 8) {
+        double v = 0.0;
+        for (int i = threadIdx.x; i < n; i += blockDim.x) v += partials[i];
+        v = block_sum(v);
+        if (threadIdx.x == 0) out[q] = v * sc.s[q];
+        return;
+    }
+    __shared__ double sm[512];
     double m = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) m = fmax(m, partials[i]);
     sm[threadIdx.x] = m;
@@ -119,7 +133,7 @@ __global__ void k_max_final(const double* __restrict__ partials, int n, double* 
         if ((int)threadIdx.x < o) sm[threadIdx.x] = fmax(sm[threadIdx.x], sm[threadIdx.x + o]);
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[0] = sm[0];
+    if (threadIdx.x == 0) out[8] = sm[0];
 }
 
 static double binom(int n, int k) {
@@ -169,12 +183,10 @@ mgq_status mgq_partial_loops(const mgq_lattice* lat, double* out, void* stream) 
     });
     double* sc = ws_scalars(lat);
     const double V = (double)g.V;
-    for (int d = 0; d < 3; d++)
-        launch_final_sum(ws_partials(lat) + d * nb, nb, 1.0 / (6.0 * (4 - d) * (3 - d) * binom(4, d) * V / 16.0),
-                         sc + 24 + d, st);
-    for (int d = 0; d < 5; d++)
-        launch_final_sum(ws_partials(lat) + (3 + d) * nb, nb, 1.0 / (18.0 * binom(4, d) * V / 16.0), sc + 27 + d, st);
-    k_max_final<<<1, 256, 0, st>>>(ws_partials(lat) + 8 * nb, nb, sc + 32);
+    LoopScales sc9;
+    for (int d = 0; d < 3; d++) sc9.s[d] = 1.0 / (6.0 * (4 - d) * (3 - d) * binom(4, d) * V / 16.0);
+    for (int d = 0; d < 5; d++) sc9.s[3 + d] = 1.0 / (18.0 * binom(4, d) * V / 16.0);
+    k_partial_final<<<9, 512, 0, st>>>(ws_partials(lat), nb, sc9, sc + 24);
     if ((s = cuda_check("mgq_partial_loops"))) return s;
     return deliver(sc + 24, out, 9, st, "mgq_partial_loops");
 }

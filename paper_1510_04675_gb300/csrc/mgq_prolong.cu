@@ -2,6 +2,7 @@
 // transfer step of the prolongation (Eq. prolongation) and the interpolation
 // stages, each a repeated Jacobi APE step (Eq. APE) on the active bonds of
 // stage d that minimises the partial action S_d (Eq. smoothing).
+#include <cstring>
 #include <vector>
 
 #include "mgq_internal.h"
@@ -695,6 +696,14 @@ mgq_status mgq_prolongate(const mgq_lattice* coarse, mgq_lattice* fine, double c
     S.partials = ws_partials(fine);
     void* scratch[1] = {ws_links(fine)};
     if ((s = prolong_run(coarse, fine, scratch, 1, c, rel_tol, max_iter, 0, S, st))) return s;
+    if (iters_out && sd_out && !is_device_ptr(iters_out) && !is_device_ptr(sd_out)) {
+        // both results lie in five neighbouring scalars: one copy, one synchronisation
+        double buf[5];
+        if ((s = deliver(sc + 58, buf, 5, st, "mgq_prolongate"))) return s;
+        memcpy(iters_out, buf, 3 * sizeof(int));
+        memcpy(sd_out, buf + 2, 3 * sizeof(double));
+        return MGQ_OK;
+    }
     if (iters_out && (s = deliver_int(S.iters, iters_out, 3, st, "mgq_prolongate"))) return s;
     if (sd_out && (s = deliver(S.sd, sd_out, 3, st, "mgq_prolongate"))) return s;
     return MGQ_OK;

@@ -19,7 +19,10 @@ def test_columns_equal_one_thread_per_link(gpu, dims, n_hb):
     gpu.mgq_init_links(a, 1)
     b = gpu.copy_lattice(a)
     plaq = gpu.mgq_update_sweeps(a, 5.8, 3, 2, n_hb, 2, plaq_out=True)
-    batch = gpu.Batch([b], [5.8], max_sweeps=2)
+    # beside a lattice large enough that the launches take one thread per link
+    filler = gpu.Lattice([16, 16, 16, 16], "f64", seed=1)
+    gpu.mgq_init_links(filler, 0)
+    batch = gpu.Batch([b, filler], [5.8, 5.8], max_sweeps=2)
     rec = batch.plaquette_buffer(2)
     gpu.mgq_update_sweeps_batched(batch, 3, 2, n_hb, 2, plaq_out=rec)
     assert torch.equal(a.links, b.links)

@@ -21,7 +21,10 @@ def test_terms_equal_one_thread_per_link(gpu, prec, dims):
     gpu.mgq_init_links(a, 1)
     b = gpu.copy_lattice(a)
     plaq = gpu.mgq_update_sweeps(a, 5.9, 7, 2, 1, 2, plaq_out=True)
-    batch = gpu.Batch([b], [5.9], max_sweeps=2)
+    # beside a lattice large enough that the launches take one thread per link
+    filler = gpu.Lattice([24, 24, 24, 24], prec, seed=1)
+    gpu.mgq_init_links(filler, 0)
+    batch = gpu.Batch([b, filler], [5.9, 5.9], max_sweeps=2)
     rec = batch.plaquette_buffer(2)
     gpu.mgq_update_sweeps_batched(batch, 7, 2, 1, 2, plaq_out=rec)
     assert torch.equal(a.links, b.links)
