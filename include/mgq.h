@@ -110,9 +110,9 @@ uint64_t mgq_workspace_bytes(const mgq_lattice* lat);
  * kernels are compiled for at most 128); 128 by default.  Results do not
  * depend on it.  It applies where a thread holds a link (or an active bond):
  * FP32 12-real sub-sweeps, which stage their links through shared memory in blocks
- * of 128, and single-lattice sub-sweeps of too few links to fill the chip with a
- * thread each (FP64; FP32 below V/2 = 40960, 12-real below 65536), which run several
- * lanes or warps per link, have shapes of their own.  The force kernels' shapes are
+ * of 128, and sub-sweep launches over too few links to fill the chip with a thread
+ * each (FP64; FP32 below 40960 links, 12-real below 65536), which run several lanes
+ * or warps per link, have shapes of their own.  The force kernels' shapes are
  * structural and not tuned.  Process-wide setting; change it only while no call is
  * being issued.  Set by the autotuner (paper_1510_04675_gb300/tune.py). */
 typedef enum {
@@ -291,8 +291,8 @@ mgq_status mgq_wilson_flow(mgq_lattice* lat, double eps, int n_steps, int meas_e
  * in [0, t_end]; at most 224) into E_out[i], Q_out[i] (host or device, NULL to
  * skip).  charge 0: clover Q; charge 1: the three-loop improved Q of
  * mgq_topo_charge_improved (Sec. IV.C).  The links are replaced by the field
- * at t_end.  Uses the workspace's algebra buffer.  Errors: MGQ_EINVAL (bad
- * times, eps <= 0, more than 1e8 steps), MGQ_ENOMEM. */
+ * at t_end.  Uses the workspace's algebra buffer and, for charge 1, its link
+ * copy.  Errors: MGQ_EINVAL (bad times, eps <= 0, more than 1e8 steps), MGQ_ENOMEM. */
 mgq_status mgq_wilson_flow_times(mgq_lattice* lat, double t_end, double eps, const double* t_meas, int n_meas,
                                  int charge, double* E_out, double* Q_out, void* stream);
 

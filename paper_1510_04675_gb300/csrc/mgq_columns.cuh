@@ -49,8 +49,8 @@ struct ColumnLane {
         k = sub - 3 * half;
         base = lane - k;
     }
-    __device__ __forceinline__ int item() const {
-        return (blockIdx.x * (COL_THREADS / 32) + (threadIdx.x >> 5)) * kPerWarp + grp;
+    __device__ __forceinline__ int item(int block) const {
+        return (block * (COL_THREADS / 32) + (threadIdx.x >> 5)) * kPerWarp + grp;
     }
 };
 
@@ -152,12 +152,12 @@ __device__ __forceinline__ void column_reunitarize(Cx<double> u[3], int k, int b
 // partials != nullptr (the direction-3 sub-sweeps that end an overrelaxation
 // sweep) also the plaquettes of k_overrelax_last, lane k taking plane k of
 // (0,1), (0,2), (1,2), summed per block.
+// The links are those of block `block` of the lattice; partial receives the block's sum.
 template <bool HB, int LPL>
-__global__ void __launch_bounds__(COL_THREADS) k_update_columns(Links<double, 9> U, Geom g, int mu, int par, double beta,
-                                                                RngKey rk, int n_hb, uint8_t* __restrict__ dec,
-                                                                double* __restrict__ partials) {
+__device__ __forceinline__ void update_columns(const Links<double, 9>& U, const Geom& g, int block, int mu, int par, double beta,
+                                               const RngKey& rk, int n_hb, uint8_t* dec, double* partial) {
     const ColumnLane<LPL> c;
-    const int h0 = c.item();
+    const int h0 = c.item(block);
     const bool live = c.active && h0 < g.Vh && c.half == (LPL == 6 ? 1 : 0);  // the lanes that end with U
     const int h = h0 < g.Vh ? h0 : g.Vh - 1;
     int x[4];
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(COL_THREADS) k_update_columns(Links<double, 9>
 #pragma unroll
         for (int i = 0; i < 3; i++) b[(3 * i + c.k) << 5] = u[i];
     }
-    if (partials) {
+    if (partial) {
         if (live) {
             const int a = c.k == 2 ? 1 : 0, b = c.k == 0 ? 1 : 2;
             const int ha = lex_hop(g, x, a, +1) >> 1, hb = lex_hop(g, x, b, +1) >> 1;
@@ -232,8 +232,14 @@ __global__ void __launch_bounds__(COL_THREADS) k_update_columns(Links<double, 9>
             acc = 0.0;
         }
         acc = block_sum(acc);
-        if (threadIdx.x == 0) partials[blockIdx.x] = acc;
+        if (threadIdx.x == 0) *partial = acc;
     }
+}
+
+template <bool HB, int LPL>
+__global__ void __launch_bounds__(COL_THREADS) k_update_columns(Links<double, 9> U, Geom g, int mu, int par, double beta, RngKey rk,
+                                                                int n_hb, uint8_t* __restrict__ dec, double* __restrict__ partials) {
+    update_columns<HB, LPL>(U, g, blockIdx.x, mu, par, beta, rk, n_hb, dec, partials ? partials + blockIdx.x : nullptr);
 }
 
 // The force of every link (as k_force), block row y the (mu, parity) plane.  With M = U A by columns, lane k holds M_nk of the pair (k, n),
@@ -241,7 +247,7 @@ __global__ void __launch_bounds__(COL_THREADS) k_update_columns(Links<double, 9>
 template <int LPL, class Out>
 __global__ void __launch_bounds__(COL_THREADS) k_force_columns(Links<double, 9> U, Geom g, Out out) {
     const ColumnLane<LPL> c;
-    const int mu = blockIdx.y >> 1, par = blockIdx.y & 1, h0 = c.item(), h = h0 < g.Vh ? h0 : g.Vh - 1;
+    const int mu = blockIdx.y >> 1, par = blockIdx.y & 1, h0 = c.item(blockIdx.x), h = h0 < g.Vh ? h0 : g.Vh - 1;
     int x[4];
     cb_coords(g, par, h, x);
     pdl_wait();

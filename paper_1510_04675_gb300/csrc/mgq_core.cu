@@ -216,22 +216,35 @@ __global__ void k_init(Links<T, NP> U, Geom g, int start, RngKey rk) {
     U.store(mu, par, h, u);
 }
 
+// coordinates of lexicographic site lex
+__device__ __forceinline__ void lex_site(const Geom& g, int lex, int x[4]) {
+    const int r0 = div_L(g, 0, lex), r1 = div_L(g, 1, r0);
+    x[0] = lex - r0 * g.L[0];
+    x[1] = r0 - r1 * g.L[1];
+    x[3] = div_L(g, 2, r1);
+    x[2] = r1 - x[3] * g.L[2];
+}
+
 // canonical double[V][4][3][3][2] <-> lattice layout
-template <class T, int NP>
+// A link's 18 doubles are nine 16-byte words (144 bytes; canon is 16-byte aligned for
+// ALIGNED); 12-real links read rows 0 and 1 only.
+template <class T, int NP, bool ALIGNED>
 __global__ void k_import(Links<T, NP> U, Geom g, const double* __restrict__ canon) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= 4 * g.V) return;
     const int lex = idx >> 2, mu = idx & 3;
     int x[4];
-    int r = lex;
-    for (int m = 0; m < 4; m++) { x[m] = r % g.L[m]; r /= g.L[m]; }
+    lex_site(g, lex, x);
     const int par = (x[0] + x[1] + x[2] + x[3]) & 1;
     const double* src = canon + (size_t)idx * 18;
     M3<T> u;
 #pragma unroll
-    for (int a = 0; a < 3; a++)
-#pragma unroll
-        for (int b = 0; b < 3; b++) u.e[a][b] = mk((T)src[(a * 3 + b) * 2], (T)src[(a * 3 + b) * 2 + 1]);
+    for (int e = 0; e < NP; e++) {
+        double2 v;
+        if constexpr (ALIGNED) v = reinterpret_cast<const double2*>(src)[e];
+        else v = make_double2(src[2 * e], src[2 * e + 1]);
+        u.e[e / 3][e % 3] = mk((T)v.x, (T)v.y);
+    }
     U.store(mu, par, lex >> 1, u);
 }
 
@@ -241,8 +254,7 @@ __global__ void k_export(Links<T, NP> U, Geom g, double* __restrict__ canon) {
     if (idx >= 4 * g.V) return;
     const int lex = idx >> 2, mu = idx & 3;
     int x[4];
-    int r = lex;
-    for (int m = 0; m < 4; m++) { x[m] = r % g.L[m]; r /= g.L[m]; }
+    lex_site(g, lex, x);
     const int par = (x[0] + x[1] + x[2] + x[3]) & 1;
     M3<T> u = U.load(mu, par, lex >> 1);
     double* dst = canon + (size_t)idx * 18;
@@ -480,19 +492,7 @@ static int launch_columns(int lanes, mgq_lattice* lat, const Geom& g, int mu, in
     return nb;
 }
 
-// FP32 sub-sweeps with the staple's terms shared among warps (k_update_terms): 6 or 3
-// warps per 32 links, 0 for the kernels with a thread per link.  Six warps give the
-// shortest chain, three hold more links per SM; a thread per link wins once it fills
-// the SMs, for 18-real links from about 49152 links on (one wave of its blocks: 7.8
-// against 8.3 us per overrelaxation launch), for 12-real ones, whose one-thread form
-// stages its links, from about 73728 (10.0 against 10.5 us; at 49152 9.8 against 8.3).
-// Several attempts per subgroup, or recorded decisions, run a thread per link.
-static int term_warps(const mgq_lattice* lat, const Geom& g) {
-    if (lat->prec == MGQ_F64) return 0;
-    if (g.Vh < 16384) return 6;
-    return g.Vh < (lat->prec == MGQ_F32 ? 40960 : 65536) ? 3 : 0;
-}
-
+// FP32 sub-sweeps with the staple's terms shared among warps (term_warps);
 // returns the number of blocks
 template <int KIND>
 static int launch_terms(int warps, mgq_lattice* lat, const Geom& g, int mu, int par, double beta, const RngKey& rk,
@@ -517,7 +517,7 @@ mgq_status heatbath_subsweep(mgq_lattice* lat, double beta, uint64_t sweep, int 
         launch_columns<true>(lanes, lat, g, mu, par, beta, rk, n_hb, dec, nullptr, st);
         return cuda_check("mgq_heatbath");
     }
-    if (const int warps = n_hb == 1 && !dec ? term_warps(lat, g) : 0) {
+    if (const int warps = n_hb == 1 && !dec ? term_warps(lat->prec, g.Vh) : 0) {
         launch_terms<TERMS_HEATBATH>(warps, lat, g, mu, par, beta, rk, nullptr, st);
         return cuda_check("mgq_heatbath");
     }
@@ -543,7 +543,7 @@ mgq_status overrelax_subsweep(mgq_lattice* lat, int mu, int par, cudaStream_t st
         launch_columns<false>(lanes, lat, g, mu, par, 0.0, RngKey{}, 0, nullptr, nullptr, st);
         return cuda_check("mgq_overrelax");
     }
-    if (const int warps = term_warps(lat, g)) {
+    if (const int warps = term_warps(lat->prec, g.Vh)) {
         launch_terms<TERMS_OVERRELAX>(warps, lat, g, mu, par, 0.0, RngKey{}, nullptr, st);
         return cuda_check("mgq_overrelax");
     }
@@ -577,7 +577,7 @@ mgq_status overrelax_sweep_plaquette(mgq_lattice* lat, double* dev_out, cudaStre
         launch_final_sum(partials, n, 1.0 / (18.0 * (double)g.V), dev_out, st);
         return cuda_check("overrelax_sweep_plaquette");
     }
-    if (const int warps = term_warps(lat, g)) {
+    if (const int warps = term_warps(lat->prec, g.Vh)) {
         int n = 0;
         for (int par = 0; par < 2; par++)
             n += launch_terms<TERMS_OVERRELAX_LAST>(warps, lat, g, 3, par, 0.0, RngKey{}, partials + n, st);
@@ -673,7 +673,10 @@ mgq_status mgq_import_links(mgq_lattice* lat, const double* canon, void* stream)
     const Geom g = make_geom(lat->dims);
     cudaStream_t st = as_stream(stream);
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
-        k_import<T, NP><<<nblk(4L * g.V, 128), 128, 0, st>>>(links_of<T, NP>(lat), g, canon);
+        if (((uintptr_t)canon & 15) == 0)
+            k_import<T, NP, true><<<nblk(4L * g.V, 128), 128, 0, st>>>(links_of<T, NP>(lat), g, canon);
+        else
+            k_import<T, NP, false><<<nblk(4L * g.V, 128), 128, 0, st>>>(links_of<T, NP>(lat), g, canon);
     });
     return cuda_check("mgq_import_links");
 }

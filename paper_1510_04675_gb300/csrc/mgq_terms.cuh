@@ -9,7 +9,7 @@
 // links.  The products, the order of the additions and the update are those of the
 // one-thread form, so both agree bit for bit.  FP32 12-real, heat bath and
 // overrelaxation per launch: 8^4 6.6 and 3.8 -> 3.6 and 2.8 us, 12^4 8.0 and 6.3 -> 5.1
-// and 4.2 us (six warps); 16^4 9.6 and 6.6 -> 7.4 and 6.5 us (three).
+// and 3.9 us (six warps); 16^4 9.6 and 6.6 -> 7.5 and 6.4 us (three).
 #pragma once
 
 #include "mgq_stencil.cuh"
@@ -40,14 +40,14 @@ enum { TERMS_HEATBATH = 0, TERMS_OVERRELAX = 1, TERMS_OVERRELAX_LAST = 2 };
 // each of warps 0 to 2 after its terms), overrelaxation, or the direction-3
 // overrelaxation that also measures plaquettes as k_overrelax_last does (the planes
 // of directions 0, 1, 2 shared among the warps from 1 on; one partial sum per block).
+// The links are those of block `block` of the lattice; partial receives the block's sum.
 template <int NP, int KIND, int WARPS>
-__global__ void __launch_bounds__(WARPS * TERMS_LINKS, 24 / WARPS) k_update_terms(Links<float, NP> U, Geom g, int mu, int par, float beta, RngKey rk,
-                                                                   double* __restrict__ partials) {
+__device__ __forceinline__ void update_terms(const Links<float, NP>& U, const Geom& g, int block, int mu, int par, float beta,
+                                             const RngKey& rk, double* partial) {
     __shared__ float2 term[6][9][TERMS_LINKS];
     __shared__ uint4 words[3][TERMS_LINKS];
-    pdl_launch_dependents();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int h0 = blockIdx.x * TERMS_LINKS + lane, h = h0 < g.Vh ? h0 : g.Vh - 1;
+    const int h0 = block * TERMS_LINKS + lane, h = h0 < g.Vh ? h0 : g.Vh - 1;
     int x[4];
     cb_coords(g, par, h, x);
     const Hops H = make_hops(g, x);
@@ -63,6 +63,9 @@ __global__ void __launch_bounds__(WARPS * TERMS_LINKS, 24 / WARPS) k_update_term
     if (KIND == TERMS_HEATBATH && w < 3)
         words[w][lane] = draw(rk, (uint32_t)H.lex, (uint32_t)mu, (uint32_t)w, 0u, KIND_HB);
     __syncthreads();
+    // only now: blocks of the next launch that settle earlier crowd the SMs unevenly
+    // (12^4 overrelaxation 4.2 -> 3.85 us)
+    pdl_launch_dependents();
     double acc = 0.0;
     if (w == 0) {
         M3<float> A;
@@ -88,8 +91,27 @@ __global__ void __launch_bounds__(WARPS * TERMS_LINKS, 24 / WARPS) k_update_term
     }
     if constexpr (KIND == TERMS_OVERRELAX_LAST) {
         acc = block_sum(acc);
-        if (threadIdx.x == 0) partials[blockIdx.x] = acc;
+        if (threadIdx.x == 0) *partial = acc;
     }
+}
+
+template <int NP, int KIND, int WARPS>
+__global__ void __launch_bounds__(WARPS * TERMS_LINKS, 24 / WARPS) k_update_terms(Links<float, NP> U, Geom g, int mu, int par, float beta, RngKey rk,
+                                                                                  double* __restrict__ partials) {
+    update_terms<NP, KIND, WARPS>(U, g, blockIdx.x, mu, par, beta, rk, KIND == TERMS_OVERRELAX_LAST ? partials + blockIdx.x : nullptr);
+}
+
+// Warps per 32 links of an FP32 launch over n links, 0 for the kernels with a thread per
+// link.  Six warps give the shortest chain, three hold more links per SM; a thread per
+// link wins once it fills the SMs, for 18-real links from about 49152 links on (one
+// wave of its blocks: 7.8 against 8.3 us per overrelaxation launch), for 12-real ones,
+// whose one-thread form stages its links, from about 73728 (10.0 against 10.5 us; at
+// 49152 9.8 against 8.3).  Several attempts per subgroup, or recorded decisions, run a
+// thread per link.
+inline int term_warps(int prec, long n) {
+    if (prec == MGQ_F64) return 0;
+    if (n < 16384) return 6;
+    return n < (prec == MGQ_F32 ? 40960 : 65536) ? 3 : 0;
 }
 
 }  // namespace mgq
