@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, batch_blocks<T, NP>()) k_overre
 // warp (blocks of TERMS_LINKS links), FP64 with a column per lane (12 lattices of 6^4,
 // 8^4 and 4^3x8, one compound sweep with plaquettes: 12-real 273 -> 170 us, FP64 6.9 -> 2.1
 // ms).
-template <int NP, int KIND, int WARPS>
+template <int NP, int KIND, int WARPS, bool FMA>
 __global__ void __launch_bounds__(WARPS * TERMS_LINKS, 24 / WARPS)
     k_update_terms_batched(const __grid_constant__ Batch<float> B, int mu, int par, uint32_t idx_lo, uint32_t idx_hi,
                            double* __restrict__ partials) {
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(WARPS * TERMS_LINKS, 24 / WARPS)
     rk.key = d.key;
     rk.idx_lo = idx_lo;
     rk.idx_hi = idx_hi;
-    update_terms<NP, KIND, WARPS>(U, geom_of(d), blockIdx.x - B.prefix[l], mu, par, d.beta, rk,
+    update_terms<NP, KIND, WARPS, FMA>(U, geom_of(d), blockIdx.x - B.prefix[l], mu, par, d.beta, rk,
                                   KIND == TERMS_OVERRELAX_LAST ? partials + par * B.prefix[B.n] + blockIdx.x : nullptr);
 }
 
@@ -234,11 +234,13 @@ __global__ void k_plaquette_batched_final(const __grid_constant__ Batch<T> B, co
     if (threadIdx.x == 0) out[l] = v / (18.0 * (double)B.d[l].g.V);
 }
 
-// one FP32 sub-sweep of the launch with `warps` warps per 32 links
+// one FP32 sub-sweep of the launch over `links` links with `warps` warps per 32 links
 template <int NP, int KIND>
-static void launch_terms_batched(int warps, const Batch<float>& B, int mu, int par, uint64_t sweep, double* partials, cudaStream_t st) {
-    launch_pdl(warps == 6 ? k_update_terms_batched<NP, KIND, 6> : k_update_terms_batched<NP, KIND, 3>, B.prefix[B.n],
-               warps * TERMS_LINKS, st, B, mu, par, (uint32_t)(sweep & 0xffffffffu), (uint32_t)(sweep >> 32), partials);
+static void launch_terms_batched(int warps, long links, const Batch<float>& B, int mu, int par, uint64_t sweep, double* partials, cudaStream_t st) {
+    launch_pdl(warps == 6                 ? k_update_terms_batched<NP, KIND, 6, true>
+               : term_single_fma(links) ? k_update_terms_batched<NP, KIND, 3, true>
+                                        : k_update_terms_batched<NP, KIND, 3, NP == 9>,  // 18-real launches stay below
+               B.prefix[B.n], warps * TERMS_LINKS, st, B, mu, par, (uint32_t)(sweep & 0xffffffffu), (uint32_t)(sweep >> 32), partials);
 }
 // one FP64 sub-sweep with `lanes` lanes per link
 template <bool HB>
@@ -368,12 +370,12 @@ mgq_status mgq_update_sweeps_batched(mgq_lattice* lats, int n_lat, const double*
                         Batch<T> Bt;
                         fill_batch(Bt, lats, betas, first, n, TERMS_LINKS, true);
                         sweeps([&](int mu, int par) {
-                            if (n_hb == 1) launch_terms_batched<NP, TERMS_HEATBATH>(warps, Bt, mu, par, sweep, nullptr, st);
+                            if (n_hb == 1) launch_terms_batched<NP, TERMS_HEATBATH>(warps, links, Bt, mu, par, sweep, nullptr, st);
                             else heatbath(mu, par);
                         }, [&](int mu, int par) {
-                            launch_terms_batched<NP, TERMS_OVERRELAX>(warps, Bt, mu, par, sweep, nullptr, st);
+                            launch_terms_batched<NP, TERMS_OVERRELAX>(warps, links, Bt, mu, par, sweep, nullptr, st);
                         }, [&](int par) {
-                            launch_terms_batched<NP, TERMS_OVERRELAX_LAST>(warps, Bt, 3, par, sweep, partials, st);
+                            launch_terms_batched<NP, TERMS_OVERRELAX_LAST>(warps, links, Bt, 3, par, sweep, partials, st);
                         });
                         if (fold)
                             k_overrelax_batched_last_final<T><<<n, 256, 0, st>>>(Bt, partials, results + (size_t)i * n_lat + first);

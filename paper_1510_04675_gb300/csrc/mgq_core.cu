@@ -499,11 +499,12 @@ static int launch_terms(int warps, mgq_lattice* lat, const Geom& g, int mu, int 
                         double* partials, cudaStream_t st) {
     const int nb = nblk(g.Vh, TERMS_LINKS);
     if (lat->prec == MGQ_F32)
-        launch_pdl(warps == 6 ? k_update_terms<9, KIND, 6> : k_update_terms<9, KIND, 3>, nb, warps * TERMS_LINKS, st,
+        launch_pdl(warps == 6 ? k_update_terms<9, KIND, 6, true> : k_update_terms<9, KIND, 3, true>, nb, warps * TERMS_LINKS, st,
                    links_of<float, 9>(lat), g, mu, par, (float)beta, rk, partials);
     else
-        launch_pdl(warps == 6 ? k_update_terms<6, KIND, 6> : k_update_terms<6, KIND, 3>, nb, warps * TERMS_LINKS, st,
-                   links_of<float, 6>(lat), g, mu, par, (float)beta, rk, partials);
+        launch_pdl(warps == 6 ? k_update_terms<6, KIND, 6, true> : term_single_fma(g.Vh) ? k_update_terms<6, KIND, 3, true>
+                                                                                         : k_update_terms<6, KIND, 3, false>,
+                   nb, warps * TERMS_LINKS, st, links_of<float, 6>(lat), g, mu, par, (float)beta, rk, partials);
     return nb;
 }
 

@@ -8,8 +8,8 @@
 // shared memory, and warp 0 adds the six in staple_two_row's order and updates the
 // links.  The products, the order of the additions and the update are those of the
 // one-thread form, so both agree bit for bit.  FP32 12-real, heat bath and
-// overrelaxation per launch: 8^4 6.6 and 3.8 -> 3.6 and 2.8 us, 12^4 8.0 and 6.3 -> 5.1
-// and 3.9 us (six warps); 16^4 9.6 and 6.6 -> 7.5 and 6.4 us (three).
+// overrelaxation per launch: 8^4 6.6 and 3.8 -> 3.3 and 2.5 us, 12^4 8.0 and 6.3 -> 4.7
+// and 3.7 us (six warps); 16^4 9.6 and 6.6 -> 6.7 and 6.0 us (three).
 #pragma once
 
 #include "mgq_stencil.cuh"
@@ -19,17 +19,17 @@ namespace mgq {
 constexpr int TERMS_LINKS = 32;  // per block
 
 // half-term w of the staple of U_mu(x), as in staple_two_row: direction w / 2 of
-// those other than mu, upper (even w) or lower
-template <int NP>
+// those other than mu, upper (even w) or lower; FMA as in two_rows
+template <bool FMA, int NP>
 __device__ __forceinline__ M3<float> staple_half_term(const Links<float, NP>& U, const Hops& H, int mu, int par, int w) {
     const int op = par ^ 1, i = w >> 1, nu = i < mu ? i : i + 1;
     const int fmu = pick(H.fwd, mu);
     M3<float> r;
     if ((w & 1) == 0) {
-        r = up_term(U.load_rows(nu, op, (H.lex + fmu) >> 1), U.load(mu, op, (H.lex + pick(H.fwd, nu)) >> 1), U.load(nu, par, H.lex >> 1));
+        r = up_term<FMA>(U.load_rows(nu, op, (H.lex + fmu) >> 1), U.load(mu, op, (H.lex + pick(H.fwd, nu)) >> 1), U.load(nu, par, H.lex >> 1));
     } else {
         const int b = pick(H.bwd, nu), hmn = (H.lex + b) >> 1;
-        r = down_term(U.load_rows(mu, op, hmn), U.load(nu, par, (H.lex + fmu + b) >> 1), U.load(nu, op, hmn));
+        r = down_term<FMA>(U.load_rows(mu, op, hmn), U.load(nu, par, (H.lex + fmu + b) >> 1), U.load(nu, op, hmn));
     }
     return r;
 }
@@ -41,7 +41,7 @@ enum { TERMS_HEATBATH = 0, TERMS_OVERRELAX = 1, TERMS_OVERRELAX_LAST = 2 };
 // overrelaxation that also measures plaquettes as k_overrelax_last does (the planes
 // of directions 0, 1, 2 shared among the warps from 1 on; one partial sum per block).
 // The links are those of block `block` of the lattice; partial receives the block's sum.
-template <int NP, int KIND, int WARPS>
+template <int NP, int KIND, int WARPS, bool FMA>
 __device__ __forceinline__ void update_terms(const Links<float, NP>& U, const Geom& g, int block, int mu, int par, float beta,
                                              const RngKey& rk, double* partial) {
     __shared__ float2 term[6][9][TERMS_LINKS];
@@ -56,7 +56,7 @@ __device__ __forceinline__ void update_terms(const Links<float, NP>& U, const Ge
     if (w == 0) u = U.load(mu, par, h);
 #pragma unroll 1
     for (int k = w * (6 / WARPS); k < (w + 1) * (6 / WARPS); k++) {
-        const M3<float> t = staple_half_term(U, H, mu, par, k);
+        const M3<float> t = staple_half_term<FMA>(U, H, mu, par, k);
 #pragma unroll
         for (int e = 0; e < 9; e++) term[k][e][lane] = make_float2(t.e[e / 3][e % 3].re, t.e[e / 3][e % 3].im);
     }
@@ -95,16 +95,16 @@ __device__ __forceinline__ void update_terms(const Links<float, NP>& U, const Ge
     }
 }
 
-template <int NP, int KIND, int WARPS>
+template <int NP, int KIND, int WARPS, bool FMA>
 __global__ void __launch_bounds__(WARPS * TERMS_LINKS, 24 / WARPS) k_update_terms(Links<float, NP> U, Geom g, int mu, int par, float beta, RngKey rk,
                                                                                   double* __restrict__ partials) {
-    update_terms<NP, KIND, WARPS>(U, g, blockIdx.x, mu, par, beta, rk, KIND == TERMS_OVERRELAX_LAST ? partials + blockIdx.x : nullptr);
+    update_terms<NP, KIND, WARPS, FMA>(U, g, blockIdx.x, mu, par, beta, rk, KIND == TERMS_OVERRELAX_LAST ? partials + blockIdx.x : nullptr);
 }
 
 // Warps per 32 links of an FP32 launch over n links, 0 for the kernels with a thread per
 // link.  Six warps give the shortest chain, three hold more links per SM; a thread per
-// link wins once it fills the SMs, for 18-real links from about 49152 links on (one
-// wave of its blocks: 7.8 against 8.3 us per overrelaxation launch), for 12-real ones,
+// link wins once it fills the SMs, for 18-real links from 40960 on (one wave of its
+// blocks; overrelaxation of 49152 links 7.8 against 8.3 us), for 12-real ones,
 // whose one-thread form stages its links, from about 73728 (10.0 against 10.5 us; at
 // 49152 9.8 against 8.3).  Several attempts per subgroup, or recorded decisions, run a
 // thread per link.
@@ -113,5 +113,12 @@ inline int term_warps(int prec, long n) {
     if (n < 16384) return 6;
     return n < (prec == MGQ_F32 ? 40960 : 65536) ? 3 : 0;
 }
+
+// The products of such a launch: single FMAs, whose chain is shorter (12-real heat bath
+// and overrelaxation of 16^4 7.3 and 6.2 -> 6.7 and 6.0 us, 18-real 6.9 and 6.0 -> 6.7
+// and 5.5), except where the SMs hold a full wave of three-warp blocks and more:
+// there issue counts and the packed forms have fewer (16^3x24: packed 10.1 and 8.1,
+// single 10.3 and 8.6 us; 16^3x20: 9.6 and 7.1 against 9.4 and 7.0).  The bits are the same.
+inline bool term_single_fma(long n) { return n < 49152; }
 
 }  // namespace mgq
