@@ -254,8 +254,8 @@ mgq_status mgq_wilson_loop(const mgq_lattice* lat, int m, int n, double* out, vo
  * chi_munu(n) = d, normalised by N^{1x1}_d = 2 (D-d)(D-d-1) C(D,d) N_0/2^D),
  * out[3..7] displaced loops W^{2x2}_d (2x2 loops from sites with chi(n) = d,
  * N^{2x2}_d = C(D,2) C(D,d) N_0/2^D), out[8] h = max_p N_c [1 - W^{1x1}_p]
- * (admissibility when h < 0.067).  Needs the workspace (its link copy holds
- * the lines of two links). */
+ * (admissibility when h < 0.067).  Needs the workspace (its link copy and
+ * algebra buffer hold the lines of two links). */
 mgq_status mgq_partial_loops(const mgq_lattice* lat, double* out, void* stream);
 
 /* Clover energy density E = (1/V) sum_x -1/2 sum_{mu,nu} Tr G_munu^2 and
@@ -271,7 +271,7 @@ mgq_status mgq_topo_charge(const mgq_lattice* lat, double* E_out, double* Q_out,
  * Q = 3/2 Q_1 - 3/5 Q_2 / 2^4 + 1/10 Q_3 / 3^4, the tree-level coefficients
  * that cancel the O(a^2) and O(a^4) terms of the m x m clovers.
  * Q_out[4] = {Q, Q_1, Q_2, Q_3} (host or device).  Needs the workspace (its
- * link copy holds the lines of m links).
+ * link copy and algebra buffer hold the lines of m links).
  * Errors: MGQ_EINVAL, MGQ_ENOMEM. */
 mgq_status mgq_topo_charge_improved(const mgq_lattice* lat, double* Q_out, void* stream);
 

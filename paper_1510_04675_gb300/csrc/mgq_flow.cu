@@ -10,8 +10,9 @@ namespace mgq {
 // using Tr(X_a X_b) = -delta_ab / 2, with G from the leaves of the line field A of
 // m links a side (m = 1: the links).  One thread per site and dual pair of planes
 // (block row y): its two field strengths stay in registers, and a small lattice
-// has three times the threads of a thread per site (24^3x48, FP32 12-real: 352 ->
-// 245 us; 16^4: 44 -> 29 us).
+// has three times the threads of a thread per site (mgq_topo_charge on 24^3x48, FP32
+// 12-real: 396 -> 291 us a call, 16^4: 83 -> 58 us; bound by the FMAs of its ten full
+// products a plane and the twelve link loads that feed them).
 template <class T, int NP>
 __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 1 : 4) k_clover(Links<T, NP> A, Geom g, int m, double* __restrict__ partials,
                                                                        const int* __restrict__ gate) {
@@ -47,18 +48,19 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 1 : 4) k_clover(Links<T,
     }
 }
 
-int clover_partials(const mgq_lattice* lat, const void* lines, int m, double* partials, const int* gate, cudaStream_t st) {
+int clover_partials(const mgq_lattice* lat, int m, double* partials, const int* gate, cudaStream_t st) {
     const Geom g = make_geom(lat->dims);
     const int nb = reduction_blocks(g.V, 128);  // at most 1184: 2 x 3 x 1184 partial sums
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
-        k_clover<T, NP><<<dim3(nb, 3), 128, 0, st>>>(links_at<T, NP>(const_cast<void*>(lines), lat->dims), g, m, partials, gate);
+        if (m == 1) k_clover<T, NP><<<dim3(nb, 3), 128, 0, st>>>(links_of<T, NP>(lat), g, 1, partials, gate);
+        else k_clover<T, 9><<<dim3(nb, 3), 128, 0, st>>>(links_at<T, 9>(ws_lines(lat), lat->dims), g, m, partials, gate);
     });
     return 3 * nb;
 }
 
 mgq_status clover_into(const mgq_lattice* lat, double* partials, double* dev_out, cudaStream_t st) {
     const Geom g = make_geom(lat->dims);
-    const int nb = clover_partials(lat, lat->links, 1, partials, nullptr, st);
+    const int nb = clover_partials(lat, 1, partials, nullptr, st);
     launch_final_sum2(partials, nb, 1.0 / (double)g.V, 1.0, dev_out, st);
     return cuda_check("clover");
 }

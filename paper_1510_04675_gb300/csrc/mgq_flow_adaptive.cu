@@ -218,7 +218,7 @@ mgq_status mgq_wilson_flow_adaptive(mgq_lattice* lat, double t_end, double tol, 
     const size_t nwords = links_bytes(lat) / 16;
 
     auto next = [&]() {
-        const int nb = clover_partials(lat, lat->links, 1, partials, &c->meas, st);
+        const int nb = clover_partials(lat, 1, partials, &c->meas, st);
         launch_pdl(k_adapt_next, 1, 512, st, c, partials, nb, invV, meas, t_end, eps_max, dt_meas, nm);
     };
     auto trial = [&]() {

@@ -47,6 +47,10 @@ inline double* ws_partials(const mgq_lattice* lat) { return reinterpret_cast<dou
 inline double* ws_scalars(const mgq_lattice* lat) { return reinterpret_cast<double*>((char*)lat->work + WS_SCALARS); }
 inline void* ws_links(const mgq_lattice* lat) { return (char*)lat->work + WS_LINKS; }
 inline void* ws_alg(const mgq_lattice* lat) { return (char*)lat->work + ws_alg_offset(lat); }
+// line fields (line_field): full matrices whatever the links' format, from the link copy
+// on; beside 12-real links they reach into the algebra field, which follows it (12 + 8
+// reals a link for 18)
+inline void* ws_lines(const mgq_lattice* lat) { return ws_links(lat); }
 
 // Validates a lattice descriptor; need_work additionally checks the workspace.
 mgq_status check_lattice(const mgq_lattice* lat, bool need_work, const char* fn);
@@ -106,13 +110,14 @@ mgq_status exp_update_to(const mgq_lattice* lat, void* links_out, void* B, doubl
 // E (site average) and Q of the clover field strength into dev_out[0], dev_out[1]
 mgq_status clover_into(const mgq_lattice* lat, double* partials, double* dev_out, cudaStream_t st);
 // Per-block E and Q partial sums (E at partials[0..nb), Q at partials[nb..2nb)) of
-// the clover with lines of m links a side at `lines` (the links, or line_field's
-// products); skipped when gate != nullptr and *gate == 0.  Returns nb.
-int clover_partials(const mgq_lattice* lat, const void* lines, int m, double* partials, const int* gate, cudaStream_t st);
-// lines_out <- the products of m links in every direction, lines_out(x) =
-// lines_in(x) U(x + m - 1): lines_in holds those of m - 1 links (the links for
-// m = 2) and may be lines_out itself
-void line_field(const mgq_lattice* lat, const void* lines_in, void* lines_out, int m, cudaStream_t st);
+// the clover with lines of m links a side (m = 1: the links; m > 1: the lines that
+// line_field left in the workspace); skipped when gate != nullptr and *gate == 0.
+// Returns nb.
+int clover_partials(const mgq_lattice* lat, int m, double* partials, const int* gate, cudaStream_t st);
+// The workspace's line field <- the products of m links in every direction, lines(x)
+// = lines(x) U(x + m - 1) from those of m - 1 links (m = 2: from the links).  All three
+// rows are kept: rebuilt from the other two, row 2 would carry their roundings.
+void line_field(const mgq_lattice* lat, int m, cudaStream_t st);
 
 inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 

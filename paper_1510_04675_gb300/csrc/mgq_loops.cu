@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(128) k_wilson_loop(Links<T, NP> U, Geom g, int
 // with the 2x2 loops multiplied out link by link and thirds taken in FP64 per loop,
 // now 177 us after 40 us for the lines.
 template <class T, int NP>
-__global__ void __launch_bounds__(128) k_partial_loops(Links<T, NP> U, Links<T, NP> U2, Geom g, double* __restrict__ partials) {
+__global__ void __launch_bounds__(128) k_partial_loops(Links<T, NP> U, Links<T, 9> U2, Geom g, double* __restrict__ partials) {
     const int mu = plane_mu(blockIdx.y), nu = plane_nu(blockIdx.y);
     double a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     T least = T(3);
@@ -176,9 +176,9 @@ mgq_status mgq_partial_loops(const mgq_lattice* lat, double* out, void* stream) 
     int nbx = reduction_blocks(g.V, 128);
     if (nbx > (int)(WS_NPARTIALS / 54)) nbx = (int)(WS_NPARTIALS / 54);
     const int nb = 6 * nbx;
-    line_field(lat, lat->links, ws_links(lat), 2, st);
+    line_field(lat, 2, st);
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
-        k_partial_loops<T, NP><<<dim3(nbx, 6), 128, 0, st>>>(links_of<T, NP>(lat), links_at<T, NP>(ws_links(lat), lat->dims), g,
+        k_partial_loops<T, NP><<<dim3(nbx, 6), 128, 0, st>>>(links_of<T, NP>(lat), links_at<T, 9>(ws_lines(lat), lat->dims), g,
                                                              ws_partials(lat));
     });
     double* sc = ws_scalars(lat);

@@ -265,6 +265,23 @@ __device__ __forceinline__ M3<T> staple(const Links<T, NP>& U, const Geom& g, co
     else return staple_full(U, g, x, h, mu, par);
 }
 
+// One upper term a b^+ c^+ and one lower term (e d)^+ f of the staple, the left factors'
+// rows 0, 1 given: rows 0, 1 of every partial product, row 2 rebuilt; FMA as in two_rows.
+template <bool FMA = false>
+__device__ __forceinline__ M3<float> up_term(const M3<float>& a_rows, const M3<float>& b, const M3<float>& c) {
+    M3<float> r = mul_nd_2<FMA>(mul_nd_2<FMA>(a_rows, b), c);
+    rebuild_row2(r);
+    return r;
+}
+template <bool FMA = false>
+__device__ __forceinline__ M3<float> down_term(const M3<float>& e_rows, const M3<float>& d, const M3<float>& f) {
+    M3<float> t = mul_nn_2<FMA>(e_rows, d);
+    rebuild_row2(t);
+    M3<float> r = mul_dn_2<FMA>(t, f);
+    rebuild_row2(r);
+    return r;
+}
+
 // =============================================================== plaquette
 // Per site: sum over mu < nu < ND of Re Tr[U_mu(x) U_nu(x+mu) (U_nu(x) U_mu(x+nu))^+]
 // (ND = 4: all six planes; ND = 3: the planes of directions 0, 1, 2).
@@ -317,33 +334,6 @@ __device__ __forceinline__ double site_plaquettes(const Links<T, NP>& U, const G
 // written for a line field A_d(x) (the links, or products of m links) whose hops H
 // are the lines' lengths; op is the parity one line away.
 
-// a b^+ c^+ and (e d)^+ f of lines in SU(3).  FP32: rows 0, 1 of every partial
-// product, row 2 rebuilt; FMA as in two_rows.
-template <bool FMA = false, class T> __device__ __forceinline__ M3<T> up_term(const M3<T>& a_rows, const M3<T>& b, const M3<T>& c) {
-    if constexpr (sizeof(T) == 4) {
-        M3<T> r = mul_nd_2<FMA>(mul_nd_2<FMA>(a_rows, b), c);
-        rebuild_row2(r);
-        return r;
-    } else {
-        return mul_nd(mul_nd(a_rows, b), c);
-    }
-}
-template <bool FMA = false, class T> __device__ __forceinline__ M3<T> down_term(const M3<T>& e_rows, const M3<T>& d, const M3<T>& f) {
-    if constexpr (sizeof(T) == 4) {
-        M3<T> t = mul_nn_2<FMA>(e_rows, d);
-        rebuild_row2(t);
-        M3<T> r = mul_dn_2<FMA>(t, f);
-        rebuild_row2(r);
-        return r;
-    } else {
-        return mul_dn(mul_nn(e_rows, d), f);
-    }
-}
-// a link that enters as a left factor: FP32 needs its rows 0, 1 only
-template <class T, int NP> __device__ __forceinline__ M3<T> load_left(const Links<T, NP>& U, int mu, int par, int h) {
-    if constexpr (sizeof(T) == 4) return U.load_rows(mu, par, h);
-    else return U.load(mu, par, h);
-}
 template <class T> __device__ __forceinline__ void acc_sub(M3<T>& a, const M3<T>& b) {
 #pragma unroll
     for (int i = 0; i < 3; i++)
@@ -358,24 +348,25 @@ template <class T> __device__ __forceinline__ void acc_sub(M3<T>& a, const M3<T>
 // for that link:
 //   l1 - l4^+ = U_mu(x) [U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+ - U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu)]
 //   l2 - l3^+ = [U_nu(x) U_mu(x-mu+nu)^+ U_nu(x-mu)^+ - U_nu(x-nu)^+ U_mu(x-mu-nu)^+ U_nu(x-mu-nu)] U_mu(x-mu)
-// ten products, eight of them in two-row form in FP32, where four separate leaves
-// take twelve full ones.
+// ten products where four separate leaves take twelve.  All three rows are multiplied
+// out: rows 0, 1 with row 2 = conj(row0 x row1) would be an eighth less work, but row 2
+// then carries the roundings of the other two, and matrices off SU(3) another value.
 template <class T, int NP>
 __device__ __forceinline__ void clover_coeffs(const Links<T, NP>& U, const Hops& H, int par, int op, int mu, int nu, T out[8]) {
     const int fm = pick(H.fwd, mu), fn = pick(H.fwd, nu), bm = pick(H.bwd, mu), bn = pick(H.bwd, nu);
     const int x = H.lex;
-    M3<T> Q;
-    {
-        M3<T> D = up_term<true>(load_left(U, nu, op, (x + fm) >> 1), U.load(mu, op, (x + fn) >> 1), U.load(nu, par, x >> 1));
-        acc_sub(D, down_term<true>(load_left(U, mu, op, (x + bn) >> 1), U.load(nu, par, (x + fm + bn) >> 1), U.load(nu, op, (x + bn) >> 1)));
-        Q = mul_nn(U.load(mu, par, x >> 1), D);
-    }
-    {
-        M3<T> D = up_term<true>(load_left(U, nu, par, x >> 1), U.load(mu, par, (x + bm + fn) >> 1), U.load(nu, op, (x + bm) >> 1));
-        acc_sub(D, down_term<true>(load_left(U, mu, par, (x + bm + bn) >> 1), U.load(nu, op, (x + bn) >> 1),
-                             U.load(nu, par, (x + bm + bn) >> 1)));
-        acc_add(Q, mul_nn(D, U.load(mu, op, (x + bm) >> 1)));
-    }
+    // a b^+ c^+ - (e d)^+ f
+    auto sides = [](const M3<T>& a, const M3<T>& b, const M3<T>& c, const M3<T>& e, const M3<T>& d, const M3<T>& f) {
+        M3<T> D = mul_nd(mul_nd(a, b), c);
+        acc_sub(D, mul_dn(mul_nn(e, d), f));
+        return D;
+    };
+    M3<T> Q = mul_nn(U.load(mu, par, x >> 1),
+                     sides(U.load(nu, op, (x + fm) >> 1), U.load(mu, op, (x + fn) >> 1), U.load(nu, par, x >> 1),
+                           U.load(mu, op, (x + bn) >> 1), U.load(nu, par, (x + fm + bn) >> 1), U.load(nu, op, (x + bn) >> 1)));
+    acc_add(Q, mul_nn(sides(U.load(nu, par, x >> 1), U.load(mu, par, (x + bm + fn) >> 1), U.load(nu, op, (x + bm) >> 1),
+                            U.load(mu, par, (x + bm + bn) >> 1), U.load(nu, op, (x + bn) >> 1), U.load(nu, par, (x + bm + bn) >> 1)),
+                      U.load(mu, op, (x + bm) >> 1)));
     ta_coeffs(Q, out);
 #pragma unroll
     for (int a = 0; a < 8; a++) out[a] *= T(0.25);
@@ -385,6 +376,11 @@ __device__ __forceinline__ void clover_coeffs(const Links<T, NP>& U, const Hops&
 __device__ __forceinline__ int dual_mu(int p) { return p == 0 ? 2 : 1; }
 __device__ __forceinline__ int dual_nu(int p) { return p == 2 ? 2 : 3; }
 
+// a link that enters as a left factor: FP32 needs its rows 0, 1 only
+template <class T, int NP> __device__ __forceinline__ M3<T> load_left(const Links<T, NP>& U, int mu, int par, int h) {
+    if constexpr (sizeof(T) == 4) return U.load_rows(mu, par, h);
+    else return U.load(mu, par, h);
+}
 // Re Tr of the loop A_mu(x) A_nu(x+mu) (A_nu(x) A_mu(x+nu))^+ of SU(3) lines.  FP32:
 // a = A_mu(x) A_nu(x+mu) and b = A_nu(x) A_mu(x+nu) are in SU(3), so rows 0, 1 of
 // each suffice: with s_ij = row_i(a) . conj(row_j(b)), Tr(a b^+) = s00 + s11 +

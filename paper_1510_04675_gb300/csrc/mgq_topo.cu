@@ -12,35 +12,31 @@
 namespace mgq {
 
 // The m x m leaves are the 1 x 1 leaves of the field of straight lines of m links,
-// which one pass per m extends by a link (line_field, into the workspace's link
-// copy): a leaf is four line loads instead of 4 m link products (24^3x48, FP32
-// 12-real, the three charges: 4.83 ms -> 0.82 ms, of which 3 x 245 us for the
-// clovers and 2 x 40 us for the lines).
-
-template <class T, int NP>
-__global__ void __launch_bounds__(128) k_line_extend(Links<T, NP> U, Links<T, NP> in, Links<T, NP> out, Geom g, int len) {
+// which one pass per m extends by a link (line_field, in the workspace): a leaf is four
+// line loads instead of 4 m link products (24^3x48, FP32 12-real, the three charges:
+// 4.92 ms with every leaf multiplied out, now 0.94 ms; 0.81 ms with rows 0, 1 of the
+// products only, which left 10 to 40 % more rounding error in the flowed E and the
+// charges).
+// NPI: planes of the lines extended, those of the links for the first pass.
+template <class T, int NP, int NPI>
+__global__ void __launch_bounds__(128) k_line_extend(Links<T, NP> U, Links<T, NPI> in, Links<T, 9> out, Geom g, int len) {
     const int mu = blockIdx.y >> 1, par = blockIdx.y & 1, h = blockIdx.x * blockDim.x + threadIdx.x;
     if (h >= g.Vh) return;
     int x[4];
     cb_coords(g, par, h, x);
     const Hops H = make_hops(g, x, len);
     const M3<T> u = U.load(mu, par ^ (len & 1), (H.lex + pick(H.fwd, mu)) >> 1);
-    M3<T> r;
-    if constexpr (sizeof(T) == 4) {
-        r = mul_nn_2(in.load_rows(mu, par, h), u);
-        rebuild_row2(r);
-    } else {
-        r = mul_nn(in.load(mu, par, h), u);
-    }
-    out.store(mu, par, h, r);
+    out.store(mu, par, h, mul_nn(in.load(mu, par, h), u));
 }
 
-void line_field(const mgq_lattice* lat, const void* lines_in, void* lines_out, int m, cudaStream_t st) {
+void line_field(const mgq_lattice* lat, int m, cudaStream_t st) {
     const Geom g = make_geom(lat->dims);
     dispatch_prec(lat->prec, [&]<class T, int NP>() {
-        k_line_extend<T, NP><<<dim3((g.Vh + 127) / 128, 8), 128, 0, st>>>(
-            links_of<T, NP>(lat), links_at<T, NP>(const_cast<void*>(lines_in), lat->dims), links_at<T, NP>(lines_out, lat->dims),
-            g, m - 1);
+        const dim3 grid((g.Vh + 127) / 128, 8);
+        const Links<T, NP> U = links_of<T, NP>(lat);
+        const Links<T, 9> lines = links_at<T, 9>(ws_lines(lat), lat->dims);
+        if (m == 2) k_line_extend<T, NP, NP><<<grid, 128, 0, st>>>(U, U, lines, g, 1);
+        else k_line_extend<T, NP, 9><<<grid, 128, 0, st>>>(U, lines, lines, g, m - 1);
     });
 }
 
@@ -51,13 +47,9 @@ __global__ void k_improved_combine(double* out) {
 
 // {Q_improved, Q_1x1, Q_2x2, Q_3x3} into dev_out[0..3] (device)
 mgq_status improved_charge_into(const mgq_lattice* lat, double* partials, double* dev_out, cudaStream_t st) {
-    const void* lines = lat->links;
     for (int m = 1; m <= 3; m++) {
-        if (m > 1) {
-            line_field(lat, lines, ws_links(lat), m, st);
-            lines = ws_links(lat);
-        }
-        const int nb = clover_partials(lat, lines, m, partials, nullptr, st);
+        if (m > 1) line_field(lat, m, st);
+        const int nb = clover_partials(lat, m, partials, nullptr, st);
         launch_final_sum(partials + nb, nb, 1.0, dev_out + m, st);
     }
     k_improved_combine<<<1, 1, 0, st>>>(dev_out);
