@@ -71,6 +71,11 @@ typedef enum {
     MGQ_ENONUNITARY = 6     /* mgq_check_unitarity found a link off SU(3)         */
 } mgq_status;
 
+/* Storage and arithmetic of the links.  MGQ_F32_C12 keeps rows 0 and 1; row 2 is
+ * conj(row0 x row1).  In both FP32 formats the sub-sweeps, plaquette, force, flow
+ * and prolongation take every link for an SU(3) matrix (row 2 of a product comes
+ * from its rows 0 and 1); the loops, the clover observables and the
+ * vector-Jacobian products multiply the matrices as they are. */
 typedef enum { MGQ_F64 = 0, MGQ_F32 = 1, MGQ_F32_C12 = 2 } mgq_prec;
 typedef enum { MGQ_WILSON = 0 } mgq_action;               /* the paper's action (Sec. III) */
 typedef enum { MGQ_PERIODIC = 0, MGQ_OPEN = 1 } mgq_bc;   /* periodic only (Sec. IV.A)    */

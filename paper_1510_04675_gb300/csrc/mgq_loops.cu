@@ -8,15 +8,12 @@
 namespace mgq {
 
 // P <- P times the `len` links in direction mu from the site (lexicographic index
-// lex, coordinate c along mu, parity par) on, which move along.  FP32: rows 0, 1
-// of P (a left factor throughout).
+// lex, coordinate c along mu, parity par) on, which move along.
 template <class T, int NP>
 __device__ __forceinline__ void extend_line(M3<T>& P, const Links<T, NP>& U, int mu, int len, int L, int stride, int& lex,
                                             int& c, int& par) {
     for (int k = 0; k < len; k++) {
-        const M3<T> u = U.load(mu, par, lex >> 1);
-        if constexpr (sizeof(T) == 4) P = mul_nn_2(P, u);
-        else P = mul_nn(P, u);
+        P = mul_nn(P, U.load(mu, par, lex >> 1));
         const bool last = ++c == L;
         lex += last ? stride * (1 - L) : stride;
         if (last) c = 0;
@@ -31,7 +28,7 @@ __device__ __forceinline__ M3<T> corner_path(const Links<T, NP>& U, const Geom& 
     const int st[4] = {1, g.L[0], g.L[0] * g.L[1], g.L[0] * g.L[1] * g.L[2]};
     const int smu = pick(st, mu), Lmu = pick(g.L, mu);
     int lex = lex_of(g, x), c = pick(x, mu);
-    M3<T> P = load_left(U, mu, par, lex >> 1);
+    M3<T> P = U.load(mu, par, lex >> 1);
     const bool last = ++c == Lmu;
     lex += last ? smu * (1 - Lmu) : smu;
     if (last) c = 0;
@@ -46,8 +43,10 @@ __device__ __forceinline__ int plane_mu(int p) { return p < 3 ? 0 : (p < 5 ? 1 :
 __device__ __forceinline__ int plane_nu(int p) { return p < 3 ? p + 1 : (p < 5 ? p - 1 : 3); }
 
 // Re Tr L^m_mu(x) L^n_nu(x+m mu) [L^n_nu(x) L^m_mu(x+n nu)]^+, one thread per site
-// and plane (block row y): two paths of m + n links, FP32 in two rows throughout
-// (2x3 loops of 24^3x48, FP32 12-real: 355 -> 176 us)
+// and plane (block row y): two paths of m + n links, all rows multiplied out (2x3 loops
+// of 24^3x48, FP32 12-real, a call: 383 us with a thread for a site's six planes, 296
+// us so; 209 us with rows 0, 1 of the paths only, which added 10 to 30 % to the rounding
+// error of the loops)
 template <class T, int NP>
 __global__ void __launch_bounds__(128) k_wilson_loop(Links<T, NP> U, Geom g, int m, int n, double* __restrict__ partials) {
     const int mu = plane_mu(blockIdx.y), nu = plane_nu(blockIdx.y);
@@ -57,8 +56,7 @@ __global__ void __launch_bounds__(128) k_wilson_loop(Links<T, NP> U, Geom g, int
         int x[4];
         cb_coords(g, par, h, x);
         const M3<T> a = corner_path(U, g, x, par, mu, m, nu, n), b = corner_path(U, g, x, par, nu, n, mu, m);
-        if constexpr (sizeof(T) == 4) acc += (double)retr_two_row(a, b);
-        else acc += retr_nd(a, b);
+        acc += (double)retr_nd(a, b);
     }
     acc = block_sum(acc);
     if (threadIdx.x == 0) partials[blockIdx.y * gridDim.x + blockIdx.x] = acc;
@@ -67,11 +65,12 @@ __global__ void __launch_bounds__(128) k_wilson_loop(Links<T, NP> U, Geom g, int
 // 8 class sums of Re Tr (1x1 loops by chi_munu = 0..2, 2x2 loops by chi = 0..4) and
 // the least Re Tr of the 1x1 loops: partials[q * nb + block] for q = 0..7, minima in
 // partials[8 * nb + block], nb = gridDim.x * 6.  One thread per site and plane
-// (block row y); U2 holds the lines of two links.  24^3x48, FP32 12-real: 571 us
-// with the 2x2 loops multiplied out link by link and thirds taken in FP64 per loop,
-// now 177 us after 40 us for the lines.
+// (block row y); U2 holds the lines of two links.  24^3x48, a call: FP32 12-real 634 us
+// with the 2x2 loops multiplied out link by link and thirds taken in FP64 per loop, now
+// 299 us, of which 40 us for the lines; 18-real 647 -> 326 us (538 us where the compiler
+// is left to choose 96 registers).
 template <class T, int NP>
-__global__ void __launch_bounds__(128) k_partial_loops(Links<T, NP> U, Links<T, 9> U2, Geom g, double* __restrict__ partials) {
+__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 1 : 4) k_partial_loops(Links<T, NP> U, Links<T, 9> U2, Geom g, double* __restrict__ partials) {
     const int mu = plane_mu(blockIdx.y), nu = plane_nu(blockIdx.y);
     double a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     T least = T(3);

@@ -376,15 +376,17 @@ __device__ __forceinline__ void clover_coeffs(const Links<T, NP>& U, const Hops&
 __device__ __forceinline__ int dual_mu(int p) { return p == 0 ? 2 : 1; }
 __device__ __forceinline__ int dual_nu(int p) { return p == 2 ? 2 : 3; }
 
-// a link that enters as a left factor: FP32 needs its rows 0, 1 only
-template <class T, int NP> __device__ __forceinline__ M3<T> load_left(const Links<T, NP>& U, int mu, int par, int h) {
-    if constexpr (sizeof(T) == 4) return U.load_rows(mu, par, h);
-    else return U.load(mu, par, h);
+// Re Tr of the loop A_mu(x) A_nu(x+mu) (A_nu(x) A_mu(x+nu))^+ of lines A.
+template <class T, int NP>
+__device__ __forceinline__ T loop_retr(const Links<T, NP>& U, const Hops& H, int par, int op, int mu, int nu) {
+    const int x = H.lex >> 1, xm = (H.lex + pick(H.fwd, mu)) >> 1, xn = (H.lex + pick(H.fwd, nu)) >> 1;
+    const M3<T> a = mul_nn(U.load(mu, par, x), U.load(nu, op, xm));
+    return retr_nd(a, mul_nn(U.load(nu, par, x), U.load(mu, op, xn)));
 }
-// Re Tr of the loop A_mu(x) A_nu(x+mu) (A_nu(x) A_mu(x+nu))^+ of SU(3) lines.  FP32:
-// a = A_mu(x) A_nu(x+mu) and b = A_nu(x) A_mu(x+nu) are in SU(3), so rows 0, 1 of
-// each suffice: with s_ij = row_i(a) . conj(row_j(b)), Tr(a b^+) = s00 + s11 +
-// conj(s00 s11 - s01 s10) (row 2 = conj(row0 x row1); Binet-Cauchy).
+
+// The plaquette of FP32 links in SU(3): rows 0, 1 of a = U_mu(x) U_nu(x+mu) and b =
+// U_nu(x) U_mu(x+nu) suffice: with s_ij = row_i(a) . conj(row_j(b)), Tr(a b^+) = s00 +
+// s11 + conj(s00 s11 - s01 s10) (row 2 = conj(row0 x row1); Binet-Cauchy).
 __device__ __forceinline__ float retr_two_row(const M3<float>& a, const M3<float>& b) {
     Cx<float> sij[2][2];
 #pragma unroll
@@ -395,16 +397,11 @@ __device__ __forceinline__ float retr_two_row(const M3<float>& a, const M3<float
     const Cx<float> d = sij[0][0] * sij[1][1] - sij[0][1] * sij[1][0];
     return sij[0][0].re + sij[1][1].re + d.re;
 }
-template <class T, int NP>
-__device__ __forceinline__ T loop_retr(const Links<T, NP>& U, const Hops& H, int par, int op, int mu, int nu) {
+template <int NP>
+__device__ __forceinline__ float plaquette_retr(const Links<float, NP>& U, const Hops& H, int par, int op, int mu, int nu) {
     const int x = H.lex >> 1, xm = (H.lex + pick(H.fwd, mu)) >> 1, xn = (H.lex + pick(H.fwd, nu)) >> 1;
-    if constexpr (sizeof(T) == 4) {
-        const M3<T> a = mul_nn_2<NP == 9>(U.load_rows(mu, par, x), U.load(nu, op, xm));
-        return retr_two_row(a, mul_nn_2<NP == 9>(U.load_rows(nu, par, x), U.load(mu, op, xn)));
-    } else {
-        const M3<T> a = mul_nn(U.load(mu, par, x), U.load(nu, op, xm));
-        return retr_nd(a, mul_nn(U.load(nu, par, x), U.load(mu, op, xn)));
-    }
+    const M3<float> a = mul_nn_2<NP == 9>(U.load_rows(mu, par, x), U.load(nu, op, xm));
+    return retr_two_row(a, mul_nn_2<NP == 9>(U.load_rows(nu, par, x), U.load(mu, op, xn)));
 }
 
 // =============================================================== SU(2) steps

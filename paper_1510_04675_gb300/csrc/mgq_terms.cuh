@@ -87,7 +87,7 @@ __device__ __forceinline__ void update_terms(const Links<float, NP>& U, const Ge
     } else if (KIND == TERMS_OVERRELAX_LAST && h0 < g.Vh) {
         // planes 01, 02, 12
         for (int p = w - 1; p < 3; p += WARPS - 1)
-            acc += (double)loop_retr(U, H, par, par ^ 1, p == 2 ? 1 : 0, p == 0 ? 1 : 2);
+            acc += (double)plaquette_retr(U, H, par, par ^ 1, p == 2 ? 1 : 0, p == 0 ? 1 : 2);
     }
     if constexpr (KIND == TERMS_OVERRELAX_LAST) {
         acc = block_sum(acc);

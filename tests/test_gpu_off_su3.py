@@ -53,3 +53,16 @@ def test_clover_gradient_off_su3(gpu, orc, prec, obs):
         gpu.mgq_clover_vjp(lat, obs, 1.0, lam)
         grads[p] = gpu.alg_to_numpy(lat, lam)
     assert np.max(np.abs(grads[prec] - grads["f64"])) < 1.3e-5 * np.max(np.abs(grads["f64"]))
+
+
+# a 4x3 loop is a chain of 14 products and a trace, 15 x 3 x 2^-24 = 2.7e-6 of matrices grown by up to 2, averaged over
+# sites and planes; h takes three times the largest single loop's
+@pytest.mark.parametrize("dims", DIMS)
+@pytest.mark.parametrize("prec", ["f64", "f32", "f32c12"])
+def test_loops_off_su3(gpu, orc, dims, prec):
+    U, tol = _field(orc, dims, prec), 1e-12 if prec == "f64" else 5.4e-6
+    lat = gpu.Lattice(dims, prec)
+    lat.from_numpy(U)
+    for m, n in [(1, 1), (2, 1), (2, 3), (1, 5), (4, 3)]:
+        assert abs(gpu.mgq_wilson_loop(lat, m, n) - orc.wilson_loop(U, dims, m, n)) < tol
+    assert np.max(np.abs(gpu.mgq_partial_loops(lat) - orc.partial_loops(U, dims))) < 3 * tol
