@@ -145,6 +145,14 @@ __device__ __forceinline__ M3<T> psi_at(const Alg<T>& P, int mu, int par, int h)
 // insertion at a time, summed; the insertion at m itself is the self term
 // -TA(W_m A_m Psi_m), A_m the staple.
 
+template <class T> __device__ __forceinline__ M3<T> zero3() {
+    M3<T> r;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) r.e[i][j] = mk(T(0), T(0));
+    return r;
+}
 template <class T> __device__ __forceinline__ M3<T> msub(const M3<T>& a, const M3<T>& b) {
     M3<T> r;
 #pragma unroll
@@ -163,12 +171,14 @@ template <class T> __device__ __forceinline__ M3<T> msub(const M3<T>& a, const M
 // each summed by the product rule over the running prefix, plus the staples'
 // share of the self term: scale * (-TA(U_m (sum_nu R_up + R_dn + A Psi_m))), A = sum_nu
 // (X1 X2 X3 + Y1 Y2 Y3).  X1 X2 X3 Psi_m folds into the last insertion of R_up (both
-// Psi at y); the lower staples are summed and multiplied by Psi_m once.  The planes
-// run in a rolled loop, a plane's two sides one after the other, so that the live
-// matrices stay in registers, and the four warps of a block take the four
+// Psi at y); the lower staples are summed and multiplied by Psi_m once.  The upper
+// sides of the three planes are summed and taken to the algebra first, then the lower
+// ones: one running sum over all of them has the larger partial sums (FP32 error
+// against FP64 8.5e-8, a sum per side 8.0e-8).  The planes run in rolled loops, so that
+// the live matrices stay in registers, and the four warps of a block take the four
 // directions at the same 32 sites, whose links and cotangents they share in L1.
-// 16^4, FP32 12-real: 74 us as two launches (a side each, with its own pass over
-// Lam, U_m and Psi_m), 59 us so.
+// 16^4, FP32 12-real: 72 us as two launches (a side each, with its own pass over Lam),
+// 60 us so, 58 us with the one sum.
 template <class T, int NP>
 __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 1 : 3) k_flow_vjp(Links<T, NP> U, Geom g, Alg<T> Psi, T scl, Alg<T> Lam) {
     const int rho = threadIdx.x >> 5, par = blockIdx.y, op = par ^ 1, h = blockIdx.x * 32 + (threadIdx.x & 31);
@@ -177,15 +187,12 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 1 : 3) k_flow_vjp(Links<
     cb_coords(g, par, h, x);
     const Hops H = make_hops(g, x);
     const int frho = pick(H.fwd, rho);
-    M3<T> Rs, As;
-#pragma unroll
-    for (int i = 0; i < 3; i++)
-#pragma unroll
-        for (int j = 0; j < 3; j++) Rs.e[i][j] = As.e[i][j] = mk(T(0), T(0));
+    T t[8], td[8];
+    {
+        M3<T> Rs = zero3<T>();
 #pragma unroll 1
-    for (int K = 0; K < 3; K++) {
-        const int nu = K < rho ? K : K + 1;
-        {
+        for (int K = 0; K < 3; K++) {
+            const int nu = K < rho ? K : K + 1;
             const int h_pr = (H.lex + frho) >> 1;             // y + rho  (op)
             const int h_pn = (H.lex + pick(H.fwd, nu)) >> 1;  // y + nu   (op)
             const M3<T> X1 = U.load(nu, op, h_pr);
@@ -194,16 +201,23 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 1 : 3) k_flow_vjp(Links<
             const M3<T> P2 = mul_nd(X1, X2d);         // X1 X2
             const M3<T> S = mul_nd(P2, X3d);          // X1 X2 X3, the upper staple
             // R_up + S Psi_m = Psi_nu(y+rho) S - (X1 X2 Psi_rho(y+nu)) X3 - S (Psi_nu(y) - Psi_m)
-            acc_sub(Rs, mul_nd(mul_nn(P2, psi_at<T, NP>(Psi, rho, op, h_pn)), X3d));
-            acc_add(Rs, mul_nn(psi_at<T, NP>(Psi, nu, op, h_pr), S));
+            M3<T> R = mul_nn(psi_at<T, NP>(Psi, nu, op, h_pr), S);
+            acc_sub(R, mul_nd(mul_nn(P2, psi_at<T, NP>(Psi, rho, op, h_pn)), X3d));
             T cn[8], cm[8];
             Psi.load(nu, par, h, cn);
             Psi.load(rho, par, h, cm);
 #pragma unroll
             for (int a = 0; a < 8; a++) cn[a] -= cm[a];
-            acc_sub(Rs, mul_nn(S, alg_matrix(cn)));
+            acc_sub(R, mul_nn(S, alg_matrix(cn)));
+            acc_add(Rs, R);
         }
-        {
+        ta_coeffs(mul_nn(U.load(rho, par, h), Rs), t);
+    }
+    {
+        M3<T> Rs = zero3<T>(), As = zero3<T>();
+#pragma unroll 1
+        for (int K = 0; K < 3; K++) {
+            const int nu = K < rho ? K : K + 1;
             const int bnu = pick(H.bwd, nu);
             const int h_mn = (H.lex + bnu) >> 1;            // y - nu        (op)
             const int h_mn_pr = (H.lex + bnu + frho) >> 1;  // y - nu + rho  (par)
@@ -222,13 +236,12 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 1 : 3) k_flow_vjp(Links<
             acc_add(Rs, mul_nn(Q, Y3));
             acc_add(As, mul_nn(P2, Y3));                 // Y1 Y2 Y3, the lower staple
         }
+        acc_add(Rs, mul_nn(As, psi_at<T, NP>(Psi, rho, par, h)));  // the lower staples' share of the self term
+        ta_coeffs(mul_nn(U.load(rho, par, h), Rs), td);
     }
-    acc_add(Rs, mul_nn(As, psi_at<T, NP>(Psi, rho, par, h)));  // the lower staples' share of the self term
-    T t[8];
-    ta_coeffs(mul_nn(U.load(rho, par, h), Rs), t);
     T* b = Lam.at(rho, par, h);
 #pragma unroll
-    for (int a = 0; a < 8; a++) b[a * Alg<T>::kStep] -= scl * t[a];
+    for (int a = 0; a < 8; a++) b[a * Alg<T>::kStep] -= scl * (t[a] + td[a]);
 }
 
 static inline int nblk(long n, int t) { return (int)((n + t - 1) / t); }
