@@ -53,14 +53,14 @@ __device__ __forceinline__ const Geom& geom_of(const LatDesc<T>& d) {
 // FP32 12-real links (staple_staged; the launch gives STAGED_THREADS threads and
 // STAGED_SMEM bytes), as in the single-lattice kernels, so that batched and
 // single-lattice updates agree bit for bit; plain loads otherwise.
-// early() and PACKED as in staple_staged (48 uneven lattices, one compound sweep: 3.05 ->
+// early(), PACKED and FMA as in staple_staged (48 uneven lattices, one compound sweep: 3.05 ->
 // 2.99 ms with the draws early and single-FMA rotations).
-template <class T, int NP, int MU, bool PACKED = false, class Work = NoWork>
+template <class T, int NP, int MU, bool PACKED = false, bool FMA = true, class Work = NoWork>
 __device__ __forceinline__ void staple_and_link(const Links<T, NP>& U, const Geom& g, const int x[4], int h, int par,
                                                 M3<T>& A, M3<T>& u, Work early = Work()) {
     if constexpr (sizeof(T) == 4 && NP == 6) {
         extern __shared__ float4 staged_sm[];
-        A = staple_staged<PACKED>(U, g, x, h, MU, par, staged_sm, u, early);
+        A = staple_staged<PACKED, FMA>(U, g, x, h, MU, par, staged_sm, u, early);
     } else {
         A = staple(U, g, x, h, MU, par);
         u = U.load(MU, par, h);
@@ -102,8 +102,10 @@ __global__ void __launch_bounds__(BATCH_THREADS, NHB1 ? batch_blocks<T, NP>() : 
         });
         hb_link_drawn(u, A, d.beta, r);
     } else {
-        staple_and_link<T, NP, MU>(U, g, x, h, par, A, u);
-        hb_link<(NP == 9)>(u, A, d.beta, n_hb, rk, lex, (uint32_t)MU, (uint8_t*)nullptr);
+        // packed throughout: beside the attempt loop single FMAs cost more (24 lattices of
+        // 8^3x16 to 16^4, three attempts: 456 us a sweep against 430)
+        staple_and_link<T, NP, MU, true, false>(U, g, x, h, par, A, u);
+        hb_link<true>(u, A, d.beta, n_hb, rk, lex, (uint32_t)MU, (uint8_t*)nullptr);
     }
     U.store(MU, par, h, u);
 }

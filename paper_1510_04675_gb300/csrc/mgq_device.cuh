@@ -334,7 +334,9 @@ template <> __device__ __forceinline__ void rebuild_row2<float>(M3<float>& u) {
 }
 
 // The same on the packed FMA, row 1 entries paired (same bits): the better form in
-// the staged heat bath (54.7 us per 32^4 launch, 56.0 us with single FMAs).
+// the staged heat bath (54.7 us per 32^4 launch, 56.0 us with single FMAs) and in the
+// kernels with several attempts per subgroup (a three-attempt sweep of 8^4, 12-real:
+// 66 against 70 us).
 __device__ __forceinline__ void rebuild_row2_packed(M3<float>& u) {
     float2 B[3], iB[3];
 #pragma unroll
@@ -551,7 +553,8 @@ struct Links {
             m.e[(2 * k + 1) / 3][(2 * k + 1) % 3] = mk(v.z, v.w);
         }
     }
-    __device__ __forceinline__ M3<T> load(int mu, int par, int h) const {
+    // PACKED: the form of the row-2 rebuild (see rebuild_row2_packed)
+    template <bool PACKED = false> __device__ __forceinline__ M3<T> load(int mu, int par, int h) const {
         M3<T> m;
         if constexpr (kPaired) {
             load_pairs(mu, par, h, m);
@@ -562,7 +565,10 @@ struct Links {
 #pragma unroll
                 for (int c = 0; c < 3; c++) m.e[r][c] = ldg_cx(b + ((r * 3 + c) << 5));
         }
-        if (NP == 6) rebuild_row2(m);
+        if constexpr (NP == 6) {
+            if constexpr (PACKED) rebuild_row2_packed(m);
+            else rebuild_row2(m);
+        }
         return m;
     }
     // rows 0 and 1 only (row 2 left unset), for factors whose third row is not read

@@ -63,15 +63,15 @@ __device__ __forceinline__ M3<float> staple_two_row(const LinkField& U, const Ge
         const int hpm_mn = (H.lex + fmu + H.bwd[nu]) >> 1;
         M3<float> up, dn;
         {
-            M3<float> t = mul_nd_2(U.load_rows(nu, op, hpm), U.load(mu, op, hpn));
+            M3<float> t = mul_nd_2(U.load_rows(nu, op, hpm), U.template load<true>(mu, op, hpn));
             complete<true>(t);
-            up = mul_nd_2(t, U.load(nu, par, h));
+            up = mul_nd_2(t, U.template load<true>(nu, par, h));
             complete<true>(up);
         }
         {
-            M3<float> t = mul_nn_2(U.load_rows(mu, op, hmn), U.load(nu, par, hpm_mn));
+            M3<float> t = mul_nn_2(U.load_rows(mu, op, hmn), U.template load<true>(nu, par, hpm_mn));
             complete<true>(t);
-            dn = mul_dn_2(t, U.load(nu, op, hmn));
+            dn = mul_dn_2(t, U.template load<true>(nu, op, hmn));
             complete<true>(dn);
         }
         acc_add(A, up);
@@ -151,11 +151,11 @@ struct NoWork {
     __device__ void operator()() const {}
 };
 // early(): independent work that runs while the first loads are in flight; PACKED:
-// the form of the row-2 rebuilds.  The first product of a term is packed, the second
-// takes single FMAs: overrelaxation 44.5 -> 43.8 us per 32^4 launch, 16.0 -> 15.4 us at
-// 24^4, against packed products throughout (single FMAs throughout 15.9 us at 24^4 but
-// 50.3 us at 32^4).
-template <bool PACKED = false, class Work = NoWork>
+// the form of the row-2 rebuilds; FMA: that of a term's second product.  The first
+// product of a term is packed, the second takes single FMAs: overrelaxation 44.5 ->
+// 43.8 us per 32^4 launch, 16.0 -> 15.4 us at 24^4, against packed products throughout
+// (single FMAs throughout 15.9 us at 24^4 but 50.3 us at 32^4).
+template <bool PACKED = false, bool FMA = true, class Work = NoWork>
 __device__ __forceinline__ M3<float> staple_staged(const Links<float, 6>& U, const Geom& g, const int x[4], int h,
                                                    const int MU, int par, float4* sm, M3<float>& u,
                                                    Work early = Work()) {
@@ -205,11 +205,11 @@ __device__ __forceinline__ M3<float> staple_staged(const Links<float, 6>& U, con
         M3<float> term;
         if ((k & 1) == 0) {
             const M3<float> t = mul_nd_2(staged_rows(sm, st, 0), staged_full<PACKED>(sm, st, 1));
-            term = mul_nd_2<true>(t, staged_full<PACKED>(sm, st, 2));
+            term = mul_nd_2<FMA>(t, staged_full<PACKED>(sm, st, 2));
         } else {
             M3<float> t = mul_nn_2(staged_rows(sm, st, 1), staged_full<PACKED>(sm, st, 0));
             complete<PACKED>(t);
-            term = mul_dn_2<true>(t, staged_full<PACKED>(sm, st, 2));
+            term = mul_dn_2<FMA>(t, staged_full<PACKED>(sm, st, 2));
         }
         complete<PACKED>(term);
         acc_add(A, term);
