@@ -112,7 +112,10 @@ static_assert(sizeof(ProlongCtl) == 64, "control block layout");
 
 constexpr int PB_CHUNK = 64;       // lattices per launch (kernel-parameter table)
 constexpr int PB_THREADS = 128;
-constexpr int PB_BLOCKS = 5;       // resident per SM (FP32); six: 48 lattices 20.2 against 20.4 ms, 8^4 -> 16^4 11.5 against 11.2
+// resident blocks per SM (FP32).  With six instead of five: 16 lattices each of 6^4, 8^4
+// and 4^3x8 doubled with 20 steps a stage 20.2 against 20.4 ms, but one 8^4 of beta = 5.8
+// to 16^4 with the 0.001 % rule 11.5 against 11.2 ms (both FP32 12-real).
+constexpr int PB_BLOCKS = 5;
 constexpr int PB_SD_LANES = 256;  // partial-action lanes per block (any block size)
 constexpr int PB_SD_MAXBLK = 512;  // partial-action blocks per lattice
 
@@ -497,15 +500,21 @@ static inline int nblk(long n, int t) { return (int)((n + t - 1) / t); }
 // lattice's blocks and bonds leave three quarters of the chip's places free, k = 2
 // while they fit in one wave, else 4 (8^4 -> 16^4), up to PB_SD_MAXBLK; a small lattice
 // alone waits for these chains (4^4 -> 8^4 with the 0.001 % rule 7.4 -> 6.2 ms with k =
-// 1, 4x6x4x8 9.1 -> 8.4 ms).  In a call over many lattices at most the lattice's share
-// of about 2048 blocks, so that the blocks stay large when there is parallelism
-// across lattices (48 lattices of 8^3x16 to 16^4, 20 steps a stage: 21.8 ms with a
-// share of 4096, 20.4 ms).
-static int sd_blocks(const Geom& g, double total_sites) {
+// 1, 4x6x4x8 9.1 -> 8.4 ms).  FP64 blocks, one or two to an SM, start from k = 2: with k = 1
+// they take the places of the bonds (20 steps a stage, k = 1 and 2: 4^4 -> 8^4 11.9 and
+// 10.4 ms, 4^3x8 18.7 and 14.2 ms).
+// In a call over many lattices at most the lattice's share of about 2048 blocks, so
+// that the blocks stay large when there is parallelism across lattices (16 lattices
+// each of 6^4, 8^4 and 4^3x8, 20 steps a stage: 21.8 ms with a share of 4096, 20.4 ms), but no
+// more than 12 plaquettes a lane: a launch holds PB_CHUNK lattices however many the call
+// has, and its bonds end before lanes longer than theirs (200 lattices of 4^3x8 to 8^4,
+// 18-real, 6 steps a stage: 30.3 ms without this limit, 26.2 ms with it).
+static int sd_blocks(const Geom& g, double total_sites, int prec) {
     const long wave = 152L * PB_BLOCKS, bonds = nblk(3L * g.V / 2, PB_THREADS);
     auto blocks = [&](int k) { return (long)nblk(3L * g.V, k * PB_SD_LANES); };
-    const long full = 4 * (blocks(1) + bonds) <= wave ? blocks(1) : blocks(2) + bonds <= wave ? blocks(2) : blocks(4);
+    const long full = prec != MGQ_F64 && 4 * (blocks(1) + bonds) <= wave ? blocks(1) : blocks(2) + bonds <= wave ? blocks(2) : blocks(4);
     long b = (long)((2048.0 * g.V + total_sites - 1.0) / total_sites);
+    if (b < blocks(12)) b = blocks(12);
     if (b > full) b = full;
     if (b > PB_SD_MAXBLK) b = PB_SD_MAXBLK;
     return b < 1 ? 1 : (int)b;
@@ -546,7 +555,7 @@ static void fill_pbatch(PBatch<T>& B, const mgq_lattice* coarse, const mgq_latti
         D.gc = make_geom(coarse[first + i].dims);
         B.prefix[i + 1] = B.prefix[i] + nblk(8L * D.gf.Vh, PB_THREADS);
         // bond blocks for the largest stage set (24 V_c bonds); the copy at a stage start loops
-        const int nS = sd_blocks(D.gf, tsites), nA = nblk(24L * D.gc.V, block_size(MGQ_KERNEL_APE, F.prec));
+        const int nS = sd_blocks(D.gf, tsites, F.prec), nA = nblk(24L * D.gc.V, block_size(MGQ_KERNEL_APE, F.prec));
         B.aprefix[i + 1] = B.aprefix[i] + nA;
         B.sprefix[i + 1] = B.sprefix[i] + nS;
     }
@@ -629,7 +638,7 @@ static mgq_status check_pair(const mgq_lattice* coarse, const mgq_lattice* fine,
 static uint64_t pb_state_bytes(const mgq_lattice* fine, int n) {
     uint64_t nparts = 0;
     const double ts = total_sites(fine, n);
-    for (int i = 0; i < n; i++) nparts += (uint64_t)sd_blocks(make_geom(fine[i].dims), ts);
+    for (int i = 0; i < n; i++) nparts += (uint64_t)sd_blocks(make_geom(fine[i].dims), ts, fine[i].prec);
     return round256((uint64_t)n * sizeof(ProlongCtl)) + round256((uint64_t)n * sizeof(unsigned) + sizeof(int)) +
            round256(nparts * sizeof(double)) + round256((uint64_t)3 * n * sizeof(int)) +
            round256((uint64_t)3 * n * sizeof(double));
@@ -638,7 +647,7 @@ static uint64_t pb_state_bytes(const mgq_lattice* fine, int n) {
 static PbState pb_state_at(void* work, const mgq_lattice* fine, int n) {
     uint64_t nparts = 0;
     const double ts = total_sites(fine, n);
-    for (int i = 0; i < n; i++) nparts += (uint64_t)sd_blocks(make_geom(fine[i].dims), ts);
+    for (int i = 0; i < n; i++) nparts += (uint64_t)sd_blocks(make_geom(fine[i].dims), ts, fine[i].prec);
     char* p = static_cast<char*>(work);
     PbState S;
     S.ctl = reinterpret_cast<ProlongCtl*>(p);

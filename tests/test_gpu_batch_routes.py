@@ -29,3 +29,24 @@ def _compare(gpu, prec, shapes, n_hb, n_or=2):
 @pytest.mark.parametrize("shapes", [[[6, 6, 6, 6], [2, 4, 6, 8], [4, 4, 10, 10]], [[16, 16, 16, 32], [8, 8, 8, 16]]])
 def test_several_attempts(gpu, prec, shapes):
     _compare(gpu, prec, shapes, 3)
+
+
+# 130 lattices: three launches a step; the partial sums' layout follows the whole call, the bits are those of one alone
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_prolongation_of_many_lattices(gpu, prec):
+    shapes = [[2, 2, 2, 2], [2, 4, 2, 4], [4, 4, 4, 2]]
+    coarse = []
+    for i in range(130):
+        c = gpu.Lattice(shapes[i % 3], prec, seed=23, lattice_id=i)
+        gpu.mgq_init_links(c, 1)
+        coarse.append(c)
+    fine = [gpu.Lattice([2 * v for v in c.dims], prec) for c in coarse]
+    batch = gpu.ProlongBatch(coarse, fine)
+    gpu.mgq_prolongate_batched(batch, 0.05, 0.0, 3)
+    iters, sd = batch.iters.cpu().numpy(), batch.sd.cpu().numpy()
+    for i in (0, 1, 62, 63, 64, 65, 127, 128, 129):
+        alone = gpu.Lattice(fine[i].dims, prec)
+        it, s = gpu.mgq_prolongate(coarse[i], alone, 0.05, 0.0, 3)
+        assert torch.equal(alone.links, fine[i].links) and list(iters[i]) == it
+        # sums of at most 3 V terms of O(1) in other groupings
+        assert np.max(np.abs(sd[i] - np.array(s))) < 1e-11 * max(1.0, np.max(np.abs(s)))
