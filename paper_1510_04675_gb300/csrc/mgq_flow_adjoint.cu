@@ -35,8 +35,9 @@ template <class T> __device__ __forceinline__ M3<T> commutator_ah(const M3<T>& a
 }
 
 // Per link: X = ca Za + cb Zb; Xi = J(X)* Lam, the series summed until a term drops
-// below the precision's rounding of the partial sum (|X| is O(eps): a few terms; at
-// most 12 in FP64 and 8 in FP32, enough for |X| <= 0.5); Lam <- e^{-X} Lam e^{X};
+// below the precision's rounding of the partial sum (|X| is O(eps): a few terms; the
+// n-th is below d^n / (n+1)!, d the largest difference of X's eigenvalues, so that 40 reach
+// FP64 rounding up to d = 6); Lam <- e^{-X} Lam e^{X};
 // Out <- s Xi + p Prev (cb == 0, p == 0: Zb, Prev not read).
 template <class T>
 __global__ void __launch_bounds__(128) k_dexp_adjoint(Geom g, Alg<T> Za, Alg<T> Zb, T ca, T cb, Alg<T> Lam, Alg<T> Out, Alg<T> Prev,
@@ -59,7 +60,7 @@ __global__ void __launch_bounds__(128) k_dexp_adjoint(Geom g, Alg<T> Za, Alg<T> 
     M3<T> term = L, sum = L;
     const T tiny = sizeof(T) == 4 ? T(3e-8) : T(5e-17);
 #pragma unroll 1
-    for (int n = 1; n <= (sizeof(T) == 4 ? 8 : 12); n++) {
+    for (int n = 1; n <= 40; n++) {
         term = commutator_ah(X, term);
         const T f = T(-1) / T(n + 1);
         T tmax = 0, smax = 0;
