@@ -452,8 +452,9 @@ def batched_leg(api, peak_gbs, beta_lo=5.8, beta_hi=6.1, n_sweeps=20, n_or=4, se
                              "ape_steps_mean": [float(v) for v in iters.mean(axis=0)],
                              "finished": int(pb.n_done.item())},
             "ms_graph_prolongation_plus_sweeps": ms_all,
-            "launch_shapes": {"threads_per_block": dict(shapes_sw, **shapes_ape),
-                              "tuned_by": "paper_1510_04675_gb300.tune (sweeps on every 8th lattice)"},
+            "launch_shapes": {"threads_per_block": dict({k: tune.launch_threads(k, fine)[0] for k in shapes_sw}, **shapes_ape),
+                              "tuned_by": "paper_1510_04675_gb300.tune (APE step)"
+                              + (", sweeps on every 8th lattice" if any(tune.launch_threads(k, fine)[1] for k in shapes_sw) else "")},
             "plaquette_mean": float(P[-1].mean().item()), "graph": True,
             "workload": "96x12^4 + 96x16^4 + 64x8^3x16 prolongated from coarse 6^4, 8^4, 4^3x8 (beta in [5.8, 6.1]) "
                         "with the 0.001 % stopping rule on the device, 20 x (1 HB + 4 OR), FP32 12-real, "
@@ -771,10 +772,9 @@ def run_mgq(args, dims, world, rank, local):
         "gpu_launches": K * (8 + 8 * n_or + 1),
         "ms_overrelax_sweep_with_plaquette": last_ms,
         "clocks": clocks,
-        "launch_shapes": {"threads_per_block": {"heatbath": tune.STAGED_THREADS, "overrelax": tune.STAGED_THREADS}
-                          if args.prec == "f32c12" and V // 2 >= tune.STAGED_MIN_VH else launch_shapes,
-                          "tuned_by": f"fixed: staged FP32 12-real sub-sweeps (V/2 >= {tune.STAGED_MIN_VH})"
-                          if args.prec == "f32c12" and V // 2 >= tune.STAGED_MIN_VH else "paper_1510_04675_gb300.tune"},
+        "launch_shapes": {"threads_per_block": {k: tune.launch_threads(k, [lat])[0] for k in launch_shapes},
+                          "tuned_by": "paper_1510_04675_gb300.tune"
+                          if any(tune.launch_threads(k, [lat])[1] for k in launch_shapes) else "fixed: the kernels' own"},
     }
     if clocks and clocks.get("sm_mhz"):
         # clock-normalised step: SM cycles per step at the median clock of the timed region

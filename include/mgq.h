@@ -130,6 +130,15 @@ typedef enum {
 mgq_status mgq_set_block_size(int kernel, int prec, int threads);
 /* Current value, 0 for an unknown kernel or precision. */
 int mgq_get_block_size(int kernel, int prec);
+/* Threads per block of the sub-sweep launches of `kernel` over these lattices (one
+ * lattice, or a batch for the batched kernels and the APE step; only dims and prec
+ * are read): a heat bath of one attempt, overrelaxation.  *tunable (may be NULL) = 1
+ * when that is the value of mgq_set_block_size, 0 when the shape is the kernel's own
+ * -- then the setting serves heat baths of several attempts only, and in FP64 the
+ * plaquette-measuring sub-sweeps of a batch.  Of a batch in several launches: the
+ * setting as soon as one of them uses it, else the first one's shape.  0 for invalid
+ * arguments. */
+int mgq_launch_threads(int kernel, const mgq_lattice* lats, int n_lat, int* tunable);
 
 /* FP32 arithmetic probe: one launch of independent packed FP32 FMA chains on
  * every SM (4 blocks of 256 threads per SM, `iters` iterations of 16 packed

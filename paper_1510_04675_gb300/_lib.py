@@ -90,6 +90,7 @@ SIGNATURES = {
     "mgq_batch_workspace_bytes": (ctypes.c_uint64, [_P, _i, _i]),
     "mgq_set_block_size": (_st, [_i, _i, _i]),
     "mgq_get_block_size": (ctypes.c_int, [_i, _i]),
+    "mgq_launch_threads": (ctypes.c_int, [_i, _P, _i, ctypes.POINTER(ctypes.c_int)]),
     "mgq_update_sweeps_batched": (_st, [_P, _i, ctypes.POINTER(ctypes.c_double), _u64, _i, _i, _i, _vp, _vp, _u64,
                                         _vp]),
 }

@@ -288,6 +288,32 @@ using namespace mgq;
 
 extern "C" {
 
+int mgq_launch_threads(int kernel, const mgq_lattice* lats, int n_lat, int* tunable) {
+    if (tunable) *tunable = 0;
+    if (kernel < 0 || kernel >= MGQ_NKERNELS || !lats || n_lat < 1) return 0;
+    const bool batched = kernel == MGQ_KERNEL_HEATBATH_BATCHED || kernel == MGQ_KERNEL_OVERRELAX_BATCHED;
+    if (!batched && kernel != MGQ_KERNEL_APE && n_lat != 1) return 0;
+    const int prec = lats[0].prec;
+    if (prec < MGQ_F64 || prec > MGQ_F32_C12) return 0;
+    for (int i = 0; i < n_lat; i++)
+        if (!valid_dims(lats[i].dims) || lats[i].prec != prec) return 0;
+    const int set = block_size(kernel, prec);
+    int first_threads = 0;
+    for (int first = 0; first < n_lat; first += BATCH_CHUNK) {
+        long links = 0;
+        for (int i = first; i < n_lat && i < first + BATCH_CHUNK; i++) links += make_geom(lats[i].dims).Vh;
+        const int warps = term_warps(prec, links);
+        const bool columns = prec == MGQ_F64 && update_lanes(links) > 1;
+        const int fixed = kernel == MGQ_KERNEL_APE ? 0 : columns ? COL_THREADS : warps ? warps * TERMS_LINKS : prec == MGQ_F32_C12 ? STAGED_THREADS : 0;
+        if (!fixed) {
+            if (tunable) *tunable = 1;
+            return set;
+        }
+        if (!first) first_threads = fixed;
+    }
+    return first_threads;
+}
+
 uint64_t mgq_batch_workspace_bytes(const mgq_lattice* lats, int n_lat, int n_sweeps) {
     if (!lats || n_lat < 1 || n_sweeps < 0) return 0;
     for (int i = 0; i < n_lat; i++)
