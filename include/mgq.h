@@ -346,7 +346,7 @@ int mgq_flow_adaptive_measurements(double t_end, double dt_meas);
  * sum_l sum_a L_l,a e_l,a. */
 
 /* Bytes of the caller scratch of mgq_wilson_flow_step_adjoint (2 link fields
- * + 7 algebra fields); 0 on invalid extents or precision. */
+ * + 6 algebra fields); 0 on invalid extents or precision. */
 uint64_t mgq_flow_adjoint_scratch_bytes(const mgq_lattice* lat);
 
 /* g_out = J(omega)^T g_in: pulls a cotangent g_in at the field exp(omega) U back

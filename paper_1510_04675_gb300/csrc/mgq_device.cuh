@@ -265,14 +265,6 @@ template <> __device__ __forceinline__ void acc_add<float>(M3<float>& a, const M
         for (int j = 0; j < 3; j++)
             a.e[i][j] = from_f2(__fadd2_rn(make_float2(a.e[i][j].re, a.e[i][j].im), make_float2(b.e[i][j].re, b.e[i][j].im)));
 }
-template <class T> __device__ __forceinline__ M3<T> dagger(const M3<T>& a) {
-    M3<T> r;
-#pragma unroll
-    for (int i = 0; i < 3; i++)
-#pragma unroll
-        for (int j = 0; j < 3; j++) r.e[i][j] = conjg(a.e[j][i]);
-    return r;
-}
 // Re Tr(a b)
 template <class T> __device__ __forceinline__ T retr_nn(const M3<T>& a, const M3<T>& b) {
     T s = T(0);

@@ -273,7 +273,7 @@ static mgq_status dexp_adjoint(const mgq_lattice* lat, void* za, void* zb, doubl
 }
 
 uint64_t flow_adjoint_scratch(const mgq_lattice* lat) {
-    return 2 * round256(links_bytes(lat)) + 7 * round256(alg_bytes(lat));
+    return 2 * round256(links_bytes(lat)) + 6 * round256(alg_bytes(lat));
 }
 
 }  // namespace mgq

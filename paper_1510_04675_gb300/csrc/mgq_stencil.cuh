@@ -283,6 +283,20 @@ __device__ __forceinline__ M3<float> down_term(const M3<float>& e_rows, const M3
 }
 
 // =============================================================== plaquette
+// Re Tr(a b^+) of a, b in SU(3) from their rows 0, 1: with s_ij = row_i(a) .
+// conj(row_j(b)) it is s00 + s11 + conj(s00 s11 - s01 s10) (row 2 = conj(row0 x row1) and
+// the Binet-Cauchy identity for the cross products).
+__device__ __forceinline__ float retr_two_row(const M3<float>& a, const M3<float>& b) {
+    Cx<float> sij[2][2];
+#pragma unroll
+    for (int i = 0; i < 2; i++)
+#pragma unroll
+        for (int j = 0; j < 2; j++)
+            sij[i][j] = mulc(a.e[i][0], b.e[j][0]) + mulc(a.e[i][1], b.e[j][1]) + mulc(a.e[i][2], b.e[j][2]);
+    const Cx<float> d = sij[0][0] * sij[1][1] - sij[0][1] * sij[1][0];
+    return sij[0][0].re + sij[1][1].re + d.re;
+}
+
 // Per site: sum over mu < nu < ND of Re Tr[U_mu(x) U_nu(x+mu) (U_nu(x) U_mu(x+nu))^+]
 // (ND = 4: all six planes; ND = 3: the planes of directions 0, 1, 2).
 template <class T, int NP, int ND = 4>
@@ -296,24 +310,14 @@ __device__ __forceinline__ double site_plaquettes(const Links<T, NP>& U, const G
     for (int mu = 0; mu < ND - 1; mu++) {
         const int hpm = (H.lex + H.fwd[mu]) >> 1;
         if constexpr (sizeof(T) == 4) {
-            // FP32: a = U_mu(x) U_nu(x+mu) and b = U_nu(x) U_mu(x+nu) are in SU(3),
-            // so rows 0, 1 of each suffice: with s_ij = row_i(a) . conj(row_j(b)),
-            // Tr(a b^+) = s00 + s11 + conj(s00 s11 - s01 s10) (row 2 = conj(row0 x row1)
-            // and the Binet-Cauchy identity for the cross products).
+            // FP32: a = U_mu(x) U_nu(x+mu) and b = U_nu(x) U_mu(x+nu) are in SU(3)
             const M3<T> umu = U.load_rows(mu, par, h);
 #pragma unroll
             for (int nu = mu + 1; nu < ND; nu++) {
                 const int hpn = (H.lex + H.fwd[nu]) >> 1;
                 const M3<T> a = mul_nn_2(umu, U.load(nu, op, hpm));
                 const M3<T> b = mul_nn_2(U.load_rows(nu, par, h), U.load(mu, op, hpn));
-                Cx<T> sij[2][2];
-#pragma unroll
-                for (int i = 0; i < 2; i++)
-#pragma unroll
-                    for (int j = 0; j < 2; j++)
-                        sij[i][j] = mulc(a.e[i][0], b.e[j][0]) + mulc(a.e[i][1], b.e[j][1]) + mulc(a.e[i][2], b.e[j][2]);
-                const Cx<T> d = sij[0][0] * sij[1][1] - sij[0][1] * sij[1][0];
-                acc += (double)(sij[0][0].re + sij[1][1].re + d.re);
+                acc += (double)retr_two_row(a, b);
             }
         } else {
             const M3<T> umu = U.load(mu, par, h);
@@ -384,19 +388,7 @@ __device__ __forceinline__ T loop_retr(const Links<T, NP>& U, const Hops& H, int
     return retr_nd(a, mul_nn(U.load(nu, par, x), U.load(mu, op, xn)));
 }
 
-// The plaquette of FP32 links in SU(3): rows 0, 1 of a = U_mu(x) U_nu(x+mu) and b =
-// U_nu(x) U_mu(x+nu) suffice: with s_ij = row_i(a) . conj(row_j(b)), Tr(a b^+) = s00 +
-// s11 + conj(s00 s11 - s01 s10) (row 2 = conj(row0 x row1); Binet-Cauchy).
-__device__ __forceinline__ float retr_two_row(const M3<float>& a, const M3<float>& b) {
-    Cx<float> sij[2][2];
-#pragma unroll
-    for (int i = 0; i < 2; i++)
-#pragma unroll
-        for (int j = 0; j < 2; j++)
-            sij[i][j] = mulc(a.e[i][0], b.e[j][0]) + mulc(a.e[i][1], b.e[j][1]) + mulc(a.e[i][2], b.e[j][2]);
-    const Cx<float> d = sij[0][0] * sij[1][1] - sij[0][1] * sij[1][0];
-    return sij[0][0].re + sij[1][1].re + d.re;
-}
+// The plaquette of FP32 links in SU(3), as in site_plaquettes.
 template <int NP>
 __device__ __forceinline__ float plaquette_retr(const Links<float, NP>& U, const Hops& H, int par, int op, int mu, int nu) {
     const int x = H.lex >> 1, xm = (H.lex + pick(H.fwd, mu)) >> 1, xn = (H.lex + pick(H.fwd, nu)) >> 1;
