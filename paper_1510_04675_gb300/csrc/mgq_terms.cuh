@@ -102,12 +102,22 @@ __global__ void __launch_bounds__(WARPS * TERMS_LINKS, 24 / WARPS) k_update_term
 }
 
 // Warps per 32 links of an FP32 launch over n links, 0 for the kernels with a thread per
-// link.  Six warps give the shortest chain, three hold more links per SM; a thread per
-// link wins once it fills the SMs, for 18-real links from 40960 on (one wave of its
-// blocks; overrelaxation of 49152 links 7.8 against 8.3 us), for 12-real ones,
-// whose one-thread form stages its links, from about 73728 (10.0 against 10.5 us; at
-// 49152 9.8 against 8.3).  Several attempts per subgroup, or recorded decisions, run a
-// thread per link.
+// link.  Six warps give the shortest chain, three hold more links per SM, and a thread
+// per link wins once it fills the SMs; heat bath and overrelaxation of one launch, us:
+//               18-real: six      three      thread     12-real: six    three       thread (staged)
+//   n = 14336    4.6  3.7    4.9  4.2    8.7  6.9       4.8  3.9    4.6   4.2     9.5  7.6
+//       16384    5.0  3.9    5.0  4.3    8.9  7.0       5.0  4.0    4.7   4.3     8.8  7.1
+//       20480    6.3  5.0    6.8  4.8    9.2  7.5       6.4  5.1    6.4   4.8    11.7  9.8
+//       32768    8.1  6.1    6.7  5.6    9.5  7.2       8.1  6.4    6.8   6.1    10.8  8.6
+//       36864    8.3  6.5    6.8  5.7    9.4  6.6       8.4  6.6    6.7   6.1    11.6  9.2
+//       40960    9.2  7.2    9.8  7.2    9.5  7.7       9.3  7.5    9.5   7.1    11.6  9.1
+//       45056    9.8  7.7   10.0  8.0    9.5  7.8       9.7  7.7    9.8   8.0    10.7  7.8
+//       61440   12.5  9.6   11.4  9.5    9.8  7.9      12.3  9.8   11.2   9.0    11.9  9.5
+//       65536   12.8 10.0   11.7  9.7    9.7  7.9      13.3 10.2   11.8   9.7    11.7  9.4
+//       69632   13.6 10.6   11.8  9.8    9.7  7.9      13.7 10.9   12.5  10.2    11.7  9.4
+// The lines lie where the neighbours meet: 16384; 40960 for 18-real links, one wave of
+// their one-thread blocks; 65536 for 12-real ones.  Several attempts per subgroup, or
+// recorded decisions, run a thread per link.
 inline int term_warps(int prec, long n) {
     if (prec == MGQ_F64) return 0;
     if (n < 16384) return 6;
